@@ -103,9 +103,8 @@ __global__ void init_padded(T* __restrict__ G, int p, int pp, T diag, int eye) {
 // Per-block SVT gate: ||A||_F^2 <= tau^2 means every singular value of A is
 // <= tau, so the threshold removes all of them and J = 0 with no SVD.
 // The Z-step kernel of the same iteration then accumulates the next value.
-template <typename T>
-__global__ void svt_gate(const int* __restrict__ act, double* __restrict__ afro, const double* __restrict__ mu,
-                         int* __restrict__ svt_on, T* __restrict__ scale, int* __restrict__ calls,
+static __global__ void svt_gate(const int* __restrict__ act, double* __restrict__ afro, const double* __restrict__ mu,
+                         int* __restrict__ svt_on, int* __restrict__ calls,
                          int* __restrict__ fp32_on, int* __restrict__ gemm32, double margin, int nblk) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nblk) return;
@@ -117,35 +116,7 @@ __global__ void svt_gate(const int* __restrict__ act, double* __restrict__ afro,
     // rounding of the products is forgotten by the iteration
     if (afro[b] > margin * margin * tau * tau) fp32_on[b] = 1;
     gemm32[b] = (act[b] && fp32_on[b]) ? 1 : 0;
-    if (act[b]) {
-        scale[b] = (T)afro[b];
-        afro[b] = 0.0;
-    }
-}
-
-// Largest squared column norm of X (the Jacobi noise scale): one CTA per block.
-template <typename T>
-__global__ void col_norm_max(const OsjDesc<T>* __restrict__ descs, const int* __restrict__ on, T* __restrict__ scale,
-                             int nblk) {
-    const int b = blockIdx.x;
-    if (b >= nblk || !on[b]) return;
-    const OsjDesc<T> d = descs[b];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    T mx = T(0);
-    for (int j = warp; j < d.p; j += nw) {
-        const T* x = d.X + (int64_t)j * d.ldx;
-        T acc = T(0);
-        for (int i = lane; i < d.L; i += 32) acc += x[i] * x[i];
-        mx = fmax(mx, warp_sum(acc));
-    }
-    __shared__ T s_m[32];
-    if (lane == 0) s_m[warp] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        T m2 = T(0);
-        for (int w = 0; w < nw; ++w) m2 = fmax(m2, s_m[w]);
-        scale[b] = m2;
-    }
+    if (act[b]) afro[b] = 0.0;
 }
 
 // After the one-sided Jacobi the columns x_j of X are orthogonal and

@@ -58,30 +58,41 @@ cudaError_t jacobi_sweeps(const JacDesc<T>* d_desc, int nmat, int max_pp, int sw
                          const int* done_dev = nullptr, int* sweeps_run = nullptr);
 // One-sided block Jacobi (osj.cu): X (L x p, ld ldx) is rotated to orthogonal
 // columns together with W (p x p, ld ldw); pp = p rounded up to the pivot
-// width.  off points at three slots (the per-sweep convergence maxima).
+// width.  Scratch: off, three slots (the per-sweep convergence maxima); cols,
+// 2 pp values (column norms); ord, pp ints (column order).
 template <typename T>
 struct OsjDesc {
     T* X;
     T* W;
-    int* done;
     T* off;
+    T* cols;
+    int* ord;
     const int* active;
-    const T* scale;     // largest squared column norm of X
     const double* mu;   // SVT threshold is 1/mu (nullptr: measure every pair)
     int64_t ldx, ldw;
     int L, p, pp;
     int strict;         // 1: resolve pairs straddling tau to angle tol (C-step block)
-    int* ctr;           // optional: two ints of scratch; the cluster's CTAs then take the
-                        // pivots of a round from a shared counter instead of a fixed share
 };
 
-// One launch: every block is a thread-block cluster of `cluster` CTAs (0:
-// one per pivot of a round, up to osj_max_cluster()) that runs its sweeps
+// Launch shape: CTAs per block's cluster, CTAs per pivot, 512-thread CTAs or
+// not, longest columns and most columns of a block.
+struct OsjShape {
+    int cluster, split, wide, max_L, max_p;
+};
+// the shape for nmat blocks of at most max_p columns and max_L rows; cluster
+// > 0 fixes the largest cluster size to use
+template <typename T>
+OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster = 0);
+
+// Schedule of the sweeps (osj.cu); float64 always runs `sorted`.
+enum class OsjMode { kept, sorted };
+
+// One launch: every block is a thread-block cluster that runs its sweeps
 // until converged or `sweeps` are done.  `quad_exit`: stop one sweep early
 // once quadratic convergence guarantees the tolerance (see osj_svd).
 template <typename T>
-cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, int max_pp, int sweeps, T tol, int* sweeps_run,
-                       cudaStream_t s, int cluster = 0, int quad_exit = 0);
+cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
+                       cudaStream_t s, OsjMode mode, int quad_exit = 0);
 // largest cluster size osj_sweeps uses on the current device (16 or 8)
 template <typename T>
 int osj_max_cluster();

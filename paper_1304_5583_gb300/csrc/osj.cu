@@ -2,27 +2,46 @@
 //
 // For every block the L x p matrix X (X = A W for a tall A, X = A^T W for a
 // wide one, W the previous iteration's right basis) is driven to orthogonal
-// columns by rotations X <- X R, W <- W R.  The p columns are split into
-// column blocks of b = 16; in each round the pp/b column blocks are paired
-// round-robin (circle method) and every pair (a pivot of 2b = 32 columns)
-//   1. forms the 32 x 32 Gram S = X_P^T X_P afresh from the columns of X
+// columns by rotations X <- X R, W <- W R.  The columns are cut into column
+// blocks of b; in each round the column blocks are paired round-robin (circle
+// method) and every pair (a pivot of 2b columns)
+//   1. forms the 2b x 2b Gram S = X_P^T X_P afresh from the columns of X
 //      (each entry carries only the rounding of its own two columns),
-//   2. rotates S towards diagonal form in shared memory (one inner cyclic
-//      Jacobi sweep in float32, up to four in float64),
+//   2. rotates S towards diagonal form in shared memory,
 //   3. re-orthonormalises the accumulated rotation R and applies it to X_P
 //      and W_P in update form.
 // Pairs of a round touch disjoint columns.
 //
+// Two schedules (OsjMode):
+//   kept     columns in their own places, one inner pass over all pairs of a
+//            pivot.  The float32 solver: its stop test (1e-6 against float32
+//            residuals) and the blocks' paths react to the rounding of every
+//            SVT, so its arithmetic is held fixed, operation for operation.
+//   sorted   columns taken by falling norm (sorted at the start of sweeps 0, 2
+//            and 4), up to two inner passes over the pairs that cross the two
+//            column blocks (the first round of a sweep also takes the pairs
+//            inside each).  The stand-alone SVT and float64.  Small columns
+//            come together, so whole pivots need nothing, and sweeps are
+//            saved: a cold 350 x 256 float32 SVT that keeps 100 directions
+//            takes 9 sweeps and 716 rotated pivots, against 13 and 1262.
+//            (Sorting at every sweep shuffles columns of nearly equal norm and
+//            slows the float64 tail: 23 sweeps against 12.)
+//
 // One launch runs every sweep of every block: each block is a thread-block
-// cluster whose CTAs share the pairs of a round (a free CTA takes the next
-// pair from a per-block counter) and meet at a cluster barrier between rounds
-// (the barrier's release/acquire makes one round's column updates visible to
-// the next).  After each sweep the cluster reduces the
-// largest convergence measure seen in it and stops once that is below the
-// tolerance, so a converged block costs nothing further and the others are
-// not held to a common sweep count.
+// cluster whose CTAs share the pivots of a round and meet at a cluster barrier
+// between rounds (the barrier's release/acquire makes one round's column
+// updates visible to the next).  Where a cluster has more CTAs than a round
+// has pivots, `split` CTAs share one pivot: each forms the Gram of its rows,
+// the partial Grams meet through distributed shared memory, every member runs
+// the same (tiny) inner rotation and applies it to its own rows.  A Gram is
+// always the sum of the same four row-slot partials in the same order, so
+// neither the cluster size nor the split changes a bit of the result.
+// After each sweep the cluster reduces the largest convergence measure seen in
+// it and stops once that is below the tolerance, so a converged block costs
+// nothing further and the others are not held to a common sweep count.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -34,132 +53,438 @@ namespace cg = cooperative_groups;
 namespace lrr {
 namespace {
 
-constexpr int OB = 16;            // column-block width b
-constexpr int B2 = 2 * OB;        // pivot width
-constexpr int NT = 128;           // threads per CTA (one pivot at a time)
-constexpr int NW = NT / 32;
-constexpr int CH = 64;            // rows per staged chunk of the pivot columns
-constexpr int LDX = B2 + 4;       // row stride of the staged chunk (16-byte rows)
-constexpr int LO = B2 + 1;        // odd row stride of S and R (conflict-free scattered access)
-constexpr int WORK = NW * B2 * B2;   // scratch: chunk tile, then per-warp partial Grams, then R^T R and R - I
-static_assert(CH * LDX <= WORK && LO * B2 + B2 * B2 <= WORK, "scratch too small");
+// Threads per CTA (a CTA works on one pivot, or one member's share of it, at a
+// time).  512, one CTA to an SM, with the pivot's columns of X kept in shared
+// memory from the Gram to the rotation, when the blocks' clusters have the SMs
+// to themselves: a pivot's own chain of loads, products and rotations is then
+// all there is to wait for.  256 at up to 80 registers, three CTAs to an SM,
+// when there are more blocks than that (or columns too long to keep): their
+// phases cover one another's latencies.
+constexpr int NT_MANY = 256, NT_FEW = 512;
+// A Gram is summed in four row slots: of every chunk of 64 rows, slot s has the
+// 16 rows from 16 s.  Each chunk's 16 products are summed on their own and then
+// added to the slot's total; the totals are added in slot order.
+constexpr int NSLOT = 4, SR = 16, CHR = NSLOT * SR;
+constexpr size_t SMEM_MAX = 227 * 1024;
 
-// Inner sweeps per pivot, at most.  float32 runs one: the pivot need not be
-// diagonalised exactly, the next outer sweep continues from where one inner
-// sweep leaves it.  On the 1000 x 20000 solve this took 10 881 outer sweeps
-// against 11 126 with up to four inner sweeps, and 2.64 s of Jacobi time
-// against 3.20 s.  float64 keeps up to four.
-template <typename T> __host__ __device__ constexpr int inner_sweeps() { return sizeof(T) == 4 ? 1 : 4; }
-
-__device__ __forceinline__ int pcol(int i, int a, int c) { return i < OB ? a * OB + i : c * OB + (i - OB); }
+// Column-block width: float32 16 (pivots of 32 columns).  float64 8: the inner
+// rotation is bound by the float64 units (two FMA lanes per SM and clock), and
+// a 16-column pivot has an eighth of a 32-column pivot's inner work while a
+// round then has twice as many pivots to spread over the SMs.
+template <typename T> struct Cfg;
+template <> struct Cfg<float> { static constexpr int OB = 16, V = 4, LS = 34; };
+template <> struct Cfg<double> { static constexpr int OB = 8, V = 2, LS = 18; };
 
 template <typename T>
-struct Smem {
-    T work[WORK];
-    T S[B2][LO];
-    T R[B2][LO];
-    T cs[OB], sn[OB];
-    int pi[OB], qi[OB];
-    T red[NW];
-    int pick;
+struct __align__(16) Smem {                       // followed by the stage
+    static constexpr int B2 = 2 * Cfg<T>::OB;
+    static constexpr int ST = CHR + Cfg<T>::V;    // column stride of a staged chunk (conflict-free 16-byte reads)
+    static constexpr int PS = B2 + Cfg<T>::V;     // row stride of a partial Gram
+    static constexpr int PART = NSLOT * B2 * PS;  // the four partial Grams
+    static constexpr int STAGE = PART + 2 * B2 * ST;
+    T S[2][B2 * Cfg<T>::LS];
+    T R[B2 * Cfg<T>::LS];
+    T G[B2 * B2];                                 // R^T R
+    T R4[B2 * B2];                                // R - I, rows of 16-byte multiples
+    T red[NT_FEW / 32];
+    int cid[B2];                                  // physical column of each pivot column, -1: none
+    int sig[2], rot, cur;
+    OsjDesc<T> d;                                 // the block's descriptor (kept out of the registers)
 };
 
-// 16-byte vector loads from shared memory
-__device__ __forceinline__ void lds4(const float* p, float (&v)[4]) {
+// Shared memory after Smem: the partial Grams; then, with 256 threads, two
+// staged chunks, and with 512 the member's rows of the pivot columns of X, and
+// of W (at most WROWS of them at a time).  W takes the place of the partial
+// Grams, which are read before it is written; a split pivot's partial Grams
+// are also read by the other members, so there W has a place of its own.
+constexpr int WROWS = 512;
+// rows of X of a split pivot's member: of every chunk the NSLOT / split slots it owns
+__host__ __device__ constexpr int local_rows(int L, int split) {
+    return (L + CHR - 1) / CHR * (NSLOT / split) * SR;
+}
+// column strides of the kept columns: one bank quad past a multiple of 32 words
+template <typename T>
+__host__ __device__ constexpr int panel_stride(int L, int split) {
+    return (local_rows(L, split) + 31) / 32 * 32 + Cfg<T>::V;
+}
+template <typename T>
+__host__ __device__ constexpr int wpanel_stride(int p, int split) {
+    const int r = ((p + 31) / 32 + split - 1) / split * 32;
+    return (r < WROWS ? r : WROWS) + Cfg<T>::V;
+}
+
+// 16-byte vectors of shared memory
+__device__ __forceinline__ void lds16(const float* p, float (&v)[4]) {
     const float4 x = *reinterpret_cast<const float4*>(p);
     v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
 }
-__device__ __forceinline__ void lds4(const double* p, double (&v)[4]) {
+__device__ __forceinline__ void lds16(const double* p, double (&v)[2]) {
     const double2 x = *reinterpret_cast<const double2*>(p);
-    const double2 y = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+    v[0] = x.x; v[1] = x.y;
 }
 
-// One pivot (column blocks a and c) of one round: Gram, measure, rotation.
-// Returns the convergence measure of the pivot (block-uniform).
-template <typename T>
-__device__ T osj_pivot(const OsjDesc<T>& d, Smem<T>& sm, int a, int c) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+// Global stores, named as such: through a generic pointer the compiler must
+// assume that each may change shared memory, and reads the column list, R - I and
+// the next operands again after every one of them (a 4 x 16 tile took 6 us).
+// Volatile: they stay before the barriers that publish them.
+__device__ __forceinline__ void stg(float* p, float v) {
+    asm volatile("st.global.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v));
+}
+__device__ __forceinline__ void stg(double* p, double v) {
+    asm volatile("st.global.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v));
+}
 
-    // ---- 1. Gram S = X_P^T X_P over the L rows, in CH-row chunks staged in
-    //      shared memory (the next chunk is fetched into registers while the
-    //      current one is multiplied).  Warp w sums rows w*16 .. w*16+15 of a
-    //      chunk into a fresh partial (4 x 8 entries per lane); the warps'
-    //      totals are added in a fixed order at the end.
-    T* const Xs = sm.work;
-    constexpr int PER = CH * B2 / NT;           // chunk elements loaded per thread
-    const int ti = lane & 7, tj = lane >> 3;     // S rows 4ti.., cols 8tj..
-    T acc[4][8];
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Rotation that annihilates s_pq: tan(theta) = b / (d + sgn(d) sqrt(d^2 + b^2)),
+// d = s_qq - s_pp, b = 2 s_pq (the root of smaller magnitude of
+// b t^2 + 2 d t - b = 0).  d and b are first scaled by a power of two so that
+// the larger lies in [1, 2): no overflow, and b^2 underflows only where t = b / 2d
+// to working accuracy.  Hardware reciprocal and reciprocal square root: the
+// rotation only steers the pivot towards diagonal form, the accumulated R is
+// re-orthonormalised before use, and the next sweep forms its Grams afresh.
+__device__ __forceinline__ void rotation(float app, float aqq, float apq, float& c, float& s) {
+    const float d = aqq - app, b = 2.f * apq;
+    const unsigned e = __float_as_uint(fmaxf(fabsf(d), fabsf(b))) & 0x7F800000u;
+    const float sc = __uint_as_float(0x7F000000u - e);
+    const float fd = d * sc, fb = b * sc;
+    const float h = fmaf(fd, fd, fb * fb);
+    const float t = fb * rcp_approx(fd + copysignf(h * rsqrt_approx(h), fd));
+    c = rsqrt_approx(fmaf(t, t, 1.f));
+    s = t * c;
+}
+// float64: c and s from the float32 units (a float64 divide or square root
+// costs more than the rest of a round), then scaled to c^2 + s^2 = 1 in float64:
+// the rotation is orthogonal to float64 rounding and leaves about 1e-7 of s_pq,
+// which the second pass and the next sweep take.
+__device__ __forceinline__ void rotation(double app, double aqq, double apq, double& c, double& s) {
+    double d = aqq - app, b = 2.0 * apq;
+    const int e = __double2hiint(fmax(fabs(d), fabs(b))) & 0x7FF00000;
+    const double sc = __hiloint2double(0x7FE00000 - e, 0);
+    const float fd = (float)(d * sc), fb = (float)(b * sc);
+    const float h = fmaf(fd, fd, fb * fb);
+    const float t = fb * rcp_approx(fd + copysignf(h * rsqrt_approx(h), fd));
+    const float c0 = rsqrt_approx(fmaf(t, t, 1.f));
+    const double cd = (double)c0, sd = (double)(t * c0);
+    const double q = fma(-cd, cd, fma(-sd, sd, 1.0));      // the squares of 24-bit values are exact
+    const double g = q * fma(0.375, q, 0.5);               // (1 - q)^(-1/2) - 1 to O(q^3), q about 1e-7
+    c = fma(cd, g, cd);
+    s = fma(sd, g, sd);
+}
+// |s_pq| > eps sqrt(s_pp s_qq), with a square root good to a few per cent
+__device__ __forceinline__ bool needs_rotation(float app, float aqq, float apq) {
+    float q;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(fabsf(app * aqq)));
+    return fabsf(apq) > FLT_MIN && fabsf(apq) > FLT_EPSILON * q;
+}
+__device__ __forceinline__ bool needs_rotation(double app, double aqq, double apq) {
+    const int hi = __double2hiint(fabs(app * aqq));
+    const double q = __hiloint2double((hi >> 1) + 0x1FF80000, 0);    // exponent halved
+    return fabs(apq) > DBL_MIN && fabs(apq) > DBL_EPSILON * q;
+}
+
+// non-negative norms ordered by their bits (a NaN sorts first: the order stays
+// a permutation whatever the input holds)
+__device__ __forceinline__ unsigned key_of(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned long long key_of(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// part += (16 rows, column by column)^T (the same): lane (ti, tj) of 16 x 2
+// holds the entries (ti + 16u, j0 + tj + 2v) of TI x TJ, so that 16-byte reads,
+// each worth V rows of one column, meet no bank twice.
+template <typename T, int TI, int TJ>
+__device__ __forceinline__ void gram_rows(const T* st, int stride, int ti, int j0, T (&acc)[TI][TJ]) {
+    constexpr int V = Cfg<T>::V;
+    T part[TI][TJ];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < TI; ++u)
 #pragma unroll
-        for (int v = 0; v < 8; ++v) acc[u][v] = T(0);
-    // thread t fetches row t % CH of the chunk in columns t / CH + 2u (u < PER):
-    // the first PER/2 lie in column block a, the rest in column block c
-    static_assert(NT == 2 * CH && PER == B2 / 2, "fetch mapping");
+        for (int v = 0; v < TJ; ++v) part[u][v] = T(0);
+#pragma unroll
+    for (int q = 0; q < SR; q += V) {
+        T xi[TI][V];
+#pragma unroll
+        for (int u = 0; u < TI; ++u) lds16(st + (ti + 16 * u) * stride + q, xi[u]);
+#pragma unroll
+        for (int v = 0; v < TJ; ++v) {
+            T xj[V];
+            lds16(st + (j0 + 2 * v) * stride + q, xj);
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+#pragma unroll
+                for (int u = 0; u < TI; ++u) part[u][v] = fma(xi[u][e], xj[e], part[u][v]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < TI; ++u)
+#pragma unroll
+        for (int v = 0; v < TJ; ++v) acc[u][v] += part[u][v];
+}
+template <typename T, int TI, int TJ>
+__device__ __forceinline__ void put_partial(T* part, int ti, int j0, const T (&acc)[TI][TJ]) {
+#pragma unroll
+    for (int u = 0; u < TI; ++u)
+#pragma unroll
+        for (int v = 0; v < TJ; ++v) part[(ti + 16 * u) * Smem<T>::PS + j0 + 2 * v] = acc[u][v];
+}
+
+// 256 threads: the partial Grams from chunks staged by the whole CTA, the next
+// chunk's loads in flight during the products; two warps to a slot, half of
+// the columns each.  (Warps that stage their own rows and columns need no
+// barrier, but three times the shared memory and more registers.)
+template <typename T>
+__device__ __forceinline__ void gram_staged(const Smem<T>& sm, T* stage) {
+    constexpr int B2 = Smem<T>::B2, ST = Smem<T>::ST, TI = B2 / 16, TJ = B2 / 4, PER = B2 * CHR / NT_MANY;
+    const OsjDesc<T>& d = sm.d;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int slot = warp & 3, j0 = (warp >> 2) * (B2 / 2) + (lane >> 4), ti = lane & 15;
+    T* const buf = stage + Smem<T>::PART;
+    const int frow = t % CHR, fcol = t / CHR;
     T pre[PER];
-    const int frow = t % CH, fcol = t / CH;
-    const T* const pa = d.X + (int64_t)(a * OB + fcol) * d.ldx + frow;
-    const T* const pc = d.X + (int64_t)(c * OB + fcol) * d.ldx + frow;
-    const int64_t fst = 2 * d.ldx;
     auto fetch = [&](int ch) {
-        const bool rok = ch * CH + frow < d.L;
-        const int64_t ro = (int64_t)ch * CH;
+        const int row = ch * CHR + frow;
+        const bool ok = row < d.L;
+        const T* const base = d.X + row;
 #pragma unroll
-        for (int u = 0; u < PER / 2; ++u) {
-            pre[u] = (rok && a * OB + fcol + 2 * u < d.p) ? __ldcg(pa + ro + u * fst) : T(0);
-            pre[u + PER / 2] = (rok && c * OB + fcol + 2 * u < d.p) ? __ldcg(pc + ro + u * fst) : T(0);
+        for (int u = 0; u < PER; ++u) {
+            const int gc = sm.cid[fcol + u * (NT_MANY / CHR)];
+            pre[u] = (ok && gc >= 0) ? __ldcg(base + (int64_t)gc * d.ldx) : T(0);
         }
     };
-    const int nchunk = (d.L + CH - 1) / CH;
+    T acc[TI][TJ];
+#pragma unroll
+    for (int u = 0; u < TI; ++u)
+#pragma unroll
+        for (int v = 0; v < TJ; ++v) acc[u][v] = T(0);
+    const int nch = (d.L + CHR - 1) / CHR;
     fetch(0);
-    for (int ch = 0; ch < nchunk; ++ch) {
+    for (int ch = 0; ch < nch; ++ch) {
+        T* const st = buf + (ch & 1) * (B2 * ST);
 #pragma unroll
-        for (int u = 0; u < PER / 2; ++u) {
-            Xs[frow * LDX + fcol + 2 * u] = pre[u];
-            Xs[frow * LDX + OB + fcol + 2 * u] = pre[u + PER / 2];
-        }
-        __syncthreads();
-        if (ch + 1 < nchunk) fetch(ch + 1);
-        T part[4][8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 8; ++v) part[u][v] = T(0);
-#pragma unroll 4
-        for (int rr = warp * (CH / NW); rr < (warp + 1) * (CH / NW); ++rr) {
-            T xi[4], xj0[4], xj1[4];
-            lds4(Xs + rr * LDX + ti * 4, xi);
-            lds4(Xs + rr * LDX + tj * 8, xj0);
-            lds4(Xs + rr * LDX + tj * 8 + 4, xj1);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    part[u][v] = fma(xi[u], xj0[v], part[u][v]);
-                    part[u][v + 4] = fma(xi[u], xj1[v], part[u][v + 4]);
-                }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 8; ++v) acc[u][v] += part[u][v];
-        __syncthreads();
+        for (int u = 0; u < PER; ++u) st[(fcol + u * (NT_MANY / CHR)) * ST + frow] = pre[u];
+        __syncthreads();      // (the buffer's last readers passed the previous chunk's barrier)
+        if (ch + 1 < nch) fetch(ch + 1);
+        gram_rows<T, TI, TJ>(st + slot * SR, ST, ti, j0, acc);
     }
-    // per-warp partials -> S (fixed order), R = I
-    T* const Pw = sm.work + warp * B2 * B2;
+    put_partial<T, TI, TJ>(stage + slot * B2 * Smem<T>::PS, ti, j0, acc);
+}
+
+// what a pivot needs to know of its block (in registers)
+template <typename T>
+struct PivotCtx {
+    T *X, *W;
+    int ldx, ldw, L, p;
+    T scale, tau, floor2;
+    T *stage, *panel, *wpanel;      // stage; kept columns of X and of W (512 threads)
+    int rank, split, member, stride, wstride;
+    bool first_round;     // first round of the sweep: pairs inside the column blocks too
+};
+
+// 512 threads: the member's rows of the pivot columns into shared memory, all
+// loads in flight together (an L2 load takes about 0.65 us); rows past L are zero.
+// Local row (c own + j) 16 + i is row 64 c + 16 (member own + j) + i.
+template <typename T>
+__device__ __forceinline__ int global_row(int lr, int own, int member) {
+    const int g = lr / SR;
+    return g / own * CHR + (member * own + g % own) * SR + lr % SR;
+}
+template <typename T>
+__device__ __forceinline__ void load_panel(const PivotCtx<T>& d, const Smem<T>& sm, int own, int member) {
+    constexpr int B2 = Smem<T>::B2, KB = B2 / 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nr = (d.stride - Cfg<T>::V) / 32;            // 32-row groups
+    for (int w = warp; w < nr * 2; w += NT_FEW / 32) {
+        const int lr = (w >> 1) * 32 + lane, k0 = (w & 1) * KB;
+        const int row = global_row<T>(lr, own, member);
+        const bool ok = row < d.L;
+        const T* const base = d.X + row;
+        T* const dst = d.panel + lr;
+        T pre[KB];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+        for (int k = 0; k < KB; ++k) {
+            const int gc = sm.cid[k0 + k];
+            pre[k] = (ok && gc >= 0) ? __ldcg(base + (int64_t)gc * d.ldx) : T(0);
+        }
 #pragma unroll
-        for (int v = 0; v < 8; ++v) Pw[(ti * 4 + u) * B2 + tj * 8 + v] = acc[u][v];
+        for (int k = 0; k < KB; ++k) dst[(k0 + k) * d.stride] = pre[k];
+    }
+}
+
+// 512 threads: partial Grams from the kept columns, four warps to a slot, a
+// quarter of the columns each (a split pivot's member has fewer slots and
+// leaves the other warps out).
+template <typename T>
+__device__ __forceinline__ void gram_kept(const PivotCtx<T>& d, int own) {
+    constexpr int B2 = Smem<T>::B2, TI = B2 / 16, TJ = B2 / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j = warp >> 2, j0 = (warp & 3) * (B2 / 4) + (lane >> 4), ti = lane & 15;
+    if (j >= own) return;
+    T acc[TI][TJ];
+#pragma unroll
+    for (int u = 0; u < TI; ++u)
+#pragma unroll
+        for (int v = 0; v < TJ; ++v) acc[u][v] = T(0);
+    const int nch = (d.L + CHR - 1) / CHR;
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) gram_rows<T, TI, TJ>(d.panel + (c * own + j) * SR, d.stride, ti, j0, acc);
+    put_partial<T, TI, TJ>(d.stage + j * B2 * Smem<T>::PS, ti, j0, acc);
+}
+
+// One row of 2b pivot columns times (R - I): x_j <- x_j + sum_k x_k (R - I)_kj,
+// rows of R - I read by broadcast.  float32 uses the paired FMA (half the issue
+// slots of the scalar one, which the broadcast reads then fill).
+__device__ __forceinline__ void row_update(const float* R4, const float (&x)[32], int h, float (&o)[16]) {
+    unsigned long long a[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) a[v] = 0ull;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        unsigned long long xx;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x[k]));
+        const ulonglong2* const r = reinterpret_cast<const ulonglong2*>(R4 + k * 32 + h * 16);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const ulonglong2 q = r[v];
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a[2 * v]) : "l"(xx), "l"(q.x));
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a[2 * v + 1]) : "l"(xx), "l"(q.y));
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 8; ++v) asm("mov.b64 {%0, %1}, %2;" : "=f"(o[2 * v]), "=f"(o[2 * v + 1]) : "l"(a[v]));
+}
+__device__ __forceinline__ void row_update(const double* R4, const double (&x)[16], int h, double (&o)[8]) {
+#pragma unroll
+    for (int v = 0; v < 8; ++v) o[v] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            double q[2];
+            lds16(R4 + k * 16 + h * 8 + 2 * v, q);
+            o[2 * v] = fma(x[k], q[0], o[2 * v]);
+            o[2 * v + 1] = fma(x[k], q[1], o[2 * v + 1]);
+        }
+    }
+}
+
+// 512 threads: rows [row0, row0 + 32 RT) of kept columns times (R - I), columns
+// h OW .. h OW + OW - 1, by one warp; a lane has rows row0 + lane + 32 i.  Every
+// value of R - I is read (by broadcast) once for RT rows: with one row per lane
+// the broadcast reads, two shared-memory cycles each, took twice the time of the
+// FMAs they fed (5.4 us for 512 rows of a 32-column pivot).  store(i, v, value) receives row i's
+// output column h OW + v.
+template <int RT, typename Store>
+__device__ __forceinline__ void tile_update(const float* R4, const float* cols, int stride, int h, Store store) {
+    unsigned long long a[RT][8];
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) a[i][v] = 0ull;
+#pragma unroll 4
+    for (int k = 0; k < 32; ++k) {
+        ulonglong2 q[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) q[v] = reinterpret_cast<const ulonglong2*>(R4 + k * 32 + h * 16)[v];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            unsigned long long xx;
+            asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(cols[k * stride + 32 * i]));
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a[i][2 * v]) : "l"(xx), "l"(q[v].x));
+                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a[i][2 * v + 1]) : "l"(xx), "l"(q[v].y));
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            float o0, o1;
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(o0), "=f"(o1) : "l"(a[i][v]));
+            store(i, 2 * v, cols[(h * 16 + 2 * v) * stride + 32 * i] + o0);
+            store(i, 2 * v + 1, cols[(h * 16 + 2 * v + 1) * stride + 32 * i] + o1);
+        }
+}
+template <int RT, typename Store>
+__device__ __forceinline__ void tile_update(const double* R4, const double* cols, int stride, int h, Store store) {
+    double a[RT][8];
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) a[i][v] = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < 16; ++k) {
+        double q[8];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            double w[2];
+            lds16(R4 + k * 16 + h * 8 + 2 * v, w);
+            q[2 * v] = w[0];
+            q[2 * v + 1] = w[1];
+        }
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const double x = cols[k * stride + 32 * i];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) a[i][v] = fma(x, q[v], a[i][v]);
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+#pragma unroll
+        for (int i = 0; i < RT; ++i) store(i, v, cols[(h * 8 + v) * stride + 32 * i] + a[i][v]);
+}
+
+// One pivot (logical column blocks a and c) of one round: Gram, measure,
+// rotation.  Returns the convergence measure of the pivot (CTA-uniform);
+// top_a / top_c receive the two largest squared norms of the column blocks.
+template <typename T, int NT, bool KEEP>
+__device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx, int a, int c, T* top_a, T* top_c) {
+    constexpr int OB = Cfg<T>::OB, B2 = 2 * OB, LS = Cfg<T>::LS, NW = NT / 32;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int split = NT == NT_MANY ? 1 : cx.split, member = NT == NT_MANY ? 0 : cx.member;
+
+    if (t < B2) {
+        const int pos = t < OB ? a * OB + t : c * OB + (t - OB);
+        sm.cid[t] = pos < sm.d.p ? (KEEP ? pos : __ldcg(sm.d.ord + pos)) : -1;
+    }
+    if (t == 32) { sm.sig[0] = 0; sm.sig[1] = 0; sm.rot = 0; }
     __syncthreads();
+
+    // ---- 1. Gram
+    const int own = NSLOT / split;
+    if constexpr (NT == NT_MANY) {
+        gram_staged<T>(sm, reinterpret_cast<T*>(&sm + 1));
+        __syncthreads();
+    } else {
+        load_panel<T>(cx, sm, own, member);
+        __syncthreads();
+        gram_kept<T>(cx, own);
+        if (split == 1) __syncthreads();
+        else cl.sync();
+    }
     for (int e = t; e < B2 * B2; e += NT) {
         const int i = e / B2, j = e % B2;
-        T s = sm.work[e];
+        T p[NSLOT];
 #pragma unroll
-        for (int w = 1; w < NW; ++w) s += sm.work[w * B2 * B2 + e];
-        sm.S[i][j] = s;
-        sm.R[i][j] = (i == j) ? T(1) : T(0);
+        for (int sl = 0; sl < NSLOT; ++sl) {
+            const T* src = reinterpret_cast<T*>(&sm + 1) + (sl % own) * B2 * Smem<T>::PS + i * Smem<T>::PS + j;
+            if (NT == NT_FEW && split > 1) src = cl.map_shared_rank(src, cx.rank - member + sl / own);
+            p[sl] = *src;
+        }
+        sm.S[0][i * LS + j] = ((p[0] + p[1]) + p[2]) + p[3];
+        sm.R[i * LS + j] = (i == j) ? T(1) : T(0);
     }
     __syncthreads();
 
@@ -170,32 +495,65 @@ __device__ T osj_pivot(const OsjDesc<T>& d, Smem<T>& sm, int a, int c) {
     //      (f(s) = max(s - tau, 0) is 1-Lipschitz, so |a - b| bounds it), plus
     //      tau theta when both lie above tau (the pair then enters J as
     //      A - tau U V^T and theta = |s_ij| / (a b) is its angle defect).
-    //      Pairs with a^2 + b^2 <= tau^2 have every singular value below tau
-    //      and are removed by the SVT whatever their rotation; columns below
-    //      the rounding floor (~4 eps of the largest) are noise and skipped.  A
-    //      `strict` matrix (the block whose kept left singular subspace the C
-    //      step projects onto) also needs that subspace itself: pairs that
-    //      straddle tau are measured by t alone.
-    const T noise = T(4) * num<T>::eps();
-    const T floor2 = noise * noise * (*d.scale) + num<T>::tiny();
-    const T tau = d.mu ? (T)(1.0 / *d.mu) : T(0);
-    const T tau2 = tau * tau;
-    const T smax = sqrt(*d.scale);
-    const T inv_smax = T(1) / (smax + num<T>::tiny());
+    //      A pair with a^2 + b^2 <= tau^2 has its own two singular values below
+    //      tau, but many such columns together may not: a set of them stays
+    //      below tau, whatever its rotation, while every max(a^2, b^2) + p |s_ij|
+    //      <= tau^2 (Gershgorin's bound on its Gram), which is what the sorted
+    //      schedule asks of them; the kept schedule leaves them out (they are
+    //      rotated with the larger columns of their pivots).
+    //      Columns below the rounding floor (~4 eps of the largest) are noise
+    //      and skipped.  A `strict` matrix (the block whose kept left singular
+    //      subspace the C step projects onto) also needs that subspace itself:
+    //      pairs that straddle tau are measured by t alone.
+    const T tau = cx.tau, tau2 = tau * tau;
     T offm = T(0);
-    for (int e = t; e < B2 * B2; e += NT) {
-        const int i = e % B2, j = e / B2;
-        const T sii = sm.S[i][i], sjj = sm.S[j][j];
-        if (i < j && sii > floor2 && sjj > floor2 && sii + sjj > tau2) {
-            const T sij = fabs(sm.S[i][j]);
-            const T na = sqrt(sii), nb = sqrt(sjj);
-            const T hd = T(0.5) * fabs(sii - sjj);
-            const T tn = sij / (hd + sqrt(hd * hd + sij * sij) + num<T>::tiny());
-            T mm;
-            if (na > tau && nb > tau) mm = tn * fabs(na - nb) + tau * sij / (na * nb);
-            else if (na > tau || nb > tau) mm = d.strict ? tn * (*d.scale > 0 ? smax : T(1)) : tn * fabs(na - nb);
-            else mm = tn * (sqrt(sii + sjj) - tau);
-            offm = fmax(offm, mm * inv_smax);
+    if constexpr (KEEP) {
+        const T smax = sqrt(cx.scale);
+        const T inv_smax = T(1) / (smax + num<T>::tiny());
+        for (int e = t; e < B2 * B2; e += NT) {
+            const int i = e % B2, j = e / B2;
+            const T sii = sm.S[0][i * LS + i], sjj = sm.S[0][j * LS + j];
+            if (i < j && sii > cx.floor2 && sjj > cx.floor2 && sii + sjj > tau2) {
+                const T sij = fabs(sm.S[0][i * LS + j]);
+                const T na = sqrt(sii), nb = sqrt(sjj);
+                const T hd = T(0.5) * fabs(sii - sjj);
+                const T tn = sij / (hd + sqrt(hd * hd + sij * sij) + num<T>::tiny());
+                T mm;
+                if (na > tau && nb > tau) mm = tn * fabs(na - nb) + tau * sij / (na * nb);
+                else if (na > tau || nb > tau)
+                    mm = sm.d.strict ? tn * (cx.scale > 0 ? smax : T(1)) : tn * fabs(na - nb);
+                else mm = tn * (sqrt(sii + sjj) - tau);
+                offm = fmax(offm, mm * inv_smax);
+            }
+        }
+    } else {
+        // the differences are taken in T, the rest in float32 on values relative
+        // to the largest column: the measure only steers the sweeps
+        const T inv_scale = T(1) / (cx.scale + num<T>::tiny());
+        const float ftau = (float)(tau * sqrt(inv_scale));
+        for (int e = t; e < B2 * B2; e += NT) {
+            const int j = e % B2, i = e / B2;
+            if (i >= j) continue;
+            const T sii = sm.S[0][i * LS + i], sjj = sm.S[0][j * LS + j];
+            if (sii > cx.floor2 && sjj > cx.floor2) {
+                const T sij = fabs(sm.S[0][i * LS + j]);
+                const float a2 = (float)(sii * inv_scale), b2 = (float)(sjj * inv_scale);
+                const float fs = (float)(sij * inv_scale), df = fabsf((float)((sii - sjj) * inv_scale));
+                const float na = sqrtf(a2), nb = sqrtf(b2), gap = df / (na + nb);       // |na - nb|
+                // tangent 2 s / (|a^2 - b^2| + sqrt((a^2 - b^2)^2 + 4 s^2)), scaled against underflow
+                const float m = fmaxf(df, 2.f * fs), mi = m > 0.f ? 1.f / m : 0.f;
+                const float u = df * mi, w = 2.f * fs * mi;
+                const float tn = w / (u + sqrtf(fmaf(u, u, w * w)) + FLT_MIN);
+                float mm;
+                if (sii + sjj <= tau2) {
+                    const T g = fmax(sii, sjj) + T(sm.d.p) * sij;
+                    const float fg = (float)((g - tau2) * inv_scale);
+                    mm = fg / (sqrtf((float)(g * inv_scale)) + ftau);
+                } else if (sii > tau2 && sjj > tau2) mm = tn * gap + ftau * fs / (na * nb);
+                else if (sii > tau2 || sjj > tau2) mm = sm.d.strict ? tn : tn * gap;
+                else mm = tn * (float)((sii + sjj - tau2) * inv_scale) / (sqrtf(a2 + b2) + ftau);
+                offm = fmax(offm, (T)mm);
+            }
         }
     }
     offm = warp_max(offm);
@@ -204,162 +562,398 @@ __device__ T osj_pivot(const OsjDesc<T>& d, Smem<T>& sm, int a, int c) {
     T mx = T(0);
 #pragma unroll
     for (int w = 0; w < NW; ++w) mx = fmax(mx, sm.red[w]);
+
+    // two largest diagonal entries of each column block (read by the next
+    // rounds' skip test; member 0 writes them)
+    const T* Sd = sm.S[0];
+    auto tops = [&]() {
+        if (member == 0 && (t == 0 || t == 32)) {
+            T n1 = T(0), n2 = T(0);
+            const int o = t == 0 ? 0 : OB;
+            for (int i = 0; i < OB; ++i) {
+                const T v = Sd[(o + i) * LS + o + i];
+                if (!(v <= n1)) { n2 = n1; n1 = v; }      // a NaN counts as large
+                else if (!(v <= n2)) n2 = v;
+            }
+            T* const dst = t == 0 ? top_a : top_c;
+            dst[0] = n1;
+            dst[1] = n2;
+        }
+    };
     // a pivot already orthogonal to a few eps needs no rotation (4 eps in
     // float32: on data with one dominant singular value the measure, relative
     // to the largest column, must resolve pairs well below it)
-    if (mx <= (sizeof(T) == 4 ? T(4) : T(16)) * num<T>::eps()) return mx;
+    if (mx <= (sizeof(T) == 4 ? T(4) : T(16)) * num<T>::eps()) {
+        tops();
+        __syncthreads();      // cid and S are rewritten by the next pivot
+        return mx;
+    }
 
-    // ---- 3. rotate the pivot Gram towards diagonal form (all threads of the
-    //      CTA): one inner sweep in float32; in float64 up to four, where
-    //      rotations that only mix noise columns do not keep the sweeps going
-    const int rot = inner_jacobi<T, B2, NT, LO>(sm.S, sm.R, sm.cs, sm.sn, sm.pi, sm.qi, num<T>::tiny(), floor2,
-                                                inner_sweeps<T>(),
-                                                sizeof(T) == 4 ? T(3e-4) : T(0));
-    if (!rot) return mx;
+    // 512 threads: the first rows of W are fetched while the pivot rotates (split
+    // members take alternate chunks)
+    const int wchunks = ((cx.p + 31) / 32 - member + split - 1) / split, wrows = wchunks * 32;
+    auto wrow = [&](int lw) { return ((lw / 32) * split + member) * 32 + lw % 32; };
+    T wx[NT == NT_FEW ? B2 : 1];
+    auto load_w = [&](int row) {
+        if constexpr (NT == NT_FEW) {
+            const T* const base = cx.W + row;
+#pragma unroll
+            for (int k = 0; k < B2; ++k) {
+                const int gc = sm.cid[k];
+                wx[k] = (row < cx.p && gc >= 0) ? __ldcg(base + (int64_t)gc * cx.ldw) : T(0);
+            }
+        }
+    };
+    if (t < wrows) load_w(wrow(t));
+
+    // ---- 3. rotate the pivot Gram towards diagonal form.  Thread (k, l) of
+    //      b x b owns the 2 x 2 sub-block of pairs k and l: it reads the old S,
+    //      works out pair k's rotation itself, takes pair l's from the lane that
+    //      has it, and writes the other S buffer, so a round costs one barrier
+    //      of these b^2 threads and one chain of shared read, rotation, write
+    //      (0.25 us; 0.7 us with a barrier on either side of the rotations).
+    //      Sorted: 62 rounds in the first round of a sweep, else 32, or half of
+    //      that when the first pass found only small angles (float32; no tangent
+    //      above 3e-4, in float64 1e-8: what the second would still find is the
+    //      square of that).  Kept: 31 rounds.
+    if (t < OB * OB) {
+        const int k = t % OB, l = t / OB;
+        const T exit_tan = sizeof(T) == 4 ? T(3e-4) : T(1e-8);
+        int cur = 0, rotated = 0;
+        const int r_first = KEEP ? 0 : cx.first_round ? -(OB - 1) : 0, r_end = KEEP ? B2 - 1 : OB;
+        for (int pass = 0; pass < (KEEP ? 1 : 2); ++pass) {
+            int big = 0;
+            for (int r = r_first; r < r_end; ++r) {
+                int pk, qk, pl, ql;
+                if (KEEP) {
+                    pk = circle_item(k, r, B2); qk = circle_item(B2 - 1 - k, r, B2);
+                    pl = circle_item(l, r, B2); ql = circle_item(B2 - 1 - l, r, B2);
+                } else if (r >= 0) {
+                    pk = k; qk = OB + ((k + r) & (OB - 1));
+                    pl = l; ql = OB + ((l + r) & (OB - 1));
+                } else {
+                    // pairs inside column block a (first half) and c
+                    constexpr int H = OB / 2;
+                    const int rr = r + OB - 1, ok = k < H ? 0 : OB, ol = l < H ? 0 : OB;
+                    pk = ok + circle_item(k & (H - 1), rr, OB); qk = ok + circle_item(OB - 1 - (k & (H - 1)), rr, OB);
+                    pl = ol + circle_item(l & (H - 1), rr, OB); ql = ol + circle_item(OB - 1 - (l & (H - 1)), rr, OB);
+                }
+                const T* const S = sm.S[cur];
+                T* const D = sm.S[cur ^ 1];
+                const T app = S[pk * LS + pk], aqq = S[qk * LS + qk], apq = S[pk * LS + qk];
+                const T s_pu = S[pk * LS + pl], s_pv = S[pk * LS + ql], s_qu = S[qk * LS + pl], s_qv = S[qk * LS + ql];
+                const T x0 = sm.R[k * LS + pl], y0 = sm.R[k * LS + ql];
+                const T x1 = sm.R[(k + OB) * LS + pl], y1 = sm.R[(k + OB) * LS + ql];
+                // (always computed, then selected: a branch costs more than the
+                // few lanes it would spare)
+                T ck, sk;
+                bool act;
+                if constexpr (KEEP) {
+                    act = fabs(apq) > num<T>::tiny() && fabs(apq) > num<T>::eps() * sqrt(fabs(app * aqq));
+                    jacobi_rotation<T>(app, aqq, apq, ck, sk);
+                } else {
+                    act = needs_rotation(app, aqq, apq);
+                    rotation(app, aqq, apq, ck, sk);
+                }
+                ck = act ? ck : T(1);
+                sk = act ? sk : T(0);
+                rotated |= act;
+                if (!KEEP) big |= act && fabs(apq) > cx.floor2 && fabs(sk) > exit_tan * ck;
+                const T clr = __shfl_sync(0xffffffffu, ck, l), slr = __shfl_sync(0xffffffffu, sk, l);
+                // (fused multiply-adds written out: which product of a sum of two is
+                // rounded first is part of the kept schedule's arithmetic)
+                const T r_pu = fma(ck, s_pu, -(sk * s_qu)), r_pv = fma(ck, s_pv, -(sk * s_qv));
+                const T r_qu = fma(sk, s_pu, ck * s_qu), r_qv = fma(sk, s_pv, ck * s_qv);
+                // float32: the rotated pair's own off-diagonal entries are zero
+                // by construction (to the rounding of the next fresh Gram)
+                const bool zero = sizeof(T) == 4 && k == l && sk != T(0);
+                D[pk * LS + pl] = fma(clr, r_pu, -(slr * r_pv));
+                D[pk * LS + ql] = zero ? T(0) : fma(slr, r_pu, clr * r_pv);
+                D[qk * LS + pl] = zero ? T(0) : fma(clr, r_qu, -(slr * r_qv));
+                D[qk * LS + ql] = fma(slr, r_qu, clr * r_qv);
+                sm.R[k * LS + pl] = fma(clr, x0, -(slr * y0));
+                sm.R[k * LS + ql] = fma(slr, x0, clr * y0);
+                sm.R[(k + OB) * LS + pl] = fma(clr, x1, -(slr * y1));
+                sm.R[(k + OB) * LS + ql] = fma(slr, x1, clr * y1);
+                cur ^= 1;
+                if (r == r_end - 1) {
+                    if (big) sm.sig[pass] = 1;
+                    if (rotated) sm.rot = 1;
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(OB * OB) : "memory");
+            }
+            if (!KEEP && !sm.sig[pass]) break;
+        }
+        if (t == 0) sm.cur = cur;
+    }
+    __syncthreads();
+    Sd = sm.S[sm.cur];
+    tops();
+    if (!sm.rot) {
+        __syncthreads();
+        return mx;
+    }
 
     // R is a product of some hundred plane rotations, orthogonal only to
     // ~sqrt(count) eps; one Newton-Schulz step R <- R (3I - R^T R)/2 restores
     // orthogonality to ~eps^2 before R touches X and W (applied to graded
     // columns the defect would mix eps-sized parts of the large columns into
     // the small ones)
-    T* const G = sm.work;                     // R^T R, stride LO
-    T* const R4 = sm.work + LO * B2;          // R - I, stride B2 (16-byte rows)
-    constexpr int PE = B2 * B2 / NT;
+    constexpr int PE = B2 * B2 / 256;             // consecutive entries of a row per thread
+    const int ni = t * PE / B2, nj = t * PE % B2;
+    if (t < 256) {
+        T g[PE];
 #pragma unroll
-    for (int u = 0; u < PE; ++u) {
-        const int e = t + u * NT, i = e % B2, j = e / B2;
-        T g = T(0);
+        for (int u = 0; u < PE; ++u) g[u] = T(0);
 #pragma unroll 8
-        for (int k = 0; k < B2; ++k) g = fma(sm.R[k][i], sm.R[k][j], g);
-        G[i * LO + j] = g;
-    }
-    __syncthreads();
-    T y[PE];
+        for (int k = 0; k < B2; ++k) {
+            const T x = sm.R[k * LS + ni];
 #pragma unroll
-    for (int u = 0; u < PE; ++u) {
-        const int e = t + u * NT, i = e % B2, j = e / B2;
-        T s = T(0);
-#pragma unroll 8
-        for (int k = 0; k < B2; ++k) s = fma(sm.R[i][k], G[k * LO + j], s);
-        y[u] = s;
+            for (int u = 0; u < PE; ++u) g[u] = fma(x, sm.R[k * LS + nj + u], g[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < PE; ++u) sm.G[ni * B2 + nj + u] = g[u];
     }
     __syncthreads();
     // the rotation is applied in update form, x_j <- x_j + sum_k x_k (R - I)_kj:
     // once the sweeps have converged R - I is tiny and so is the rounding it
     // adds, instead of a fresh eps |x| at every application
+    if (t < 256) {
+        T y[PE];
 #pragma unroll
-    for (int u = 0; u < PE; ++u) {
-        const int e = t + u * NT, i = e % B2, j = e / B2;
-        const T rn = T(1.5) * sm.R[i][j] - T(0.5) * y[u];
-        R4[i * B2 + j] = rn - (i == j ? T(1) : T(0));
+        for (int u = 0; u < PE; ++u) y[u] = T(0);
+#pragma unroll 8
+        for (int k = 0; k < B2; ++k) {
+            const T x = sm.R[ni * LS + k];
+#pragma unroll
+            for (int u = 0; u < PE; ++u) y[u] = fma(x, sm.G[k * B2 + nj + u], y[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < PE; ++u) {
+            const T rn = fma(T(1.5), sm.R[ni * LS + nj + u], T(-0.5) * y[u]);
+            sm.R4[ni * B2 + nj + u] = rn - (ni == nj + u ? T(1) : T(0));
+        }
     }
     __syncthreads();
 
-    // ---- 4. X_P <- X_P R and W_P <- W_P R: one row per lane, the 32 pivot
-    //      columns of that row in registers, rows of R - I read by broadcast
-    for (int pass = 0; pass < 2; ++pass) {
-        T* base = pass == 0 ? d.X : d.W;
-        const int64_t ld = pass == 0 ? d.ldx : d.ldw;
-        const int rows = pass == 0 ? d.L : d.p;
-        for (int r0 = warp * 32; r0 < rows; r0 += NT) {
-            const int row = r0 + lane;
-            const bool ok = row < rows;
+    // ---- 4. X_P <- X_P R and W_P <- W_P R
+    constexpr int OW = 8 * (8 / sizeof(T));       // output columns at a time: 16 floats, 8 doubles
+    static_assert(B2 == 2 * OW, "two halves");
+    if constexpr (NT == NT_MANY) {
+        // the rows of X, then those of W, in one sequence from L2, a row's 2b
+        // pivot columns in a thread's registers
+        const OsjDesc<T>& d = sm.d;
+        const int rows = d.L + d.p;
+        for (int r0 = 0; r0 < rows; r0 += NT) {
+            const int row = r0 + t;
+            const bool ok = row < rows, isx = row < d.L;
+            if (r0 + warp * 32 >= rows) break;
+            T* const base = isx ? d.X + row : d.W + (row - d.L);
+            const int ld = isx ? d.ldx : d.ldw;
             T x[B2];
 #pragma unroll
             for (int k = 0; k < B2; ++k) {
-                const int gc = pcol(k, a, c);
-                x[k] = (ok && gc < d.p) ? __ldcg(base + row + (int64_t)gc * ld) : T(0);
+                const int gc = sm.cid[k];
+                x[k] = (ok && gc >= 0) ? __ldcg(base + (int64_t)gc * ld) : T(0);
             }
-            // outputs in groups of OW columns (fewer live registers for float64)
-            constexpr int OW = 8;
 #pragma unroll
-            for (int half = 0; half < B2 / OW; ++half) {
+            for (int h = 0; h < 2; ++h) {
                 T o[OW];
-#pragma unroll
-                for (int v = 0; v < OW; ++v) o[v] = T(0);
-#pragma unroll
-                for (int k = 0; k < B2; ++k) {
-                    T rk[OW];
-#pragma unroll
-                    for (int q = 0; q < OW / 4; ++q) {
-                        T v4[4];
-                        lds4(R4 + k * B2 + half * OW + q * 4, v4);
-#pragma unroll
-                        for (int z = 0; z < 4; ++z) rk[q * 4 + z] = v4[z];
-                    }
-#pragma unroll
-                    for (int v = 0; v < OW; ++v) o[v] = fma(x[k], rk[v], o[v]);
-                }
+                row_update(sm.R4, x, h, o);
 #pragma unroll
                 for (int v = 0; v < OW; ++v) {
-                    const int j = half * OW + v;
-                    const int gc = pcol(j, a, c);
-                    if (ok && gc < d.p) base[row + (int64_t)gc * ld] = x[j] + o[v];
+                    const int gc = sm.cid[h * OW + v];
+                    if (ok && gc >= 0) base[(int64_t)gc * ld] = x[h * OW + v] + o[v];
                 }
             }
+        }
+    } else {
+        // from shared memory, one warp per tile of RT 32-row groups and half
+        // the columns: the tiles of X first, then those of the W rows fetched above
+        // (W rows past the first WROWS follow in turn)
+        constexpr int RT = sizeof(T) == 4 ? 4 : 1;
+        const int xg = (cx.stride - Cfg<T>::V) / 32, lrows = local_rows(cx.L, split);
+        for (int w0 = 0; w0 < wrows || w0 == 0; w0 += WROWS) {
+            const int wg = min(wchunks - w0 / 32, WROWS / 32);
+            if (t < wg * 32) {
+                if (w0 > 0) load_w(wrow(w0 + t));
+#pragma unroll
+                for (int k = 0; k < B2; ++k) cx.wpanel[k * cx.wstride + t] = wx[k];
+            }
+            __syncthreads();
+            const int xt = w0 == 0 ? (xg + RT - 1) / RT : 0, wt = (wg + RT - 1) / RT;
+            for (int tile = warp; tile < 2 * (xt + wt); tile += NT / 32) {
+                const int h = tile & 1, g0 = tile / 2 < xt ? tile / 2 * RT : (tile / 2 - xt) * RT;
+                int gcs[OW];
+#pragma unroll
+                for (int v = 0; v < OW; ++v) gcs[v] = sm.cid[h * OW + v];
+                if (tile / 2 < xt) {
+                    tile_update<RT>(sm.R4, cx.panel + g0 * 32 + lane, cx.stride, h, [&](int i, int v, T val) {
+                        const int lr = (g0 + i) * 32 + lane, row = global_row<T>(lr, own, member);
+                        if (lr < lrows && row < cx.L && gcs[v] >= 0) stg(cx.X + (int64_t)gcs[v] * cx.ldx + row, val);
+                    });
+                } else {
+                    tile_update<RT>(sm.R4, cx.wpanel + g0 * 32 + lane, cx.wstride, h, [&](int i, int v, T val) {
+                        const int row = wrow(w0 + (g0 + i) * 32 + lane);
+                        if (g0 + i < wg && row < cx.p && gcs[v] >= 0) stg(cx.W + (int64_t)gcs[v] * cx.ldw + row, val);
+                    });
+                }
+            }
+            if (w0 + WROWS < wrows) __syncthreads();
         }
     }
     __syncthreads();
     return mx;
 }
 
-// One cluster per matrix (blockIdx.y); the cluster's CTAs share the pivots of
-// each round.  `off` holds three slots per matrix (one per sweep, reused every
-// third sweep), `done` is set when the matrix converged.
+// One cluster per matrix (blockIdx.y).  `off` holds three slots per matrix
+// (one per sweep, reused every third sweep).
 // With `quad_exit`, a sweep whose measure o (taken before its rotations)
 // satisfies 16 o^2 <= tol ends the loop without a confirming sweep: cyclic
 // Jacobi converges quadratically near the end (the off-diagonal part after a
 // sweep is O(o^2)), so the rotations of that sweep already bring the matrix
 // below the tolerance.
-template <typename T>
-__global__ void __launch_bounds__(NT, 5) osj_svd(const OsjDesc<T>* __restrict__ descs, int sweeps, T tol,
-                                              int* __restrict__ sweeps_run, int quad_exit) {
+template <typename T, int NT, bool KEEP>
+__global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDesc<T>* __restrict__ descs, int sweeps, T tol,
+                                              int* __restrict__ sweeps_run, int quad_exit, int split) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem<T>& sm = *reinterpret_cast<Smem<T>*>(smem_raw);
+    constexpr int OB = Cfg<T>::OB, NW = NT / 32;
     const int mat = blockIdx.y;
-    const OsjDesc<T> d = descs[mat];
+    if (threadIdx.x == 0) sm.d = descs[mat];
+    __syncthreads();
+    const OsjDesc<T>& d = sm.d;
     if (d.active && *d.active == 0) return;     // uniform over the cluster
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), csize = (int)cl.num_blocks();
-    const int nb = d.pp / OB, npairs = nb / 2;
-    const int t = threadIdx.x;
-    if (rank == 0 && t == 0) {
-        d.off[0] = T(0); d.off[1] = T(0); d.off[2] = T(0);
-        *d.done = 0;
-        if (d.ctr) { atomicExch(d.ctr, 0); atomicExch(d.ctr + 1, 0); }
+    const int team = rank / split, nteams = csize / split;
+    const int nb = 2 * ((d.p + 2 * OB - 1) / (2 * OB)), npairs = nb / 2;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    T* const nrm = d.cols;                      // squared column norms
+    T* const top = d.cols + d.pp;               // 2 parities x nb x 2 largest norms
+    if (rank == 0 && t == 0) { d.off[0] = T(0); d.off[1] = T(0); d.off[2] = T(0); }
+    PivotCtx<T> cx;
+    cx.X = d.X; cx.W = d.W;
+    cx.ldx = (int)d.ldx; cx.ldw = (int)d.ldw; cx.L = d.L; cx.p = d.p;
+    cx.rank = rank; cx.split = split; cx.member = rank % split;
+    cx.stage = reinterpret_cast<T*>(&sm + 1);
+    cx.stride = panel_stride<T>(d.L, split);
+    cx.wstride = wpanel_stride<T>(d.p, split);
+    if (NT == NT_FEW) {
+        // partial Grams | W (over them unless split) | X
+        constexpr int B2 = 2 * OB;
+        cx.wpanel = split > 1 ? cx.stage + Smem<T>::PART : cx.stage;
+        cx.panel = cx.stage + (split > 1 ? Smem<T>::PART + B2 * cx.wstride : max(Smem<T>::PART, B2 * cx.wstride));
     }
+    cx.tau = d.mu ? (T)(1.0 / *d.mu) : T(0);
     // scaled off-diagonals below ~64 eps are at the rounding level of the
     // fresh pivot Grams
     const T t_eff = fmax(tol, T(64) * num<T>::eps());
-    cl.sync();
-    int R = 0;        // rounds run so far (selects the counter of the round)
+    int par = 0;          // parity of the round: which copy of `top` it reads
     for (int sw = 0; sw < sweeps; ++sw) {
-        T mine = T(0);
-        for (int r = 0; r < nb - 1; ++r, ++R) {
-            if (d.ctr) {
-                // pivots go to whichever CTA of the cluster is free: a pivot
-                // that rotates costs several times one that is already
-                // orthogonal.  Counter R & 1 serves this round; the other one,
-                // last used in the previous round (finished at the cluster
-                // barrier), is reset for the next.
-                if (rank == 0 && t == 0) {
-                    atomicExch(d.ctr + ((R + 1) & 1), 0);
-                    __threadfence();
+        if (KEEP ? sw == 0 : sw <= 4 && sw % 2 == 0) {
+            // squared norms, a warp per column
+            for (int j = rank * NW + warp; j < d.p; j += csize * NW) {
+                const T* const x = d.X + j * d.ldx;
+                T acc = T(0);
+                for (int i = lane; i < d.L; i += 32) {
+                    const T v = __ldcg(x + i);
+                    acc = fma(v, v, acc);
                 }
-            }
-            for (int k = 0;; ++k) {
-                int P = rank + k * csize;          // fixed share without a counter
-                if (d.ctr) {
-                    if (t == 0) sm.pick = atomicAdd(d.ctr + (R & 1), 1);
-                    __syncthreads();
-                    P = sm.pick;
-                    __syncthreads();
-                }
-                if (P >= npairs) break;
-                const int a = circle_item(P, r, nb), c = circle_item(nb - 1 - P, r, nb);
-                mine = fmax(mine, osj_pivot<T>(d, sm, a, c));
+                acc = warp_sum(acc);
+                if (lane == 0) nrm[j] = acc;
             }
             cl.sync();
+            // each column's place in the order: how many come before it
+            constexpr int TS = Smem<T>::PART;
+            T* const stage = reinterpret_cast<T*>(&sm + 1);
+            for (int jb = rank * NT; !KEEP && jb < d.p; jb += csize * NT) {
+                const int j = jb + t;
+                const auto kj = key_of(j < d.p ? __ldcg(nrm + j) : T(0));
+                int before = 0;
+                for (int i0 = 0; i0 < d.p; i0 += TS) {
+                    const int cnt = min(TS, d.p - i0);
+                    __syncthreads();
+                    for (int i = t; i < cnt; i += NT) stage[i] = __ldcg(nrm + i0 + i);
+                    __syncthreads();
+                    for (int i = 0; i < cnt; ++i) {
+                        const auto ki = key_of(stage[i]);
+                        before += (ki > kj || (ki == kj && i0 + i < j)) ? 1 : 0;
+                    }
+                }
+                if (j < d.p) d.ord[before] = j;
+            }
+            if (!KEEP) cl.sync();
+            // the two largest norms of every column block
+            if (rank == 0)
+                for (int b = t; b < nb; b += NT) {
+                    T n1 = T(0), n2 = T(0);
+                    for (int q = 0; q < OB; ++q) {
+                        const int pos = b * OB + q;
+                        if (pos >= d.p || (!KEEP && q >= 2)) break;
+                        const T v = __ldcg(nrm + (KEEP ? pos : __ldcg(d.ord + pos)));
+                        if (!(v <= n1)) { n2 = n1; n1 = v; }
+                        else if (!(v <= n2)) n2 = v;
+                    }
+                    top[(par * nb + b) * 2] = n1;
+                    top[(par * nb + b) * 2 + 1] = n2;
+                }
+            cl.sync();
+            if (sw == 0) {
+                // the largest column: the scale of the measure and of the rounding floor
+                T mx = T(0);
+                for (int b = lane; b < nb; b += 32) mx = fmax(mx, __ldcg(top + 2 * b));
+                cx.scale = warp_max(mx);
+                const T noise = T(4) * num<T>::eps();
+                cx.floor2 = noise * noise * cx.scale + num<T>::tiny();
+            }
+        }
+        T mine = T(0);
+        for (int r = 0; r < nb - 1; ++r) {
+            cx.first_round = r == 0;
+            const T* const ti = top + par * nb * 2;
+            T* const to = top + (par ^ 1) * nb * 2;
+            // Every warp lists the pivots that need work, 32 pairs at a time,
+            // and the teams take them in turn.  A pair of column blocks is
+            // skipped when no two of its columns reach a^2 + b^2 > tau^2 or when
+            // at most one of them is above the rounding floor: its measure
+            // would be zero.  The norms are one rotation old at most and good
+            // to a few eps of the column block's largest, hence the margins.
+            // (Sorted: nor does any pair come near Gershgorin's bound.)
+            int cnt = 0;
+            bool met = split == 1;
+            for (int P0 = 0; P0 < npairs; P0 += 32) {
+                const int P = P0 + lane;
+                bool work = false;
+                int a = 0, c = 0;
+                if (P < npairs) {
+                    a = circle_item(P, r, nb);
+                    c = circle_item(nb - 1 - P, r, nb);
+                    const T a1 = __ldcg(ti + 2 * a), a2 = __ldcg(ti + 2 * a + 1);
+                    const T c1 = __ldcg(ti + 2 * c), c2 = __ldcg(ti + 2 * c + 1);
+                    const T n1 = a1 > c1 ? a1 : c1, n2 = a1 > c1 ? (a2 > c1 ? a2 : c1) : (c2 > a1 ? c2 : a1);
+                    work = !((n1 + (KEEP ? n2 : T(d.p) * sqrt(n1 * n2))) * T(1.001) <= cx.tau * cx.tau) &&
+                           !(n2 * T(4) <= cx.floor2);
+                    if (!work && rank == 0 && warp == 0) {
+                        to[2 * a] = a1; to[2 * a + 1] = a2;
+                        to[2 * c] = c1; to[2 * c + 1] = c2;
+                    }
+                }
+                unsigned mask = __ballot_sync(0xffffffffu, work);
+                while (mask) {
+                    const int bit = __ffs(mask) - 1;
+                    mask &= mask - 1;
+                    if (cnt++ % nteams != team) continue;
+                    const int pa = __shfl_sync(0xffffffffu, a, bit), pc = __shfl_sync(0xffffffffu, c, bit);
+                    mine = fmax(mine, osj_pivot<T, NT, KEEP>(sm, cl, cx, pa, pc, to + 2 * pa, to + 2 * pc));
+                    met = true;
+                }
+            }
+            // a split pivot has one cluster barrier inside; every CTA passes
+            // exactly one per round (a round has at most one pivot per team)
+            if (!met) cl.sync();
+            cl.sync();
+            par ^= 1;
         }
         if (t == 0) {
             atomic_max_nonneg(d.off + sw % 3, mine);
@@ -368,11 +962,64 @@ __global__ void __launch_bounds__(NT, 5) osj_svd(const OsjDesc<T>* __restrict__ 
         cl.sync();
         const T o = __ldcg(d.off + sw % 3);
         if (rank == 0 && t == 0 && sweeps_run) sweeps_run[mat] += 1;
-        if (o <= t_eff || (quad_exit && T(16) * o * o <= t_eff)) {
-            if (rank == 0 && t == 0) *d.done = 1;
-            break;
-        }
+        if (o <= t_eff || (quad_exit && T(16) * o * o <= t_eff)) break;
     }
+}
+
+// pivots of a round
+template <typename T>
+int pairs_of(int p) { return (p + 2 * Cfg<T>::OB - 1) / (2 * Cfg<T>::OB); }
+
+template <typename T>
+size_t smem_bytes(const OsjShape& sh) {
+    constexpr size_t B2 = Smem<T>::B2, part = Smem<T>::PART;
+    size_t words = Smem<T>::STAGE;
+    if (sh.wide) {
+        const size_t w = B2 * (size_t)wpanel_stride<T>(sh.max_p, sh.split);
+        // a tile may read (never write) up to three 32-row groups past the last one
+        words = (sh.split > 1 ? part + w : std::max(part, w)) + B2 * (size_t)panel_stride<T>(sh.max_L, sh.split) + 128;
+    }
+    return sizeof(Smem<T>) + sizeof(T) * words;
+}
+
+template <typename T, int NT, bool KEEP>
+cudaError_t launch(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
+                   cudaStream_t s, int quad_exit, int* resident) {
+    // resident != nullptr: no launch, only how many such clusters fit the device
+    static std::atomic<uint64_t> smem_set{0};
+    cudaError_t e = ensure_smem_limit(osj_svd<T, NT, KEEP>, NT == NT_FEW ? (int)SMEM_MAX : (int)smem_bytes<T>(OsjShape{1, 1, 0, 1, 1}),
+                                      smem_set);
+    if (e != cudaSuccess) return e;
+    if (shape.cluster > 8) {
+        e = cudaFuncSetAttribute(osj_svd<T, NT, KEEP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)shape.cluster, (unsigned)nmat, 1);
+    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.dynamicSmemBytes = smem_bytes<T>(shape);
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)shape.cluster; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (resident) return cudaOccupancyMaxActiveClusters(resident, osj_svd<T, NT, KEEP>, &cfg);
+    e = cudaLaunchKernelEx(&cfg, osj_svd<T, NT, KEEP>, d_desc, sweeps, tol, sweeps_run, quad_exit, shape.split);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+template <typename T>
+int resident_clusters(OsjShape sh) {
+    int n = 0;
+    if (smem_bytes<T>(sh) > SMEM_MAX) return 0;
+    // (both schedules use the same shared memory and register limits)
+    const cudaError_t e = sh.wide ? launch<T, NT_FEW, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, &n)
+                                  : launch<T, NT_MANY, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, &n);
+    if (e != cudaSuccess) n = 0;
+    (void)cudaGetLastError();
+    return n;
 }
 
 }  // namespace
@@ -382,93 +1029,48 @@ int osj_max_cluster() {
     // 16 (the non-portable limit) when the device schedules clusters that
     // large for this kernel, else 8
     static std::atomic<int> big_ok{-1};
-    if (big_ok.load() < 0) {
-        int ok = 0;
-        const size_t smem = sizeof(Smem<T>);
-        static std::atomic<uint64_t> smem_set{0};
-        if (ensure_smem_limit(osj_svd<T>, (int)smem, smem_set) == cudaSuccess &&
-            cudaFuncSetAttribute(osj_svd<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(16, 1, 1);
-            cfg.blockDim = dim3(NT, 1, 1);
-            cfg.dynamicSmemBytes = smem;
-            cudaLaunchAttribute at;
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = 16; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            int nclus = 0;
-            if (cudaOccupancyMaxActiveClusters(&nclus, osj_svd<T>, &cfg) == cudaSuccess && nclus > 0) ok = 1;
-        }
-        (void)cudaGetLastError();
-        big_ok.store(ok);
-    }
+    if (big_ok.load() < 0) big_ok.store(resident_clusters<T>(OsjShape{16, 1, 0, 1, 1}) > 0 ? 1 : 0);
     return big_ok.load() ? 16 : 8;
 }
 
 template <typename T>
-int default_cluster(int nmat, int max_pairs, int cmax, size_t smem) {
-    int best = 1;
-    for (int c = std::min(cmax, std::max(1, max_pairs)); c >= 1; c /= 2) {
-        if (c > 8 && cudaFuncSetAttribute(osj_svd<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-            continue;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)c, 1, 1);
-        cfg.blockDim = dim3(NT, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        int nclus = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclus, osj_svd<T>, &cfg) == cudaSuccess && nclus >= nmat) {
-            best = c;
-            break;
-        }
-        best = c;
+OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster) {
+    // Cluster size: the caller's choice (autotuned), else the largest (up to
+    // one CTA per pivot of a round) at which every block's cluster can be
+    // resident at once -- a block waiting for a second wave would double the
+    // time of the whole batch.  A cluster with room for several CTAs per pivot
+    // splits its pivots, while a member keeps at least two chunks of rows.
+    // Wide CTAs where a whole round's pivots fit the chip that way.
+    const int pairs = std::max(1, pairs_of<T>(max_p)), cmax = osj_max_cluster<T>();
+    const int limit = cluster > 0 ? std::min(cluster, cmax) : cmax;
+    auto fits = [&](const OsjShape& sh) { return resident_clusters<T>(sh) >= nmat; };
+    for (int split = 4; split >= 1; split /= 2) {
+        const OsjShape sh{pairs * split, split, 1, max_L, max_p};
+        if (sh.cluster > limit || (split > 1 && split * 64 > max_L + max_p)) continue;
+        if (fits(sh)) return sh;
     }
-    (void)cudaGetLastError();
-    return best;
+    for (int c = std::min(limit, pairs); c > 1; --c)
+        if (cluster > 0 || fits(OsjShape{c, 1, 0, max_L, max_p})) return OsjShape{c, 1, 0, max_L, max_p};
+    return OsjShape{1, 1, 0, max_L, max_p};
 }
 
 template <typename T>
-cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, int max_pp, int sweeps, T tol, int* sweeps_run,
-                       cudaStream_t s, int cluster, int quad_exit) {
-    if (nmat <= 0 || max_pp <= 0 || sweeps <= 0) return cudaSuccess;
-    const int max_pairs = max_pp / B2;
-    const size_t smem = sizeof(Smem<T>);
-    static std::atomic<uint64_t> smem_set{0};
-    cudaError_t e = ensure_smem_limit(osj_svd<T>, (int)smem, smem_set);
-    if (e != cudaSuccess) return e;
-    // cluster size: the caller's choice (autotuned), else the largest (up to
-    // one CTA per pivot of a round) at which every block's cluster can be
-    // resident at once -- a block waiting for a second wave would double the
-    // time of the whole batch
-    const int cmax = osj_max_cluster<T>();
-    int csize = cluster > 0 ? std::min(cluster, cmax) : default_cluster<T>(nmat, max_pairs, cmax, smem);
-    csize = std::max(1, std::min(csize, max_pairs));
-    if (csize > 8) {
-        e = cudaFuncSetAttribute(osj_svd<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
+cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
+                       cudaStream_t s, OsjMode mode, int quad_exit) {
+    if (nmat <= 0 || sweeps <= 0) return cudaSuccess;
+    if constexpr (sizeof(T) == 4) {
+        if (mode == OsjMode::kept)
+            return shape.wide ? launch<T, NT_FEW, true>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr)
+                              : launch<T, NT_MANY, true>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr);
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)csize, (unsigned)nmat, 1);
-    cfg.blockDim = dim3(NT, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)csize; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, osj_svd<T>, d_desc, sweeps, tol, sweeps_run, quad_exit);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return shape.wide ? launch<T, NT_FEW, false>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr)
+                      : launch<T, NT_MANY, false>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr);
 }
 
-template cudaError_t osj_sweeps<float>(const OsjDesc<float>*, int, int, int, float, int*, cudaStream_t, int, int);
-template cudaError_t osj_sweeps<double>(const OsjDesc<double>*, int, int, int, double, int*, cudaStream_t, int, int);
+template cudaError_t osj_sweeps<float>(const OsjDesc<float>*, int, OsjShape, int, float, int*, cudaStream_t, OsjMode, int);
+template cudaError_t osj_sweeps<double>(const OsjDesc<double>*, int, OsjShape, int, double, int*, cudaStream_t, OsjMode, int);
+template OsjShape osj_shape<float>(int, int, int, int);
+template OsjShape osj_shape<double>(int, int, int, int);
 template int osj_max_cluster<float>();
 template int osj_max_cluster<double>();
 

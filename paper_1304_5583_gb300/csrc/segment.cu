@@ -243,8 +243,8 @@ __global__ void col_norms(const float* __restrict__ X, int64_t rows, int p, doub
 struct SegBuf {
     float *X, *W, *U, *Uk, *A, *Y, *Y2, *G, *Ri;
     double *d, *cost;
-    float *sc, *of3, *d2;
-    int *done, *on, *idx, *labels;
+    float *cols, *of3, *d2;
+    int *ord, *on, *idx, *labels;
     OsjDesc<float>* od;
     GemmDesc<float>* gd;
 };
@@ -269,10 +269,10 @@ size_t seg_layout(SegBuf& b, char* base, int64_t n, int k, int K, int restarts) 
     b.Ri = (float*)take(sizeof(float) * K * K);
     b.d = (double*)take(sizeof(double) * std::max<int64_t>(n, k));
     b.cost = (double*)take(sizeof(double) * restarts);
-    b.sc = (float*)take(sizeof(float));
+    b.cols = (float*)take(sizeof(float) * 2 * pp);
     b.of3 = (float*)take(sizeof(float) * 3);
     b.d2 = (float*)take(sizeof(float) * n * restarts);
-    b.done = (int*)take(sizeof(int));
+    b.ord = (int*)take(sizeof(int) * pp);
     b.on = (int*)take(sizeof(int));
     b.idx = (int*)take(sizeof(int) * k);
     b.labels = (int*)take(sizeof(int) * n * restarts);
@@ -338,12 +338,11 @@ int lrr_segment(const float* F, int64_t ldf, const float* G, int64_t ldg, int64_
     }
     OsjDesc<float> od{};
     const int one = 1;
-    od.X = b.X; od.W = b.W; od.done = b.done; od.off = b.of3; od.active = b.on; od.scale = b.sc; od.mu = nullptr;
+    od.X = b.X; od.W = b.W; od.off = b.of3; od.cols = b.cols; od.ord = b.ord; od.active = b.on; od.mu = nullptr;
     od.ldx = n; od.ldw = pp; od.L = (int)n; od.p = kk; od.pp = pp; od.strict = 1;
     STRY(cudaMemcpyAsync(b.od, &od, sizeof(od), cudaMemcpyHostToDevice, s));
     STRY(cudaMemcpyAsync(b.on, &one, sizeof(int), cudaMemcpyHostToDevice, s));
-    k::col_norm_max<float><<<1, 256, 0, s>>>(b.od, b.on, b.sc, 1);
-    STRY(osj_sweeps<float>(b.od, 1, pp, 40, 2e-6f, nullptr, s, 0));
+    STRY(osj_sweeps<float>(b.od, 1, osj_shape<float>(1, kk, (int)n), 40, 2e-6f, nullptr, s, OsjMode::kept));
     // kept directions: singular values s_j = ||x_j|| above rel_tol * max
     col_norms<<<(unsigned)(((int64_t)kk * 32 + 255) / 256), 256, 0, s>>>(b.X, n, kk, b.d);
     std::vector<double> sv((size_t)kk, 0.0);

@@ -105,8 +105,8 @@ struct Buffers {
     std::vector<int*> rot;
     int* rot_d;
     double *mu, *mu_fin, *resid;
-    int *act, *iters, *svt_on, *rank_cur, *rank_fin, *need_exact, *conv_bound, *conv, *jdone, *jctr, *colblk, *flag;
-    T *r1, *dmax, *r2x, *jscale, *joff;
+    int *act, *iters, *svt_on, *rank_cur, *rank_fin, *need_exact, *conv_bound, *conv, *jord, *colblk, *flag;
+    T *r1, *dmax, *r2x, *jcols, *joff;
     int64_t* perm;
     // descriptor / pointer tables
     GemmDesc<T>* gd;       // 12 * t descriptors
@@ -220,14 +220,15 @@ Buffers<T> carve(Arena& a, const lrr_problem* p, bool need_md, const std::vector
     b.need_exact = a.take<int>(t);
     b.conv_bound = a.take<int>(t);
     b.conv = a.take<int>(t);
-    b.jdone = a.take<int>(t);
-    b.jctr = a.take<int>(2 * (size_t)t);
+    size_t cols_pad = 0;      // every block's columns, each padded to the pivot width
+    for (int i = 0; i < t; ++i) cols_pad += (size_t)blk[i].ppmax;
+    b.jord = a.take<int>(cols_pad);
     b.colblk = a.take<int>(n);
     b.flag = a.take<int>(4);
     b.r1 = a.take<T>(t);
     b.dmax = a.take<T>(t);
     b.r2x = a.take<T>(t);
-    b.jscale = a.take<T>(t);
+    b.jcols = a.take<T>(2 * cols_pad);
     b.joff = a.take<T>(3 * (size_t)t);   // three convergence slots per block
     b.perm = a.take<int64_t>(n);
     b.gd = a.take<GemmDesc<T>>(16 * (size_t)t + 16);
@@ -602,14 +603,14 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     constexpr int B2 = osj_pivot_width();
     std::vector<int> pv((size_t)t), ppv((size_t)t);
     std::vector<char> tall((size_t)t);
-    int max_p = 0, max_pp = 0, max_l = 0;
+    int max_p = 0, max_pp = 0, max_L = 0;
     for (int i = 0; i < t; ++i) {
         tall[i] = blk[i].l <= r;
         pv[i] = std::min(r, blk[i].l);
         ppv[i] = round_up(pv[i], B2);
         max_p = std::max(max_p, pv[i]);
         max_pp = std::max(max_pp, ppv[i]);
-        max_l = std::max(max_l, blk[i].l);
+        max_L = std::max(max_L, std::max(r, blk[i].l));
     }
     LRR_CUDA_TRY(cudaMemcpyAsync(B.hp, B.h.data(), sizeof(T*) * t, cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(cudaMemcpyAsync(B.Wp, B.W.data(), sizeof(T*) * t, cudaMemcpyHostToDevice, s));
@@ -618,14 +619,16 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     LRR_CUDA_TRY(cudaMemcpyAsync(B.pv, pv.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(cudaMemcpyAsync(B.ppv, ppv.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
     std::vector<OsjDesc<T>> jdh((size_t)t);
+    int64_t cols_off = 0;
     for (int i = 0; i < t; ++i) {
         OsjDesc<T>& j = jdh[i];
         j.X = B.D + blk[i].col0 * r;
         j.ldx = tall[i] ? r : blk[i].l;
         j.L = tall[i] ? r : blk[i].l;
         j.W = B.W[i]; j.ldw = ppv[i]; j.p = pv[i]; j.pp = ppv[i];
-        j.done = B.jdone + i; j.off = B.joff + 3 * i; j.active = B.svt_on + i; j.scale = B.jscale + i;
-        j.ctr = B.jctr + 2 * i;
+        j.off = B.joff + 3 * i; j.active = B.svt_on + i;
+        j.cols = B.jcols + 2 * cols_off; j.ord = B.jord + cols_off;
+        cols_off += blk[i].ppmax;
         j.mu = B.mu + i;
         j.strict = (dfc && t > 1 && i == 0) ? 1 : 0;
     }
@@ -649,9 +652,8 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         }
         if (!have) {
             std::vector<int> cand;
-            const int max_pairs = max_pp / B2, cmax = osj_max_cluster<T>();
             for (int c : {4, 8, 16})
-                if (c <= cmax && (c <= max_pairs || cand.empty())) cand.push_back(std::min(c, max_pairs));
+                if (c <= osj_max_cluster<T>()) cand.push_back(c);
             std::vector<int> on((size_t)t, 1);
             std::vector<double> mu_t((size_t)t, 1e10);
             LRR_CUDA_TRY(cudaMemcpyAsync(B.svt_on, on.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
@@ -664,9 +666,9 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
                 k::fill_hash<T><<<grid1(r * n), 256, 0, s>>>(B.D, r * n, 12345u);
                 for (int i = 0; i < t; ++i)
                     k::init_padded<T><<<grid1((int64_t)ppv[i] * ppv[i]), 256, 0, s>>>(B.W[i], pv[i], ppv[i], T(1), 1);
-                k::col_norm_max<T><<<t, 256, 0, s>>>(B.jd, B.svt_on, B.jscale, t);
                 cudaEventRecord(ta, s);
-                const cudaError_t e = osj_sweeps<T>(B.jd, t, max_pp, 2, jtol_of<T>(), nullptr, s, c, quad_exit);
+                const cudaError_t e = osj_sweeps<T>(B.jd, t, osj_shape<T>(t, max_p, max_L, c), 2, jtol_of<T>(), nullptr, s,
+                                                    OsjMode::kept, quad_exit);
                 cudaEventRecord(tb, s);
                 if (e != cudaSuccess || cudaEventSynchronize(tb) != cudaSuccess) {
                     cudaEventDestroy(ta); cudaEventDestroy(tb);
@@ -682,6 +684,10 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
             g_tune_cluster[key] = jcluster;
         }
     }
+    // launch shape of the Jacobi for the blocks still active (the others' clusters
+    // leave at once); re-picked as blocks converge
+    int jshape_n = t;
+    OsjShape jshape = osj_shape<T>(t, max_p, max_L, jcluster);
 
     // grouped GEMM descriptor sets
     std::vector<GemmDesc<T>> gh;
@@ -792,7 +798,6 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     const T jtol = jtol_of<T>();
     const unsigned wgrid_n = (unsigned)((n * 32 + 255) / 256);
     auto nl = [&](int si) -> int64_t { return si < 0 ? 0 : 1; };
-    const int64_t jac_launches = 1;   // every sweep of every block in one launch
     // relative error bound of the bf16 stop-test product (stop_tc_decide), with a factor-2 margin
     const double tc_rel = 2.0 * (2.0 / 256.0 + 1.0 / 65536.0 + (double)r / 16777216.0);
     // the tensor-core stage of the stop test runs in chunks that follow one in
@@ -802,15 +807,14 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         prof.iterations += 1;
         // J-step: SVT of A = Zt + Y2t/mu through the Gram eigendecomposition
         prof.begin();
-        k::svt_gate<T><<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.afro, B.mu, B.svt_on, B.jscale, B.svtcalls,
+        k::svt_gate<<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.afro, B.mu, B.svt_on, B.svtcalls,
                                                          B.fp32_on, B.gemm32, switch_margin, t);
         LRR_CUDA_TRY(run_set(S_XT));
         LRR_CUDA_TRY(run_set(S_XW));
         prof.end(LRR_PH_GRAM, 1 + nl(S_XT) + nl(S_XW));
         prof.begin();
-        k::col_norm_max<T><<<t, 256, 0, s>>>(B.jd, B.svt_on, B.jscale, t);
-        LRR_CUDA_TRY(osj_sweeps<T>(B.jd, t, max_pp, sweeps, jtol, B.jsweeps, s, jcluster, quad_exit));
-        prof.end(LRR_PH_JACOBI, jac_launches + 1);
+        LRR_CUDA_TRY(osj_sweeps<T>(B.jd, t, jshape, sweeps, jtol, B.jsweeps, s, OsjMode::kept, quad_exit));
+        prof.end(LRR_PH_JACOBI, 1);
         prof.begin();
         k::svt_weights<T><<<t, 256, 0, s>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
         // W^T W and W (W^T W): first-order inverse for J, Newton-Schulz for the warm start
@@ -890,6 +894,13 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         std::vector<int> ah((size_t)t), fh((size_t)t);
         int done_it = 0, nneed = 0;
         const int chunk = 4;
+        auto pick_shape = [&](const std::vector<int>& act) {
+            const int na = (int)std::count_if(act.begin(), act.end(), [](int v) { return v != 0; });
+            if (na == 0 || na == jshape_n) return;
+            jshape_n = na;
+            jshape = osj_shape<T>(na, max_p, max_L, na == t ? jcluster : 0);
+        };
+        pick_shape(act0);
         tc_window = false;
         while (done_it < o->max_iter) {
             for (int c = 0; c < chunk && done_it < o->max_iter; ++c, ++done_it) {
@@ -913,6 +924,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
                 if (!any16) bf16_phase = false;
             }
             if (std::none_of(ah.begin(), ah.end(), [](int v) { return v != 0; })) break;
+            pick_shape(ah);
         }
         return LRR_OK;
     };
@@ -1089,7 +1101,7 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
     const int pp = round_up(p, B2);
     Arena sz(nullptr);
     auto lay = [&](Arena& a, T** X, T** W, T** H, T** T1, T** h, int** ints, double** dbl, OsjDesc<T>** od,
-                   GemmDesc<T>** gd, T** Wp, T** Hp, T** hp, T** scl, T** off, T** T1p) {
+                   GemmDesc<T>** gd, T** Wp, T** Hp, T** hp, T** off, T** T1p) {
         *X = a.take<T>((size_t)L * p);
         *W = a.take<T>((size_t)pp * pp);
         *H = a.take<T>((size_t)pp * pp);
@@ -1102,16 +1114,15 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
         *Wp = reinterpret_cast<T*>(a.take<T*>(1));
         *Hp = reinterpret_cast<T*>(a.take<T*>(1));
         *hp = reinterpret_cast<T*>(a.take<T*>(1));
-        *scl = a.take<T>(1);
         *off = a.take<T>(3);
         *T1p = reinterpret_cast<T*>(a.take<T*>(1));
     };
-    T *X, *W, *H, *T1, *h, *Wp, *Hp, *hp, *scl, *off, *T1p;
+    T *X, *W, *H, *T1, *h, *Wp, *Hp, *hp, *off, *T1p;
     int* ints;
     double* dbl;
     OsjDesc<T>* od;
     GemmDesc<T>* gd;
-    lay(sz, &X, &W, &H, &T1, &h, &ints, &dbl, &od, &gd, &Wp, &Hp, &hp, &scl, &off, &T1p);
+    lay(sz, &X, &W, &H, &T1, &h, &ints, &dbl, &od, &gd, &Wp, &Hp, &hp, &off, &T1p);
     void* mem = nullptr;
     if (cudaMallocAsync(&mem, sz.off + kAlign, s) != cudaSuccess) return LRR_ERR_CUDA;
     struct Free {
@@ -1119,11 +1130,10 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
         ~Free() { if (p) cudaFreeAsync(p, s); }
     } guard{mem, s};
     Arena a(mem);
-    lay(a, &X, &W, &H, &T1, &h, &ints, &dbl, &od, &gd, &Wp, &Hp, &hp, &scl, &off, &T1p);
+    lay(a, &X, &W, &H, &T1, &h, &ints, &dbl, &od, &gd, &Wp, &Hp, &hp, &off, &T1p);
     int* act = ints;          // [0]
     int* on = ints + 1;       // [1]
     int* rk = ints + 2;       // [2]
-    int* done = ints + 3;     // [3]
     int* swp = ints + 4;      // [4]
     double* mu = dbl;
     const int one[2] = {1, 1};
@@ -1143,7 +1153,9 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
     LRR_CUDA_TRY(cudaMemcpyAsync(pv, &pvals[0], sizeof(int), cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(cudaMemcpyAsync(ppv, &pvals[1], sizeof(int), cudaMemcpyHostToDevice, s));
     OsjDesc<T> d{};
-    d.X = X; d.W = W; d.done = done; d.off = off; d.active = on; d.scale = scl; d.mu = mu;
+    d.X = X; d.W = W; d.off = off; d.active = on; d.mu = mu;
+    d.cols = T1;                          // T1 and H are written only after the Jacobi: its scratch until then
+    d.ord = reinterpret_cast<int*>(H);
     d.ldx = L; d.ldw = pp; d.L = L; d.p = p; d.pp = pp; d.strict = 1;
     LRR_CUDA_TRY(cudaMemcpyAsync(od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     GemmDesc<T> g[5];
@@ -1156,8 +1168,8 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
     g[3].kscale = h;
     LRR_CUDA_TRY(cudaMemcpyAsync(gd, g, sizeof(g), cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(gemm_grouped<T>(gd, 1, !tall, false, L, p, s));
-    k::col_norm_max<T><<<1, 256, 0, s>>>(od, on, scl, 1);
-    LRR_CUDA_TRY(osj_sweeps<T>(od, 1, pp, 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), swp, s));
+    LRR_CUDA_TRY(osj_sweeps<T>(od, 1, osj_shape<T>(1, p, L), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), swp, s,
+                               OsjMode::sorted));
     k::svt_weights<T><<<1, 256, 0, s>>>(od, reinterpret_cast<T* const*>(hp), act, on, mu, rk, 1);
     LRR_CUDA_TRY(gemm_grouped<T>(gd + 1, 1, true, false, p, p, s));
     LRR_CUDA_TRY(gemm_grouped<T>(gd + 2, 1, false, false, p, p, s));
@@ -1211,7 +1223,7 @@ int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double
     const int L = (int)(tall ? rows : cols);
     const int pp = round_up(p, B2);
     struct Parts {
-        T *X, *W, *H, *T1, *h, *scl, *off;
+        T *X, *W, *H, *T1, *h, *off;
         T **Wp, **Hp, **hp, **T1p;
         int* ints;
         double* dbl;
@@ -1233,7 +1245,6 @@ int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double
         q.Hp = a.take<T*>(1);
         q.hp = a.take<T*>(1);
         q.T1p = a.take<T*>(1);
-        q.scl = a.take<T>(1);
         q.off = a.take<T>(3);
         return q;
     };
@@ -1247,7 +1258,6 @@ int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double
     int* act = q.ints;
     int* on = q.ints + 1;
     int* rk = q.ints + 2;
-    int* done = q.ints + 3;
     int* swp = q.ints + 4;
     int* pv = q.ints + 8;
     int* ppv = q.ints + 9;
@@ -1266,7 +1276,9 @@ int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double
     LRR_CUDA_TRY(cudaMemcpyAsync(q.T1p, &ptrs[3], sizeof(T*), cudaMemcpyHostToDevice, s));
     k::init_padded<T><<<grid1((int64_t)pp * pp), 256, 0, s>>>(q.W, p, pp, T(1), 1);
     OsjDesc<T> d{};
-    d.X = q.X; d.W = q.W; d.done = done; d.off = q.off; d.active = on; d.scale = q.scl; d.mu = mu;
+    d.X = q.X; d.W = q.W; d.off = q.off; d.active = on; d.mu = mu;
+    d.cols = q.T1;                        // T1 and H are written only after the Jacobi: its scratch until then
+    d.ord = reinterpret_cast<int*>(q.H);
     d.ldx = L; d.ldw = pp; d.L = L; d.p = p; d.pp = pp; d.strict = 1;
     LRR_CUDA_TRY(cudaMemcpyAsync(q.od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     GemmDesc<T> g[4];
@@ -1278,8 +1290,8 @@ int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double
     g[3].kscale = q.h;
     LRR_CUDA_TRY(cudaMemcpyAsync(q.gd, g, sizeof(g), cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(gemm_grouped<T>(q.gd, 1, !tall, false, L, p, s));
-    k::col_norm_max<T><<<1, 256, 0, s>>>(q.od, on, q.scl, 1);
-    LRR_CUDA_TRY(osj_sweeps<T>(q.od, 1, pp, 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), swp, s));
+    LRR_CUDA_TRY(osj_sweeps<T>(q.od, 1, osj_shape<T>(1, p, L), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), swp, s,
+                               OsjMode::sorted));
     k::svt_weights<T><<<1, 256, 0, s>>>(q.od, q.hp, act, on, mu, rk, 1);
     LRR_CUDA_TRY(gemm_grouped<T>(q.gd + 1, 1, true, false, p, p, s));
     LRR_CUDA_TRY(gemm_grouped<T>(q.gd + 2, 1, false, false, p, p, s));
@@ -1368,14 +1380,16 @@ int local_impl(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_res
     int64_t fwords = 0;
     for (int i = 0; i < t; ++i) fwords += 2 * l[i] * kmax[i];   // F_i, G_i
     const int B2 = osj_pivot_width();
-    int64_t wwords = 0;
+    int64_t wwords = 0, kpad = 0;
     std::vector<int> kp((size_t)t);
     for (int i = 0; i < t; ++i) {
         kp[i] = round_up((int)kmax[i], B2);
         wwords += (int64_t)kp[i] * kp[i] + l[i] * kmax[i] + l[i] * kmax[i];   // W_i, X_i, T_i
+        kpad += kp[i];
     }
     const size_t bytes = sizeof(T) * (size_t)(words + fwords + wwords) + sizeof(int64_t) * n +
-                         (sizeof(OsjDesc<T>) + sizeof(GemmDesc<T>) * 2 + 64 * sizeof(T) + 64) * (size_t)t + 4096 * 4;
+                         (sizeof(OsjDesc<T>) + sizeof(GemmDesc<T>) * 2 + 64 * sizeof(T) + 64) * (size_t)t + 4096 * 4 +
+                         (2 * sizeof(T) + sizeof(int)) * (size_t)kpad + 512;
     void* mem = nullptr;
     if (cudaMallocAsync(&mem, bytes, s) != cudaSuccess) return LRR_ERR_CUDA;
     struct Free {
@@ -1397,9 +1411,9 @@ int local_impl(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_res
     }
     OsjDesc<T>* od = a.take<OsjDesc<T>>(t);
     GemmDesc<T>* gd = a.take<GemmDesc<T>>(2 * (size_t)t);
-    T* scl = a.take<T>(t);
+    T* cols = a.take<T>(2 * kpad);
+    int* ord = a.take<int>(kpad);
     T* off3 = a.take<T>(3 * (size_t)t);
-    int* done = a.take<int>(t);
     int* on = a.take<int>(t);
     T* hk = a.take<T>((size_t)t * 1);   // placeholder (per-block masks follow)
     (void)hk;
@@ -1437,6 +1451,7 @@ int local_impl(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_res
     std::vector<OsjDesc<T>> dh((size_t)t);
     std::vector<GemmDesc<T>> g1v((size_t)t);
     int max_kp = 0;
+    int64_t cols_off = 0;
     for (int i = 0; i < t; ++i) {
         const int ki = std::max(1, fk[i]);
         k::init_padded<T><<<grid1((int64_t)kp[i] * kp[i]), 256, 0, s>>>(W[i], ki, kp[i], T(1), 1);
@@ -1444,7 +1459,8 @@ int local_impl(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_res
         g1v[i] = g;
         OsjDesc<T>& d = dh[i];
         d = OsjDesc<T>{};
-        d.X = X[i]; d.W = W[i]; d.done = done + i; d.off = off3 + 3 * i; d.active = on + i; d.scale = scl + i;
+        d.X = X[i]; d.W = W[i]; d.off = off3 + 3 * i; d.active = on + i;
+        d.cols = cols + 2 * cols_off; d.ord = ord + cols_off; cols_off += kp[i];
         d.mu = nullptr; d.ldx = l[i]; d.ldw = kp[i]; d.L = (int)l[i]; d.p = ki; d.pp = round_up(ki, B2);
         d.strict = 1;
         max_kp = std::max(max_kp, d.pp);
@@ -1455,8 +1471,8 @@ int local_impl(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_res
     LRR_CUDA_TRY(cudaMemcpyAsync(gd, g1v.data(), sizeof(GemmDesc<T>) * t, cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(gemm_grouped<T>(gd, t, true, false, (int)lmax, max_kp, s));
     LRR_CUDA_TRY(cudaMemcpyAsync(od, dh.data(), sizeof(OsjDesc<T>) * t, cudaMemcpyHostToDevice, s));
-    k::col_norm_max<T><<<t, 256, 0, s>>>(od, on, scl, t);
-    LRR_CUDA_TRY(osj_sweeps<T>(od, t, max_kp, 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), nullptr, s, 0));
+    LRR_CUDA_TRY(osj_sweeps<T>(od, t, osj_shape<T>(t, max_kp, (int)lmax), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6),
+                               nullptr, s, OsjMode::kept));
     // singular values to the host; the global top `rank`
     std::vector<std::vector<T>> xs((size_t)t);
     std::vector<std::tuple<double, int, int>> all;

@@ -212,8 +212,9 @@ struct Engine {
     int* rank_d;
     T *Wh, *Wg, *Wt;             // W^T W, W (W^T W), first-order inverse
     OsjDesc<T>* od;
-    T *oscale, *ooff;
-    int *odone, *oon;
+    T *ocols, *ooff;
+    int *oord, *oon;
+    OsjShape oshape;
     T **pW, **pH, **pT;
     int *pv, *ppv;
     GemmDesc<T>* gd;
@@ -268,8 +269,8 @@ size_t carve_engine(Engine<T>& g, Bump& b) {
     g.rank_d = b.take<int>(1);
     g.Wh = b.take<T>((size_t)pp * pp); g.Wg = b.take<T>((size_t)pp * pp); g.Wt = b.take<T>((size_t)pp * pp);
     g.od = b.take<OsjDesc<T>>(1);
-    g.oscale = b.take<T>(1); g.ooff = b.take<T>(3);
-    g.odone = b.take<int>(1); g.oon = b.take<int>(1);
+    g.ocols = b.take<T>(2 * (size_t)pp); g.ooff = b.take<T>(3);
+    g.oord = b.take<int>(pp); g.oon = b.take<int>(1);
     g.pW = b.take<T*>(1); g.pH = b.take<T*>(1); g.pT = b.take<T*>(1);
     g.pv = b.take<int>(1); g.ppv = b.take<int>(1);
     g.gd = b.take<GemmDesc<T>>(64);
@@ -396,8 +397,8 @@ int svt(Engine<T>& g, double mu, T* Uout, T* Vrout, T* Sout) {
     UTRY(g.gemm(false, false, (int)n, r, r, T(1), g.At, n, g.Wj, pp, T(0), g.X, n));
     const int one = 1;
     UTRY(cudaMemcpyAsync(g.oon, &one, sizeof(int), cudaMemcpyHostToDevice, s));
-    lrr::k::col_norm_max<T><<<1, 256, 0, s>>>(g.od, g.oon, g.oscale, 1);
-    UTRY(osj_sweeps<T>(g.od, 1, pp, 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), nullptr, s, 0));
+    UTRY(osj_sweeps<T>(g.od, 1, g.oshape, 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), nullptr, s,
+                       OsjMode::kept));
     const T tau = (T)(1.0 / mu);
     UTRY(cudaMemsetAsync(g.rank_d, 0, sizeof(int), s));
     u::svt_svals<T><<<ceil_div((int64_t)r * 32, 256), 256, 0, s>>>(g.X, n, n, r, tau, g.sv, g.fs, g.invs, g.rank_d);
@@ -564,11 +565,12 @@ template <typename T>
 int engine_init(Engine<T>& g) {
     cudaStream_t s = g.s;
     OsjDesc<T> d{};
-    d.X = g.X; d.W = g.Wj; d.done = g.odone; d.off = g.ooff; d.active = g.oon; d.scale = g.oscale;
+    d.X = g.X; d.W = g.Wj; d.off = g.ooff; d.cols = g.ocols; d.ord = g.oord; d.active = g.oon;
     // no threshold in the measure (d.mu null): the reverse pass needs every
     // singular pair resolved, including the ones the SVT removes
     d.mu = nullptr;
     d.ldx = g.n; d.ldw = g.pp; d.L = (int)g.n; d.p = g.r; d.pp = g.pp; d.strict = 1;
+    g.oshape = osj_shape<T>(1, g.r, (int)g.n);
     UTRY(cudaMemcpyAsync(g.od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     T* ptrs[3] = {g.Wj, g.Wg, g.Wt};
     UTRY(cudaMemcpyAsync(g.pW, &ptrs[0], sizeof(T*), cudaMemcpyHostToDevice, s));
