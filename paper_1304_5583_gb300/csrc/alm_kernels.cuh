@@ -104,7 +104,7 @@ __global__ void init_padded(T* __restrict__ G, int p, int pp, T diag, int eye) {
 // <= tau, so the threshold removes all of them and J = 0 with no SVD.
 // The Z-step kernel of the same iteration then accumulates the next value.
 static __global__ void svt_gate(const int* __restrict__ act, double* __restrict__ afro, const double* __restrict__ mu,
-                         int* __restrict__ svt_on, int* __restrict__ calls,
+                         int* __restrict__ svt_on, int* __restrict__ calls, int* __restrict__ rank,
                          int* __restrict__ fp32_on, int* __restrict__ gemm32, double margin, int nblk) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nblk) return;
@@ -116,14 +116,20 @@ static __global__ void svt_gate(const int* __restrict__ act, double* __restrict_
     // rounding of the products is forgotten by the iteration
     if (afro[b] > margin * margin * tau * tau) fp32_on[b] = 1;
     gemm32[b] = (act[b] && fp32_on[b]) ? 1 : 0;
-    if (act[b]) afro[b] = 0.0;
+    if (act[b]) {
+        afro[b] = 0.0;
+        rank[b] = 0;
+    }
 }
 
 // After the one-sided Jacobi the columns x_j of X are orthogonal and
 // ||x_j||^2 are the eigenvalues lambda_j of the Gram; the singular values of A
 // are sqrt(lambda_j).  h_j = max(1 - tau/||x_j||, 0), so that
 // J = X diag(h) W^T (tall) or W diag(h) X^T (wide) = U max(Sigma - tau, 0) V^T.
-// Also counts the SVT rank.  One CTA per block.
+// Also counts the SVT rank (rank[b] is zero on entry).  kWeightCols columns per
+// CTA, a warp each in turn: with one CTA per block the 487 columns of a
+// 1000 x 487 SVT took 90 us.
+constexpr int kWeightCols = 32;
 template <typename T>
 __global__ void svt_weights(const OsjDesc<T>* __restrict__ descs, T* const* __restrict__ h,
                             const int* __restrict__ act, const int* __restrict__ svt_on,
@@ -136,13 +142,14 @@ __global__ void svt_weights(const OsjDesc<T>* __restrict__ descs, T* const* __re
     const T tau_t = (T)tau;
     const int on = svt_on[b];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int j1 = min(d.pp, (int)(blockIdx.y + 1) * kWeightCols);
     int cnt = 0;
-    for (int j = warp; j < d.pp; j += nw) {
+    for (int j = blockIdx.y * kWeightCols + warp; j < j1; j += nw) {
         T w = T(0);
         if (on && j < d.p) {
             const T* x = d.X + (int64_t)j * d.ldx;
             T acc = T(0);
-            for (int i = lane; i < d.L; i += 32) acc += x[i] * x[i];
+            for (int i = lane; i < d.L; i += 32) acc = fma(x[i], x[i], acc);
             const T nrm = sqrt(warp_sum(acc));
             if (nrm > tau_t) w = T(1) - tau_t / nrm;
         }
@@ -151,14 +158,7 @@ __global__ void svt_weights(const OsjDesc<T>* __restrict__ descs, T* const* __re
             if (w > T(0)) ++cnt;
         }
     }
-    __shared__ int s_c[32];
-    if (lane == 0) s_c[warp] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int a2 = 0;
-        for (int w2 = 0; w2 < nw; ++w2) a2 += s_c[w2];
-        rank[b] = a2;
-    }
+    if (lane == 0 && cnt) atomicAdd(&rank[b], cnt);
 }
 
 // Z-step in reduced coordinates, fused with the Y2 dual step and the next

@@ -6,6 +6,11 @@
 
 namespace lrr {
 
+// --------------------------------------------------------------------- scratch
+// Stream-ordered allocation from the library's pool (scratch.cu); freed with
+// cudaFreeAsync.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+
 // ---------------------------------------------------------------- grouped GEMM
 // C_g = alpha * op(A_g) * op(B_g) + beta * C_g for every group g whose flag is
 // nonzero (flag == nullptr: always).  Column-major, op = transpose if trans*.

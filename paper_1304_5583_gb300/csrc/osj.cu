@@ -42,6 +42,9 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1010,15 +1013,32 @@ cudaError_t launch(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweep
     return cudaGetLastError();
 }
 
+// clusters of this shape that fit the current device at once; the runtime's
+// answer (some 10 us a query, and a shape is chosen by a dozen) is kept per
+// device, cluster size, thread count and shared memory
 template <typename T>
-int resident_clusters(OsjShape sh) {
+int resident_clusters(const OsjShape& sh) {
+    const size_t smem = smem_bytes<T>(sh);
+    if (smem > SMEM_MAX) return 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    static std::mutex mu;
+    static std::map<std::tuple<int, int, int, size_t>, int> known;
+    const auto key = std::make_tuple(dev, sh.cluster, sh.wide, smem);
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        const auto it = known.find(key);
+        if (it != known.end()) return it->second;
+    }
     int n = 0;
-    if (smem_bytes<T>(sh) > SMEM_MAX) return 0;
     // (both schedules use the same shared memory and register limits)
     const cudaError_t e = sh.wide ? launch<T, NT_FEW, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, &n)
                                   : launch<T, NT_MANY, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, &n);
     if (e != cudaSuccess) n = 0;
     (void)cudaGetLastError();
+    std::lock_guard<std::mutex> lock(mu);
+    if (known.size() > 4096) known.clear();
+    known[key] = n;
     return n;
 }
 

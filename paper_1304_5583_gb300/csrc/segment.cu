@@ -316,7 +316,7 @@ int lrr_segment(const float* F, int64_t ldf, const float* G, int64_t ldg, int64_
     const size_t need = seg_layout(b, nullptr, n, kk, K, restarts);
     void* own = nullptr;
     if (!workspace) {
-        if (cudaMallocAsync(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
+        if (scratch_alloc(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
         workspace = own;
         workspace_bytes = need;
     }

@@ -404,7 +404,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     const size_t need = probe.off + kAlign;
     void* own = nullptr;
     if (!ws) {
-        if (cudaMallocAsync(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
+        if (scratch_alloc(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
         ws = own;
         ws_bytes = need;
     }
@@ -807,7 +807,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         prof.iterations += 1;
         // J-step: SVT of A = Zt + Y2t/mu through the Gram eigendecomposition
         prof.begin();
-        k::svt_gate<<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.afro, B.mu, B.svt_on, B.svtcalls,
+        k::svt_gate<<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.afro, B.mu, B.svt_on, B.svtcalls, B.rank_cur,
                                                          B.fp32_on, B.gemm32, switch_margin, t);
         LRR_CUDA_TRY(run_set(S_XT));
         LRR_CUDA_TRY(run_set(S_XW));
@@ -816,7 +816,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         LRR_CUDA_TRY(osj_sweeps<T>(B.jd, t, jshape, sweeps, jtol, B.jsweeps, s, OsjMode::kept, quad_exit));
         prof.end(LRR_PH_JACOBI, 1);
         prof.begin();
-        k::svt_weights<T><<<t, 256, 0, s>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
+        k::svt_weights<T><<<dim3((unsigned)t, ceil_div(max_pp, k::kWeightCols)), 256, 0, s>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
         // W^T W and W (W^T W): first-order inverse for J, Newton-Schulz for the warm start
         LRR_CUDA_TRY(run_set(S_O1));
         LRR_CUDA_TRY(run_set(S_O2));
@@ -1089,100 +1089,115 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
 }
 
 
-// Stand-alone singular-value thresholding with the solver's own SVT kernels
-// (cold start W = I).  Scratch is taken with cudaMallocAsync on the stream.
+// Scratch of one stand-alone SVT and, after it, the small values its kernels
+// read and write, filled by one kernel from its arguments.
 template <typename T>
-int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* J, int64_t ldj, int32_t* rank_out,
-             cudaStream_t s) {
-    constexpr int B2 = osj_pivot_width();
+struct SvtParams {
+    double mu;
+    T *W, *H, *h, *T1;            // pointer tables of one entry each
+    int act, on, rank, sweeps, p, pp;
+    T off[3];
+    OsjDesc<T> od;
+    GemmDesc<T> g[3];
+};
+
+template <typename T>
+struct SvtScratch {
+    T *X, *W, *H, *T1, *h;
+    SvtParams<T>* par;
+    SvtScratch(Arena& a, int L, int p, int pp) {
+        X = a.take<T>((size_t)L * p);
+        W = a.take<T>((size_t)pp * pp);
+        H = a.take<T>((size_t)pp * pp);
+        T1 = a.take<T>((size_t)pp * pp);
+        h = a.take<T>(pp);
+        par = a.take<SvtParams<T>>(1);
+    }
+};
+
+// X = A (tall) or A^T (wide, through shared memory, 32 x 32 at a time), W = I,
+// and the parameter block; one thread block per 32 x 32 tile of X.
+template <typename T>
+__global__ void svt_begin(const T* __restrict__ A, int64_t lda, int L, int p, int pp, int tall, T* __restrict__ X,
+                          T* __restrict__ W, const SvtParams<T> par, SvtParams<T>* __restrict__ dst) {
+    __shared__ T tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t tiles_r = (L + 31) / 32, ntile = tiles_r * ((p + 31) / 32);
+    for (int64_t b = blockIdx.x; b < ntile; b += gridDim.x) {
+        const int r0 = (int)(b % tiles_r) * 32, c0 = (int)(b / tiles_r) * 32;
+        if (tall) {
+            for (int k = ty; k < 32; k += 8)
+                if (r0 + tx < L && c0 + k < p) X[r0 + tx + (int64_t)(c0 + k) * L] = A[r0 + tx + (int64_t)(c0 + k) * lda];
+        } else {
+            for (int k = ty; k < 32; k += 8)
+                if (c0 + tx < p && r0 + k < L) tile[k][tx] = A[c0 + tx + (int64_t)(r0 + k) * lda];
+            __syncthreads();
+            for (int k = ty; k < 32; k += 8)
+                if (r0 + tx < L && c0 + k < p) X[r0 + tx + (int64_t)(c0 + k) * L] = tile[tx][k];
+            __syncthreads();
+        }
+    }
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)pp * pp; e += (int64_t)gridDim.x * blockDim.x)
+        W[e] = e % pp == e / pp ? T(1) : T(0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *dst = par;
+}
+
+// Stand-alone singular-value thresholding with the solver's own SVT kernels
+// (cold start W = I) in the given scratch.
+template <typename T>
+int svt_run(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* J, int64_t ldj, int32_t* rank_out,
+            cudaStream_t s, const SvtScratch<T>& q) {
     const bool tall = cols <= rows;
-    const int p = (int)std::min(rows, cols);
-    const int L = (int)(tall ? rows : cols);
-    const int pp = round_up(p, B2);
-    Arena sz(nullptr);
-    auto lay = [&](Arena& a, T** X, T** W, T** H, T** T1, T** h, int** ints, double** dbl, OsjDesc<T>** od,
-                   GemmDesc<T>** gd, T** Wp, T** Hp, T** hp, T** off, T** T1p) {
-        *X = a.take<T>((size_t)L * p);
-        *W = a.take<T>((size_t)pp * pp);
-        *H = a.take<T>((size_t)pp * pp);
-        *T1 = a.take<T>((size_t)pp * pp);
-        *h = a.take<T>(pp);
-        *ints = a.take<int>(16);
-        *dbl = a.take<double>(4);
-        *od = a.take<OsjDesc<T>>(1);
-        *gd = a.take<GemmDesc<T>>(8);
-        *Wp = reinterpret_cast<T*>(a.take<T*>(1));
-        *Hp = reinterpret_cast<T*>(a.take<T*>(1));
-        *hp = reinterpret_cast<T*>(a.take<T*>(1));
-        *off = a.take<T>(3);
-        *T1p = reinterpret_cast<T*>(a.take<T*>(1));
-    };
-    T *X, *W, *H, *T1, *h, *Wp, *Hp, *hp, *off, *T1p;
-    int* ints;
-    double* dbl;
-    OsjDesc<T>* od;
-    GemmDesc<T>* gd;
-    lay(sz, &X, &W, &H, &T1, &h, &ints, &dbl, &od, &gd, &Wp, &Hp, &hp, &off, &T1p);
-    void* mem = nullptr;
-    if (cudaMallocAsync(&mem, sz.off + kAlign, s) != cudaSuccess) return LRR_ERR_CUDA;
-    struct Free {
-        void* p; cudaStream_t s;
-        ~Free() { if (p) cudaFreeAsync(p, s); }
-    } guard{mem, s};
-    Arena a(mem);
-    lay(a, &X, &W, &H, &T1, &h, &ints, &dbl, &od, &gd, &Wp, &Hp, &hp, &off, &T1p);
-    int* act = ints;          // [0]
-    int* on = ints + 1;       // [1]
-    int* rk = ints + 2;       // [2]
-    int* swp = ints + 4;      // [4]
-    double* mu = dbl;
-    const int one[2] = {1, 1};
-    const double mud = 1.0 / tau;
-    LRR_CUDA_TRY(cudaMemcpyAsync(act, one, sizeof(int) * 2, cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemsetAsync(swp, 0, sizeof(int), s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(mu, &mud, sizeof(double), cudaMemcpyHostToDevice, s));
-    k::init_padded<T><<<grid1((int64_t)pp * pp), 256, 0, s>>>(W, p, pp, T(1), 1);
-    T* ptrs[4] = {W, H, h, T1};
-    LRR_CUDA_TRY(cudaMemcpyAsync(T1p, &ptrs[3], sizeof(T*), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(Wp, &ptrs[0], sizeof(T*), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(Hp, &ptrs[1], sizeof(T*), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(hp, &ptrs[2], sizeof(T*), cudaMemcpyHostToDevice, s));
-    const int pvals[2] = {p, pp};
-    int* pv = ints + 8;
-    int* ppv = ints + 9;
-    LRR_CUDA_TRY(cudaMemcpyAsync(pv, &pvals[0], sizeof(int), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(ppv, &pvals[1], sizeof(int), cudaMemcpyHostToDevice, s));
-    OsjDesc<T> d{};
-    d.X = X; d.W = W; d.off = off; d.active = on; d.mu = mu;
-    d.cols = T1;                          // T1 and H are written only after the Jacobi: its scratch until then
-    d.ord = reinterpret_cast<int*>(H);
-    d.ldx = L; d.ldw = pp; d.L = L; d.p = p; d.pp = pp; d.strict = 1;
-    LRR_CUDA_TRY(cudaMemcpyAsync(od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
-    GemmDesc<T> g[5];
-    if (tall) g[0] = gdesc<T>(A, lda, W, pp, X, L, L, p, p, nullptr);          // X = A W
-    else g[0] = gdesc<T>(A, lda, W, pp, X, L, L, p, p, nullptr);               // X = A^T W
-    g[1] = gdesc<T>(W, pp, W, pp, T1, pp, p, p, p, nullptr);                   // W^T W
-    g[2] = gdesc<T>(W, pp, T1, pp, H, pp, p, p, p, nullptr);                   // W (W^T W)
-    if (tall) g[3] = gdesc<T>(X, L, T1, pp, J, ldj, (int)rows, (int)cols, p, nullptr);   // J = X h W^{-1}
-    else g[3] = gdesc<T>(T1, pp, X, L, J, ldj, (int)rows, (int)cols, p, nullptr);        // J = W^{-T} h X^T
-    g[3].kscale = h;
-    LRR_CUDA_TRY(cudaMemcpyAsync(gd, g, sizeof(g), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(gemm_grouped<T>(gd, 1, !tall, false, L, p, s));
-    LRR_CUDA_TRY(osj_sweeps<T>(od, 1, osj_shape<T>(1, p, L), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), swp, s,
+    const int p = (int)std::min(rows, cols), L = (int)std::max(rows, cols), pp = round_up(p, osj_pivot_width());
+    SvtParams<T> par{};
+    SvtParams<T>* const d = q.par;
+    par.mu = 1.0 / tau;
+    par.W = q.W; par.H = q.H; par.h = q.h; par.T1 = q.T1;
+    par.act = par.on = 1;
+    par.p = p; par.pp = pp;
+    par.od.X = q.X; par.od.W = q.W; par.od.off = d->off; par.od.active = &d->on; par.od.mu = &d->mu;
+    par.od.cols = q.T1;                   // T1 and H are written only after the Jacobi: its scratch until then
+    par.od.ord = reinterpret_cast<int*>(q.H);
+    par.od.ldx = L; par.od.ldw = pp; par.od.L = L; par.od.p = p; par.od.pp = pp; par.od.strict = 1;
+    par.g[0] = gdesc<T>(q.W, pp, q.W, pp, q.T1, pp, p, p, p, nullptr);                   // W^T W
+    par.g[1] = gdesc<T>(q.W, pp, q.T1, pp, q.H, pp, p, p, p, nullptr);                   // W (W^T W)
+    if (tall) par.g[2] = gdesc<T>(q.X, L, q.T1, pp, J, ldj, (int)rows, (int)cols, p, nullptr);   // J = X h W^{-1}
+    else par.g[2] = gdesc<T>(q.T1, pp, q.X, L, J, ldj, (int)rows, (int)cols, p, nullptr);        // J = W^{-T} h X^T
+    par.g[2].kscale = q.h;
+    const int64_t tiles = (int64_t)((L + 31) / 32) * ((p + 31) / 32);
+    svt_begin<T><<<(unsigned)std::min<int64_t>(tiles, 152 * 8), 256, 0, s>>>(A, lda, L, p, pp, tall ? 1 : 0, q.X, q.W, par, d);
+    LRR_CUDA_TRY(cudaGetLastError());
+    LRR_CUDA_TRY(osj_sweeps<T>(&d->od, 1, osj_shape<T>(1, p, L), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), &d->sweeps, s,
                                OsjMode::sorted));
-    k::svt_weights<T><<<1, 256, 0, s>>>(od, reinterpret_cast<T* const*>(hp), act, on, mu, rk, 1);
-    LRR_CUDA_TRY(gemm_grouped<T>(gd + 1, 1, true, false, p, p, s));
-    LRR_CUDA_TRY(gemm_grouped<T>(gd + 2, 1, false, false, p, p, s));
-    k::ns_orth<T><<<dim3(64, 1), 256, 0, s>>>(reinterpret_cast<T* const*>(Wp), reinterpret_cast<T* const*>(Hp),
-                                              reinterpret_cast<T* const*>(T1p), pv, ppv, on, 1);
-    LRR_CUDA_TRY(gemm_grouped<T>(gd + 3, 1, false, true, (int)rows, (int)cols, s));
+    k::svt_weights<T><<<dim3(1, (unsigned)ceil_div(pp, k::kWeightCols)), 256, 0, s>>>(&d->od, &d->h, &d->act, &d->on,
+                                                                                     &d->mu, &d->rank, 1);
+    LRR_CUDA_TRY(gemm_grouped<T>(&d->g[0], 1, true, false, p, p, s));
+    LRR_CUDA_TRY(gemm_grouped<T>(&d->g[1], 1, false, false, p, p, s));
+    k::ns_orth<T><<<dim3(64, 1), 256, 0, s>>>(&d->W, &d->H, &d->T1, &d->p, &d->pp, &d->on, 1);
+    LRR_CUDA_TRY(gemm_grouped<T>(&d->g[2], 1, false, true, (int)rows, (int)cols, s));
     int rk_h = 0;
-    LRR_CUDA_TRY(cudaMemcpyAsync(&rk_h, rk, sizeof(int), cudaMemcpyDeviceToHost, s));
+    LRR_CUDA_TRY(cudaMemcpyAsync(&rk_h, &d->rank, sizeof(int), cudaMemcpyDeviceToHost, s));
     LRR_CUDA_TRY(cudaStreamSynchronize(s));
     if (rank_out) *rank_out = rk_h;
     return LRR_OK;
 }
 
+// with its scratch allocated on the stream
+template <typename T>
+int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* J, int64_t ldj, int32_t* rank_out,
+             cudaStream_t s) {
+    const int p = (int)std::min(rows, cols), L = (int)std::max(rows, cols), pp = round_up(p, osj_pivot_width());
+    Arena sz(nullptr);
+    SvtScratch<T>(sz, L, p, pp);
+    void* mem = nullptr;
+    if (scratch_alloc(&mem, sz.off + kAlign, s) != cudaSuccess) return LRR_ERR_CUDA;
+    struct Free {
+        void* p; cudaStream_t s;
+        ~Free() { if (p) cudaFreeAsync(p, s); }
+    } guard{mem, s};
+    Arena a(mem);
+    return svt_run<T>(A, rows, cols, lda, tau, J, ldj, rank_out, s, SvtScratch<T>(a, L, p, pp));
+}
 
 // ---------------------------------------------------------------------------
 // lrr_svt_noalloc: the stand-alone SVT with all of its scratch in one
@@ -1217,91 +1232,14 @@ void* svt_scratch_address() {
 template <typename T>
 int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* J, int64_t ldj,
                      int32_t* rank_out, cudaStream_t s) {
-    constexpr int B2 = osj_pivot_width();
-    const bool tall = cols <= rows;
-    const int p = (int)std::min(rows, cols);
-    const int L = (int)(tall ? rows : cols);
-    const int pp = round_up(p, B2);
-    struct Parts {
-        T *X, *W, *H, *T1, *h, *off;
-        T **Wp, **Hp, **hp, **T1p;
-        int* ints;
-        double* dbl;
-        OsjDesc<T>* od;
-        GemmDesc<T>* gd;
-    };
-    auto lay = [&](Arena& a) {
-        Parts q;
-        q.X = a.take<T>((size_t)L * p);
-        q.W = a.take<T>((size_t)pp * pp);
-        q.H = a.take<T>((size_t)pp * pp);
-        q.T1 = a.take<T>((size_t)pp * pp);
-        q.h = a.take<T>(pp);
-        q.ints = a.take<int>(16);
-        q.dbl = a.take<double>(4);
-        q.od = a.take<OsjDesc<T>>(1);
-        q.gd = a.take<GemmDesc<T>>(8);
-        q.Wp = a.take<T*>(1);
-        q.Hp = a.take<T*>(1);
-        q.hp = a.take<T*>(1);
-        q.T1p = a.take<T*>(1);
-        q.off = a.take<T>(3);
-        return q;
-    };
+    const int p = (int)std::min(rows, cols), L = (int)std::max(rows, cols), pp = round_up(p, osj_pivot_width());
     Arena sz(nullptr);
-    lay(sz);
+    SvtScratch<T>(sz, L, p, pp);
     if (sz.off > kNoAllocScratchBytes) return LRR_ERR_TOO_LARGE;
     void* base = svt_scratch_address();
     if (!base) return LRR_ERR_CUDA;
     Arena a(base);
-    const Parts q = lay(a);
-    int* act = q.ints;
-    int* on = q.ints + 1;
-    int* rk = q.ints + 2;
-    int* swp = q.ints + 4;
-    int* pv = q.ints + 8;
-    int* ppv = q.ints + 9;
-    double* mu = q.dbl;
-    const int one[2] = {1, 1};
-    const double mud = 1.0 / tau;
-    const int pvals[2] = {p, pp};
-    T* ptrs[4] = {q.W, q.H, q.h, q.T1};
-    LRR_CUDA_TRY(cudaMemcpyAsync(act, one, sizeof(int) * 2, cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemsetAsync(swp, 0, sizeof(int), s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(mu, &mud, sizeof(double), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(pv, pvals, sizeof(int) * 2, cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(q.Wp, &ptrs[0], sizeof(T*), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(q.Hp, &ptrs[1], sizeof(T*), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(q.hp, &ptrs[2], sizeof(T*), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(cudaMemcpyAsync(q.T1p, &ptrs[3], sizeof(T*), cudaMemcpyHostToDevice, s));
-    k::init_padded<T><<<grid1((int64_t)pp * pp), 256, 0, s>>>(q.W, p, pp, T(1), 1);
-    OsjDesc<T> d{};
-    d.X = q.X; d.W = q.W; d.off = q.off; d.active = on; d.mu = mu;
-    d.cols = q.T1;                        // T1 and H are written only after the Jacobi: its scratch until then
-    d.ord = reinterpret_cast<int*>(q.H);
-    d.ldx = L; d.ldw = pp; d.L = L; d.p = p; d.pp = pp; d.strict = 1;
-    LRR_CUDA_TRY(cudaMemcpyAsync(q.od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
-    GemmDesc<T> g[4];
-    g[0] = gdesc<T>(A, lda, q.W, pp, q.X, L, L, p, p, nullptr);                         // X = A W or A^T W
-    g[1] = gdesc<T>(q.W, pp, q.W, pp, q.T1, pp, p, p, p, nullptr);                      // W^T W
-    g[2] = gdesc<T>(q.W, pp, q.T1, pp, q.H, pp, p, p, p, nullptr);                      // W (W^T W)
-    if (tall) g[3] = gdesc<T>(q.X, L, q.T1, pp, J, ldj, (int)rows, (int)cols, p, nullptr);
-    else g[3] = gdesc<T>(q.T1, pp, q.X, L, J, ldj, (int)rows, (int)cols, p, nullptr);
-    g[3].kscale = q.h;
-    LRR_CUDA_TRY(cudaMemcpyAsync(q.gd, g, sizeof(g), cudaMemcpyHostToDevice, s));
-    LRR_CUDA_TRY(gemm_grouped<T>(q.gd, 1, !tall, false, L, p, s));
-    LRR_CUDA_TRY(osj_sweeps<T>(q.od, 1, osj_shape<T>(1, p, L), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), swp, s,
-                               OsjMode::sorted));
-    k::svt_weights<T><<<1, 256, 0, s>>>(q.od, q.hp, act, on, mu, rk, 1);
-    LRR_CUDA_TRY(gemm_grouped<T>(q.gd + 1, 1, true, false, p, p, s));
-    LRR_CUDA_TRY(gemm_grouped<T>(q.gd + 2, 1, false, false, p, p, s));
-    k::ns_orth<T><<<dim3(64, 1), 256, 0, s>>>(q.Wp, q.Hp, q.T1p, pv, ppv, on, 1);
-    LRR_CUDA_TRY(gemm_grouped<T>(q.gd + 3, 1, false, true, (int)rows, (int)cols, s));
-    int rk_h = 0;
-    LRR_CUDA_TRY(cudaMemcpyAsync(&rk_h, rk, sizeof(int), cudaMemcpyDeviceToHost, s));
-    LRR_CUDA_TRY(cudaStreamSynchronize(s));
-    if (rank_out) *rank_out = rk_h;
-    return LRR_OK;
+    return svt_run<T>(A, rows, cols, lda, tau, J, ldj, rank_out, s, SvtScratch<T>(a, L, p, pp));
 }
 
 template <typename T, typename Tin>
@@ -1391,7 +1329,7 @@ int local_impl(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_res
                          (sizeof(OsjDesc<T>) + sizeof(GemmDesc<T>) * 2 + 64 * sizeof(T) + 64) * (size_t)t + 4096 * 4 +
                          (2 * sizeof(T) + sizeof(int)) * (size_t)kpad + 512;
     void* mem = nullptr;
-    if (cudaMallocAsync(&mem, bytes, s) != cudaSuccess) return LRR_ERR_CUDA;
+    if (scratch_alloc(&mem, bytes, s) != cudaSuccess) return LRR_ERR_CUDA;
     struct Free {
         void* p; cudaStream_t s;
         ~Free() { if (p) cudaFreeAsync(p, s); }
@@ -1588,7 +1526,7 @@ int lrr_gemm_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, float*
     if (M > (1 << 30) || N > lrr::kTcMaxN || K > (1 << 30)) return LRR_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int* err = nullptr;
-    if (cudaMallocAsync(&err, sizeof(int), s) != cudaSuccess) return LRR_ERR_CUDA;
+    if (lrr::scratch_alloc(reinterpret_cast<void**>(&err), sizeof(int), s) != cudaSuccess) return LRR_ERR_CUDA;
     int rc = LRR_OK;
     if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess ||
         lrr::tc_gemm_bf16(A, lda, B, ldb, C, ldc, (int)M, (int)N, (int)K, err, s) != cudaSuccess)
@@ -1609,7 +1547,7 @@ int lrr_gemm_f32(const float* A, int64_t lda, const float* B, int64_t ldb, float
     const int64_t k4 = (K + 3) / 4 * 4;
     const size_t words = (size_t)k4 * (size_t)(M + N) * 2;
     void* mem = nullptr;
-    if (cudaMallocAsync(&mem, words * sizeof(float) + 256, s) != cudaSuccess) return LRR_ERR_CUDA;
+    if (lrr::scratch_alloc(&mem, words * sizeof(float) + 256, s) != cudaSuccess) return LRR_ERR_CUDA;
     float* ah = static_cast<float*>(mem);
     float* al = ah + (size_t)k4 * M;
     float* bh = al + (size_t)k4 * M;
@@ -1644,7 +1582,7 @@ int lrr_gemm_timing(int32_t kind, int64_t M, int64_t N, int64_t K, int32_t repea
     const size_t abytes = ((size_t)kp * M * esz + 255) / 256 * 256, bbytes = ((size_t)kp * N * esz + 255) / 256 * 256;
     const size_t total = nops * (abytes + bbytes) + sizeof(float) * (size_t)M * N + 256;
     void* mem = nullptr;
-    if (cudaMallocAsync(&mem, total, s) != cudaSuccess) return LRR_ERR_CUDA;
+    if (lrr::scratch_alloc(&mem, total, s) != cudaSuccess) return LRR_ERR_CUDA;
     char* p = static_cast<char*>(mem);
     void* A0 = p; p += abytes;
     void* A1 = p; p += nops > 1 ? abytes : 0;

@@ -632,7 +632,7 @@ int unrolled_run(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unr
     const size_t need = carve_engine<T>(g, probe);
     void* own = nullptr;
     if (!ws) {
-        if (cudaMallocAsync(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
+        if (scratch_alloc(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
         ws = own;
         wsb = need;
     }
