@@ -104,12 +104,17 @@ __global__ void init_padded(T* __restrict__ G, int p, int pp, T diag, int eye) {
 // <= tau, so the threshold removes all of them and J = 0 with no SVD.
 // The Z-step kernel of the same iteration then accumulates the next value.
 static __global__ void svt_gate(const int* __restrict__ act, double* __restrict__ afro, const double* __restrict__ mu,
-                         int* __restrict__ svt_on, int* __restrict__ calls, int* __restrict__ rank,
+                         int* __restrict__ svt_on, int* __restrict__ j_on, int* __restrict__ calls,
+                         int* __restrict__ rank,
                          int* __restrict__ fp32_on, int* __restrict__ gemm32, double margin, int nblk) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nblk) return;
     const double tau = 1.0 / mu[b];
+    // J is formed while the block's SVT acts, and once more (as zero) after it
+    // stops acting; before its first SVT it is zero already
+    const int was_on = svt_on[b];
     svt_on[b] = (act[b] && afro[b] > tau * tau) ? 1 : 0;
+    j_on[b] = act[b] && (svt_on[b] || was_on);
     if (svt_on[b]) calls[b] += 1;
     // mixed precision: float32 products from the first iteration in which
     // ||A||_F exceeds margin * tau (sticky); before that J = 0 and the bf16

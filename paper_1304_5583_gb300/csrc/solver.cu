@@ -22,6 +22,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <set>
 #include <tuple>
 #include <vector>
 
@@ -105,7 +106,7 @@ struct Buffers {
     std::vector<int*> rot;
     int* rot_d;
     double *mu, *mu_fin, *resid;
-    int *act, *iters, *svt_on, *rank_cur, *rank_fin, *need_exact, *conv_bound, *conv, *jord, *colblk, *flag;
+    int *act, *iters, *svt_on, *rank_cur, *rank_fin, *need_exact, *conv_bound, *conv, *jord, *j_on, *colblk, *flag;
     T *r1, *dmax, *r2x, *jcols, *joff;
     int64_t* perm;
     // descriptor / pointer tables
@@ -223,6 +224,7 @@ Buffers<T> carve(Arena& a, const lrr_problem* p, bool need_md, const std::vector
     size_t cols_pad = 0;      // every block's columns, each padded to the pivot width
     for (int i = 0; i < t; ++i) cols_pad += (size_t)blk[i].ppmax;
     b.jord = a.take<int>(cols_pad);
+    b.j_on = a.take<int>(t);
     b.colblk = a.take<int>(n);
     b.flag = a.take<int>(4);
     b.r1 = a.take<T>(t);
@@ -363,6 +365,52 @@ template <typename T>
 struct GemmSet {
     int first = 0, count = 0, max_m = 0, max_n = 0;
     bool ta = false, tb = false;
+};
+
+// Graphs of iteration chunks, recorded on a stream of their own; they and the
+// stream end with the solve.
+struct ChunkGraphs {
+    using Key = std::tuple<int, bool, bool, int, int, int>;
+    struct Entry {
+        cudaGraphExec_t exec = nullptr;
+        int64_t launches = 0, calls[LRR_NPHASE] = {};
+    };
+    std::map<Key, Entry> known;
+    std::set<Key> seen;
+    cudaStream_t stream = nullptr;
+    bool off = false;          // recording failed once: launch directly from then on
+
+    Entry* find(const Key& k) {
+        const auto it = known.find(k);
+        return it == known.end() ? nullptr : &it->second;
+    }
+    bool again(const Key& k) { return !seen.insert(k).second; }
+    bool begin() {
+        if (off) return false;
+        off = (!stream && cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) != cudaSuccess) ||
+              cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess;
+        if (off) (void)cudaGetLastError();
+        return !off;
+    }
+    Entry* end(const Key& k, bool good) {
+        cudaGraph_t g = nullptr;
+        Entry e;
+        const bool ok = cudaStreamEndCapture(stream, &g) == cudaSuccess && good && g &&
+                        cudaGraphInstantiate(&e.exec, g, 0) == cudaSuccess;
+        if (g) cudaGraphDestroy(g);
+        if (!ok) {
+            (void)cudaGetLastError();
+            off = true;
+            return nullptr;
+        }
+        return &known.emplace(k, e).first->second;
+    }
+    ChunkGraphs() = default;
+    ChunkGraphs(const ChunkGraphs&) = delete;
+    ~ChunkGraphs() {
+        for (auto& k : known) cudaGraphExecDestroy(k.second.exec);
+        if (stream) cudaStreamDestroy(stream);
+    }
 };
 
 // ---- autotuner: launch shape of the batched Jacobi (cluster size per block),
@@ -710,13 +758,13 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         if (tall[i]) {
             xw_tall.push_back(gdesc<T>(Ai, r, B.W[i], pp_, Xi, r, r, l, l, B.svt_on + i));
             // J = X diag(h) W^{-1}:  A = X W^{-1}, so this keeps the kept directions only
-            GemmDesc<T> jd_ = gdesc<T>(Xi, r, B.T1[i], pp_, B.Jt + c0 * r, r, r, l, l, B.act + i);
+            GemmDesc<T> jd_ = gdesc<T>(Xi, r, B.T1[i], pp_, B.Jt + c0 * r, r, r, l, l, B.j_on + i);
             jd_.kscale = B.h[i];
             jmul.push_back(jd_);
         } else {
             xw_wide.push_back(gdesc<T>(Ai, r, B.W[i], pp_, Xi, l, l, r, r, B.svt_on + i));
             // J = W^{-T} diag(h) X^T:  A^T = X W^{-1}
-            GemmDesc<T> jd_ = gdesc<T>(B.T1[i], pp_, Xi, l, B.Jt + c0 * r, r, r, l, r, B.act + i);
+            GemmDesc<T> jd_ = gdesc<T>(B.T1[i], pp_, Xi, l, B.Jt + c0 * r, r, r, l, r, B.j_on + i);
             jd_.kscale = B.h[i];
             jmul.push_back(jd_);
         }
@@ -738,10 +786,11 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     const int S_O2 = add_set(false, false, orth2);
     if (gh.size() + 10 > 16 * (size_t)t + 16) return LRR_ERR_INVALID;
     LRR_CUDA_TRY(cudaMemcpyAsync(B.gd, gh.data(), sizeof(GemmDesc<T>) * gh.size(), cudaMemcpyHostToDevice, s));
+    cudaStream_t q = s;        // the iteration's launches go here: the solve's stream, or one that records a graph
     auto run_set = [&](int si) -> cudaError_t {
         if (si < 0) return cudaSuccess;
         const GemmSet<T>& g = sets[si];
-        return gemm_grouped<T>(B.gd + g.first, g.count, g.ta, g.tb, g.max_m, g.max_n, s);
+        return gemm_grouped<T>(B.gd + g.first, g.count, g.ta, g.tb, g.max_m, g.max_n, q);
     };
 
     // ---- state
@@ -807,20 +856,20 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         prof.iterations += 1;
         // J-step: SVT of A = Zt + Y2t/mu through the Gram eigendecomposition
         prof.begin();
-        k::svt_gate<<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.afro, B.mu, B.svt_on, B.svtcalls, B.rank_cur,
+        k::svt_gate<<<ceil_div(t, 128), 128, 0, q>>>(B.act, B.afro, B.mu, B.svt_on, B.j_on, B.svtcalls, B.rank_cur,
                                                          B.fp32_on, B.gemm32, switch_margin, t);
         LRR_CUDA_TRY(run_set(S_XT));
         LRR_CUDA_TRY(run_set(S_XW));
         prof.end(LRR_PH_GRAM, 1 + nl(S_XT) + nl(S_XW));
         prof.begin();
-        LRR_CUDA_TRY(osj_sweeps<T>(B.jd, t, jshape, sweeps, jtol, B.jsweeps, s, OsjMode::kept, quad_exit));
+        LRR_CUDA_TRY(osj_sweeps<T>(B.jd, t, jshape, sweeps, jtol, B.jsweeps, q, OsjMode::kept, quad_exit));
         prof.end(LRR_PH_JACOBI, 1);
         prof.begin();
-        k::svt_weights<T><<<dim3((unsigned)t, ceil_div(max_pp, k::kWeightCols)), 256, 0, s>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
+        k::svt_weights<T><<<dim3((unsigned)t, ceil_div(max_pp, k::kWeightCols)), 256, 0, q>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
         // W^T W and W (W^T W): first-order inverse for J, Newton-Schulz for the warm start
         LRR_CUDA_TRY(run_set(S_O1));
         LRR_CUDA_TRY(run_set(S_O2));
-        k::ns_orth<T><<<dim3(64, (unsigned)t), 256, 0, s>>>(B.Wp, B.Hp, B.T1p, B.pv, B.ppv, B.svt_on, t);
+        k::ns_orth<T><<<dim3(64, (unsigned)t), 256, 0, q>>>(B.Wp, B.Hp, B.T1p, B.pv, B.ppv, B.svt_on, t);
         LRR_CUDA_TRY(run_set(S_J));
         prof.end(LRR_PH_SVT_APPLY, 5);
         // Z-step
@@ -829,19 +878,19 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
             if (bf16_phase) {
                 // all columns at once; blocks already in float32 are recomputed below
                 LRR_CUDA_TRY(tc_gemm_bf16x3(B.Ubf, B.Ubf_lo, B.ldm8, B.Pbf, B.Pbf_lo, B.ldm8, B.Tt, r, r, (int)n,
-                                            (int)m, B.tc_err, s));
+                                            (int)m, B.tc_err, q));
             }
         }
         if (tc32) {
             // float32-accurate U^T P on the tensor cores for the blocks past the bf16 phase
             LRR_CUDA_TRY(tc_gemm_3xtf32(B.Uh, B.Ul, B.m4, B.Ph, B.Pl, B.m4, reinterpret_cast<float*>(B.Tt), r, r,
-                                        (int)n, (int)m, B.colblk, B.gemm32, B.tc_err, s));
+                                        (int)n, (int)m, B.colblk, B.gemm32, B.tc_err, q));
         } else {
             LRR_CUDA_TRY(run_set(S_T));
         }
         prof.end(LRR_PH_ZGEMM, bf16_phase ? 2 : 1);
         prof.begin();
-        k::z_update<T><<<wgrid_n, 256, 0, s>>>(r, n, B.colblk, B.act, B.mu, o->rho, o->mu_max, B.Tt, B.Theta, B.Jt,
+        k::z_update<T><<<wgrid_n, 256, 0, q>>>(r, n, B.colblk, B.act, B.mu, o->rho, o->mu_max, B.Tt, B.Theta, B.Jt,
                                                B.Y2t, B.Zt, B.D, B.A, B.sig, B.dinv, B.dmax, B.afro,
                                                bf16_phase ? B.Zbf : nullptr, B.Zbf_lo, B.ldr8, tc32 ? B.Dh : nullptr,
                                                tc32 ? B.Dl : nullptr, B.r4);
@@ -851,42 +900,82 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         if constexpr (std::is_same<T, float>::value) {
             if (bf16_phase)
                 LRR_CUDA_TRY(tc_gemm_bf16x3(B.USbf, B.USbf_lo, B.ldr8, B.Zbf, B.Zbf_lo, B.ldr8, B.MZ, m, (int)m,
-                                            (int)n, r, B.tc_err, s));
+                                            (int)n, r, B.tc_err, q));
         }
         if (tc32) {
             LRR_CUDA_TRY(tc_gemm_3xtf32(B.UTh, B.UTl, B.r4, B.Dh, B.Dl, B.r4, reinterpret_cast<float*>(B.MZ), m,
-                                        (int)m, (int)n, r, B.colblk, B.gemm32, B.tc_err, s));
+                                        (int)m, (int)n, r, B.colblk, B.gemm32, B.tc_err, q));
         } else {
             LRR_CUDA_TRY(run_set(S_MZ));
         }
         prof.end(LRR_PH_MZGEMM, bf16_phase ? 2 : 1);
         prof.begin();
-        k::e_update<T><<<wgrid_n, 256, 0, s>>>(m, n, B.colblk, B.act, B.mu, o->rho, o->mu_max, o->lambda,
+        k::e_update<T><<<wgrid_n, 256, 0, q>>>(m, n, B.colblk, B.act, B.mu, o->rho, o->mu_max, o->lambda,
                                                has_perp ? B.C : nullptr, B.MZ, B.Y1, B.E, B.P, B.r1,
                                                bf16_phase ? B.Pbf : nullptr, B.Pbf_lo, B.ldm8, tc32 ? B.Ph : nullptr,
                                                tc32 ? B.Pl : nullptr, B.m4);
         prof.end(LRR_PH_EUPDATE, 1);
         prof.begin();
-        k::stop_part1<T><<<ceil_div(t, 128), 128, 0, s>>>(t, B.act, B.r1, B.dmax, nu_h, 1.0 / std::sqrt((double)n), o->eps, B.need_exact,
+        k::stop_part1<T><<<ceil_div(t, 128), 128, 0, q>>>(t, B.act, B.r1, B.dmax, nu_h, 1.0 / std::sqrt((double)n), o->eps, B.need_exact,
                                                           B.conv_bound, B.any_need, B.need_cnt);
         const bool tc_stage = B.bmax && tc_window;
         if (tc_stage) {
             // ||V D||_inf from bf16 operands on the tensor cores first; the float32
             // product below then runs only for blocks that value cannot decide
-            k::d_to_bf16_needed<T><<<dim3(grid1(r), (unsigned)std::min<int64_t>(n, 4096)), 256, 0, s>>>(
+            k::d_to_bf16_needed<T><<<dim3(grid1(r), (unsigned)std::min<int64_t>(n, 4096)), 256, 0, q>>>(
                 B.D, r, r, n, B.colblk, B.need_exact, B.any_need, B.Dbf, B.ldr8);
             LRR_CUDA_TRY(tc_gemm_bf16_absmax(B.Vbf, B.ldr8, B.Dbf, B.ldr8, (int)n, (int)n, r,
-                                             TcAbsmax{B.any_need, B.colblk, B.need_exact, B.bmax}, B.tc_err, s));
-            k::stop_tc_decide<T><<<ceil_div(t, 128), 128, 0, s>>>(t, B.need_exact, B.conv_bound, B.bmax, B.dmax, nu_h,
+                                             TcAbsmax{B.any_need, B.colblk, B.need_exact, B.bmax}, B.tc_err, q));
+            k::stop_tc_decide<T><<<ceil_div(t, 128), 128, 0, q>>>(t, B.need_exact, B.conv_bound, B.bmax, B.dmax, nu_h,
                                                                  o->eps, tc_rel, B.tc_dec, B.r2x);
         }
         LRR_CUDA_TRY(run_set(S_EX));
-        k::stop_part2<T><<<ceil_div(t, 128), 128, 0, s>>>(t, B.act, B.iters, B.mu, o->rho, o->mu_max, o->eps,
+        k::stop_part2<T><<<ceil_div(t, 128), 128, 0, q>>>(t, B.act, B.iters, B.mu, o->rho, o->mu_max, o->eps,
                                                           o->max_iter, B.r1, B.dmax, B.r2x, B.need_exact,
                                                           B.conv_bound, nu_h, B.resid, B.rank_cur, B.rank_fin,
                                                           B.conv, B.mu_fin, B.afro, B.tc_dec, B.bmax, B.any_need);
         prof.end(LRR_PH_STOP, tc_stage ? 6 : 3);
         LRR_CUDA_TRY(cudaGetLastError());
+        return LRR_OK;
+    };
+    // A chunk of iterations as one graph launch: some sixteen kernels an iteration
+    // at 4 us of launch each are what a small solve takes (60 x 240: 110 of 150 us an
+    // iteration).  Recorded on a stream of its own (the legacy stream cannot be),
+    // when a set of the values that the launches depend on comes up again; with
+    // per-phase events the launches are issued one by one.
+    ChunkGraphs graphs;
+    auto run_chunk = [&](int len) -> int {
+        const auto key = std::make_tuple(len, bf16_phase, tc_window, jshape.cluster, jshape.split, jshape.wide);
+        ChunkGraphs::Entry* e = prof.on ? nullptr : graphs.find(key);
+        // (the second time a set comes up: every kernel is loaded by then)
+        if (!prof.on && !e && graphs.again(key) && graphs.begin()) {
+            const int64_t launches0 = prof.launches, iterations0 = prof.iterations;
+            int64_t calls0[LRR_NPHASE];
+            std::copy(prof.calls, prof.calls + LRR_NPHASE, calls0);
+            q = graphs.stream;
+            int rc = LRR_OK;
+            for (int c = 0; c < len && rc == LRR_OK; ++c) rc = iteration();
+            q = s;
+            e = graphs.end(key, rc == LRR_OK);
+            if (e) {
+                e->launches = prof.launches - launches0;
+                for (int i = 0; i < LRR_NPHASE; ++i) e->calls[i] = prof.calls[i] - calls0[i];
+            }
+            prof.launches = launches0;
+            prof.iterations = iterations0;
+            std::copy(calls0, calls0 + LRR_NPHASE, prof.calls);
+        }
+        if (e) {
+            LRR_CUDA_TRY(cudaGraphLaunch(e->exec, s));
+            prof.launches += e->launches;
+            prof.iterations += len;
+            for (int i = 0; i < LRR_NPHASE; ++i) prof.calls[i] += e->calls[i];
+            return LRR_OK;
+        }
+        for (int c = 0; c < len; ++c) {
+            const int rc = iteration();
+            if (rc != LRR_OK) return rc;
+        }
         return LRR_OK;
     };
     auto run_loop = [&](const std::vector<int>& act0) -> int {
@@ -903,10 +992,10 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         pick_shape(act0);
         tc_window = false;
         while (done_it < o->max_iter) {
-            for (int c = 0; c < chunk && done_it < o->max_iter; ++c, ++done_it) {
-                const int rc = iteration();
-                if (rc != LRR_OK) return rc;
-            }
+            const int len = std::min(chunk, o->max_iter - done_it);
+            const int rc = run_chunk(len);
+            if (rc != LRR_OK) return rc;
+            done_it += len;
             prof.begin();
             LRR_CUDA_TRY(cudaMemcpyAsync(ah.data(), B.act, sizeof(int) * t, cudaMemcpyDeviceToHost, s));
             if (bf16_phase) LRR_CUDA_TRY(cudaMemcpyAsync(fh.data(), B.fp32_on, sizeof(int) * t, cudaMemcpyDeviceToHost, s));
