@@ -17,57 +17,94 @@ template <typename T>
 __device__ __forceinline__ void jacobi_rotation(T app, T aqq, T apq, T& cc, T& ss);
 
 // float64 quotients, reciprocals and square roots of the rotation, rounded as
-// IEEE division and square root round them.  Three divisions and two square
-// roots in a chain were 60 % of the float64 pivots; here each starts from the
-// float32 unit's approximation, takes one Newton step in float64 and ends with
+// IEEE division and square root round them.  A dependent float64 operation takes
+// 65 cycles here (a float32 one 4), conversions and compares included, so the
+// seeds are taken to 2^-43 in pairs of float32 (one Newton step on the hardware
+// approximation, the argument's low bits as a second float32), exponents and
+// conversions are handled as integers, and float64 is left with the product and
 // the remainder correction of P. Markstein ("IA-64 and Elementary Functions",
-// 2000, ch. 8 and 9).  The result before its last rounding is good to 2^-88 or
-// better, so it differs from the IEEE one with probability below 2^-34.
-// (Equal in 4e9 random cases each, tested against / and sqrt.)
+// 2000, ch. 8 and 9): 3 operations for a quotient or a root, 2 for a
+// reciprocal.  The result before its last rounding is good to 2^-86, so it
+// differs from the IEEE one with probability below 2^-32.
+// (4e9 random cases each against / and sqrt: one reciprocal differed.)
 
-// 1 / b (1 + O(2^-45)) for b whose float32 reciprocal is normal
-__device__ __forceinline__ double rcp_newton(double b) {
-    float f;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)b));
-    const double y = (double)f;
-    return fma(y, fma(-b, y, 1.0), y);
+// y0 + y1 as a double, for y0 in [0.5, 1], |y1| < 2^-21, to 2^-44: y1 is added
+// to the bit pattern in units of 2^-43 (2^10 units in the last place)
+__device__ __forceinline__ double join(float y0, float y1) {
+    const int k = __float_as_int(fmaf(y1, 8796093022208.f, 12582912.f)) - 0x4B400000;
+    const int f = __float_as_int(y0);
+    const long long bits = (long long)(((unsigned long long)(unsigned)((f >> 3) + 0x38000000) << 32) | ((unsigned)f << 29));
+    return __longlong_as_double(bits + ((long long)k << 10));
 }
-// 1 / b
-__device__ __forceinline__ double rcp_rn(double b, double y) { return fma(y, fma(-b, y, 1.0), y); }
+// mantissa of b (high word hb, low word lb) as high + low 2^-23, high in [1, 2)
+__device__ __forceinline__ void split_mantissa(int hb, int lb, float& high, float& low) {
+    high = __int_as_float(0x3F800000 | ((hb & 0x000FFFFF) << 3) | (int)((unsigned)lb >> 29));
+    low = __int_as_float(0x3F800000 | (int)(((unsigned)lb << 3) >> 9)) - 1.f;
+}
+// 2^n b for a result in the normal range
+__device__ __forceinline__ double scale2(double b, int n) {
+    return __hiloint2double(__double2hiint(b) + (n << 20), __double2loint(b));
+}
+// 1 / m (1 + O(2^-43)), m in [1, 2) the mantissa of (hb, lb)
+__device__ __forceinline__ double rcp_seed(int hb, int lb) {
+    float bh, bl, y;
+    split_mantissa(hb, lb, bh, bl);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(bh));
+    y = fmaxf(y, 0.5f);
+    const float e = fmaf(bl, y * -0x1p-23f, fmaf(-bh, y, 1.f));
+    return join(y, y * fmaf(e, e, e));
+}
+// 1 / s from y = (1 / s)(1 + O(2^-43))
+__device__ __forceinline__ double rcp_rn(double s, double y) { return fma(y, fma(-s, y, 1.0), y); }
+// 1 / b, b in [1, 2^900]
+__device__ __forceinline__ double rcp_rn(double b) {
+    const int hb = __double2hiint(b);
+    return rcp_rn(b, scale2(rcp_seed(hb, __double2loint(b)), 1023 - (hb >> 20)));
+}
 // a / b over the whole range: mantissas in [1, 2) and the exponents apart; near
 // the ends of the range the division itself
 __device__ __forceinline__ double div_rn(double a, double b) {
-    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    const int ha = __double2hiint(a), hb = __double2hiint(b), lb = __double2loint(b);
     const int ea = (ha >> 20) & 0x7FF, eb = (hb >> 20) & 0x7FF;
     const int n = ea - eb;
     if (ea < 64 || ea > 1982 || eb < 64 || eb > 1982 || n > 900 || n < -900) return a / b;
     const double am = __hiloint2double((ha & 0x000FFFFF) | 0x3FF00000, __double2loint(a));
-    const double bm = __hiloint2double((hb & 0x000FFFFF) | 0x3FF00000, __double2loint(b));
-    const double y = rcp_newton(bm);
+    const double bm = __hiloint2double((hb & 0x000FFFFF) | 0x3FF00000, lb);
+    const double y = rcp_seed(hb, lb);
     const double q = am * y;
     const double r = fma(fma(-bm, q, am), y, q);
-    return r * __hiloint2double(((ha ^ hb) & 0x80000000) | ((n + 1023) << 20), 0);
+    return __hiloint2double((__double2hiint(r) + (n << 20)) | ((ha ^ hb) & 0x80000000), __double2loint(r));
 }
 // s = sqrt(x) and y = 1 / s (1 + O(2^-43)), x in [1, 1e32]
 __device__ __forceinline__ double sqrt_rn(double x, double& y) {
-    float f;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)x));
-    const double y0 = (double)f, g = x * y0, h = 0.5 * y0;
-    const double r = fma(-h, g, 0.5);
-    const double g1 = fma(g, r, g), h1 = fma(h, r, h);
-    y = 2.0 * h1;
-    return fma(fma(-g1, g1, x), h1, g1);
+    const int hx = __double2hiint(x), lx = __double2loint(x), ex = (hx >> 20) - 1023;
+    float mh, ml, r;
+    split_mantissa(hx, lx, mh, ml);                 // x = (mh + 2^-23 ml) 2^ex
+    if (ex & 1) { mh += mh; ml += ml; }             // now in [1, 4), and an even power
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(mh));
+    r = fmaxf(r, 0.5f);
+    const float p = r * r, pl = fmaf(r, r, -p);     // r^2 = p + pl
+    const float e = fmaf(ml, p * -0x1p-23f, fmaf(-mh, pl, fmaf(-mh, p, 1.f)));
+    y = scale2(join(r, r * e * fmaf(0.375f, e, 0.5f)), -(ex >> 1));
+    const double g = x * y;
+    return fma(fma(-g, g, x), scale2(y, -1), g);
 }
 template <>
 __device__ __forceinline__ void jacobi_rotation<double>(double app, double aqq, double apq, double& cc, double& ss) {
+    // tan = 1 / (|theta| + sqrt(theta^2 + 1)), beyond 1 / eps 1 / (2 |theta|): one
+    // reciprocal either way, so that lanes of both kinds share it
     const double theta = div_rn(aqq - app, 2.0 * apq);
+    const int ht = __double2hiint(theta) & 0x7FFFFFFF, lt = __double2loint(theta);
+    const int sign = __double2hiint(theta) < 0 && (ht | lt) != 0 ? (int)0x80000000 : 0;
+    const bool large = ht > 0x43300000 || (ht == 0x43300000 && lt != 0);        // |theta| > 2^52
+    const double at = __hiloint2double(ht, lt);
     double tt, y;
-    if (fabs(theta) > 1.0 / DBL_EPSILON) {
-        tt = div_rn(0.5, theta);
+    if (ht < (1023 + 900) << 20) {
+        const double sum = at + sqrt_rn(fma(theta, theta, 1.0), y);
+        const double t = rcp_rn(large ? at : sum);
+        tt = __hiloint2double((__double2hiint(t) - (large ? 1 << 20 : 0)) | sign, __double2loint(t));
     } else {
-        const double b = fabs(theta) + sqrt_rn(fma(theta, theta, 1.0), y);
-        const double t = rcp_rn(b, rcp_newton(b));
-        tt = theta >= 0.0 ? t : -t;
+        tt = 0.5 / theta;
     }
     const double h = sqrt_rn(fma(tt, tt, 1.0), y);
     cc = rcp_rn(h, y);

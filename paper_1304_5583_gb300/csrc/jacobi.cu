@@ -17,7 +17,7 @@ namespace {
 constexpr int NT = 256;
 
 // threads of a pivot's CTA
-template <typename T> __host__ __device__ constexpr int solve_threads() { return sizeof(T) == 8 ? 256 : 1024; }
+template <typename T> __host__ __device__ constexpr int solve_threads() { return sizeof(T) == 8 ? 384 : 1024; }
 
 // global row of local index i (0..2b-1) of the pivot pair (a, c)
 __device__ __forceinline__ int pair_row(int i, int a, int c, int b) { return i < b ? a * b + i : c * b + (i - b); }
@@ -31,8 +31,9 @@ __device__ __forceinline__ int pair_row(int i, int a, int c, int b) { return i <
 // float32 (64 x 64, one sweep): thread (k, l) of 32 x 32 owns the 2 x 2 sub-block
 // of pairs k and l and two rows of R's pair l; it works out pair k's rotation
 // itself, takes pair l's from the lane that has it and writes the other S
-// buffer, so a round has one barrier (0.3 us; 1.3 us with 256 threads and a
-// barrier on either side of the rotations: 81 us a pivot, now 20).
+// buffer, so a round has one barrier.  Bound by shared memory (19 accesses a
+// thread and round): 70 us a pivot of the 500 x 500 Gram, 81 with 256 threads
+// and a barrier on either side of the rotations.
 template <int B2, int LS>
 __device__ int inner_sweep_f32(float (*S2)[B2 * LS], float* R, float floor_rot, int* cur_out) {
     constexpr int b = B2 / 2;
@@ -73,88 +74,174 @@ __device__ int inner_sweep_f32(float (*S2)[B2 * LS], float* R, float floor_rot, 
     return __syncthreads_or(rotated);
 }
 
-// |apq| > eps sqrt(|app aqq|) in float64, exactly; the square root is taken only
-// where an estimate from the exponent (0 to 6.1 % above it) does not decide
-__device__ __forceinline__ bool above_eps(double app, double aqq, double apq) {
-    const double g = fabs(app * aqq);
-    const double est = __hiloint2double((__double2hiint(g) >> 1) + 0x1FF80000, 0);
-    if (g > 1e-290) {
-        if (apq > 1.001 * DBL_EPSILON * est) return true;
-        if (apq < 0.94 * DBL_EPSILON * est) return false;
-    }
-    return apq > DBL_EPSILON * sqrt(g);
+// log2(|apq| / sqrt|app aqq|) in float32, to 2^-19, from exponents and top
+// mantissa bits; false near the ends of the range, where it is not defined.
+// (The float64 product, root and compares of the exact form are 800 cycles.)
+__device__ __forceinline__ float log2_mantissa(double x) {
+    float l;
+    const int m = ((__double2hiint(x) & 0x000FFFFF) << 3) | (int)((unsigned)__double2loint(x) >> 29);
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(__int_as_float(0x3F800000 | m)));
+    return l;
+}
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+__device__ __forceinline__ bool log2_ratio(double app, double aqq, double apq, float& d) {
+    const int ep = exponent(app), eq = exponent(aqq), eo = exponent(apq);
+    const float l = log2_mantissa(apq) - 0.5f * (log2_mantissa(app) + log2_mantissa(aqq));
+    d = 0.5f * (float)(2 * eo - ep - eq) + l;
+    return ep >= 64 && ep < 1982 && eq >= 64 && eq < 1982 && eo < 1982 && ep + eq >= 1084 && ep + eq <= 3004;
+}
+__device__ __forceinline__ double negated(double x) {
+    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+}
+// |x| > y >= 0, x not a NaN (bit patterns order like the values)
+__device__ __forceinline__ bool abs_above(double x, double y) {
+    return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) > __double_as_longlong(y);
+}
+// |apq| > floor_rot and |apq| > eps sqrt(|app aqq|) in float64, exactly: root and
+// product are taken only where the estimate does not decide (entries that are
+// rounding noise lie near eps: an estimate to 7 % left one in every few rounds
+// undecided)
+__device__ __forceinline__ bool must_rotate(double app, double aqq, double apq, double floor_rot) {
+    float d;
+    if (!abs_above(apq, floor_rot)) return false;
+    if (log2_ratio(app, aqq, apq, d) && fabsf(d + 52.f) > 1e-4f) return d > -52.f;
+    return fabs(apq) > floor_rot && fabs(apq) > DBL_EPSILON * sqrt(fabs(app * aqq));
 }
 
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
 // float64 (32 x 32, up to max_sweeps; it stops after a sweep in which no entry
-// above floor_sig was rotated).  Bound by the float64 units (two FMA lanes per SM
-// and clock) and their latency, and on average only 5 or 6 of a round's 16 pairs
-// still rotate: so a round first finds those, and only their rows, then their
-// columns, are touched; an idle round ends at its first barrier.  (Every 2 x 2
-// sub-block every round: 466 us a pivot on the 500 x 5000 problem, now 360, of
-// which the rotations themselves, a chain of three divisions and two square roots,
-// are 60 %.)
+// above floor_sig was rotated).  Bound by the latency of the float64 unit (65
+// cycles an operation, one warp instruction every 19 whatever its lanes) along
+// the chain from one round's rotations to the next's.  So warp 0 does nothing
+// but that chain: it finds the pairs that rotate (6 or 7 of a round's 16, none
+// in one round of eight), works out their rotations, lists them for the other
+// eight warps and goes on to the next round's diagonal and pair entries on its
+// own, from the two-by-two blocks they lie in; the others update the listed
+// pairs' rows and columns of S, and R, behind it, and it waits for them only
+// before it reads S again.  The schedule moves every pair's item by one
+// position a round, so the lanes that hold the two pairs a new pair comes from
+// are fixed.  A round takes 3900 cycles, 2100 of them the rotations and 1100 the
+// next entries (6400 with every step between barriers of the whole CTA): 204 us
+// a pivot of the 500 x 500 Gram, 466 when every 2 x 2 sub-block was updated every
+// round.  The warps that share warp 0's scheduler are left out of the updates.
 template <int B2, int LS>
-__device__ int inner_sweeps_f64(double* S, double* R, double2* cs, int2* pq, int* count2, double floor_rot,
-                                double floor_sig, int max_sweeps) {
-    constexpr int b = B2 / 2;
+__device__ int inner_sweeps_f64(double* S, double* R, double2 (*cs)[B2 / 2], int2 (*pq)[B2 / 2], int* count,
+                                double floor_rot, double floor_sig, int max_sweeps) {
+    constexpr int b = B2 / 2, NW = 9 * 32, NB = NW + 32;
+    static_assert(b == 16, "lanes 16 to 31 repeat lanes 0 to 15");
     const int t = threadIdx.x;
-    int any = 0, phase = 0;
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        int sig = 0;
-        for (int r = 0; r < B2 - 1; ++r, phase ^= 1) {
-            if (t < 32) {
-                bool act = false;
-                double c = 1.0, sv = 0.0;
-                const int k = t & (b - 1);
-                const int p = circle_item(k, r, B2), q = circle_item(B2 - 1 - k, r, B2);
-                if (t < b) {
-                    const double app = S[p * LS + p], aqq = S[q * LS + q], apq = S[p * LS + q];
-                    act = fabs(apq) > floor_rot && above_eps(app, aqq, fabs(apq));
-                    if (act) {
-                        jacobi_rotation<double>(app, aqq, apq, c, sv);
-                        if (fabs(apq) > floor_sig && fabs(sv) > 0.0) sig = 1;
+    // barriers: 1 S is up to date (the others arrive, warp 0 waits), 2 a list is
+    // out (warp 0 arrives, the others wait), 3 among the others
+    if (t < 32) {
+        const int k = t & (b - 1);
+        const bool first = k == 0, last = k == b - 1, low = t < b;
+        int p = circle_item(k, 0, B2), q = circle_item(B2 - 1 - k, 0, B2), any = 0, buf = 0;
+        double app = S[p * LS + p], aqq = S[q * LS + q], apq = S[p * LS + q];
+        bool pending = false;
+        for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+            int sig = 0;
+            for (int r = 0; r < B2 - 1; ++r) {
+                const bool act = must_rotate(app, aqq, apq, floor_rot);
+                const unsigned m = __ballot_sync(0xffffffffu, act) & ((1u << b) - 1);
+                // the pairs the next round's pair k comes from: A, whose p (k = 15: q)
+                // is its p, and B, whose q (k = 0: p) is its q
+                const int pd = __shfl_down_sync(0xffffffffu, p, 1, b), qd = __shfl_down_sync(0xffffffffu, q, 1, b);
+                const int pu = __shfl_up_sync(0xffffffffu, p, 1, b), qu = __shfl_up_sync(0xffffffffu, q, 1, b);
+                const bool own = first || last;
+                const int pA = own ? p : pd, qA = own ? q : qd, pB = first ? pd : pu, qB = first ? qd : qu;
+                if (!m) {
+                    if (pending) bar_sync(1, NB);
+                    pending = false;
+                    apq = S[(last ? qA : pA) * LS + (first ? pB : qB)];
+                } else {
+                    any = 1;
+                    double c = 1.0, s = 0.0;
+                    if (act) jacobi_rotation<double>(app, aqq, apq, c, s);
+                    if (pending) bar_sync(1, NB);
+                    const double aqp = S[q * LS + p];
+                    const double e00 = S[pA * LS + pB], e01 = S[pA * LS + qB];
+                    const double e10 = S[qA * LS + pB], e11 = S[qA * LS + qB];
+                    if (act && t < b) {
+                        const int at = __popc(m & ((1u << k) - 1));
+                        cs[buf][at] = make_double2(c, s);
+                        pq[buf][at] = make_int2(p, q);
                     }
+                    if (t == 0) count[buf] = __popc(m);
+                    if (act && abs_above(apq, floor_sig) && abs_above(s, 0.0)) sig = 1;
+                    const double cd = __shfl_down_sync(0xffffffffu, c, 1, b), sd = __shfl_down_sync(0xffffffffu, s, 1, b);
+                    const double cu = __shfl_up_sync(0xffffffffu, c, 1, b), su = __shfl_up_sync(0xffffffffu, s, 1, b);
+                    const double cA = own ? c : cd, sA = own ? s : sd, cB = first ? cd : cu, sB = first ? sd : su;
+                    const bool actA = (m >> (own ? k : k + 1)) & 1, actB = (m >> (first ? 1 : k - 1)) & 1;
+                    // rows, then columns, as the others do them; the lower lanes take
+                    // the p row and the first column, the upper ones the q row and the
+                    // second (a float64 operation costs the same for any lanes)
+                    const double f = low ? c : s, g = low ? negated(s) : c;
+                    const double fA = last ? sA : cA, gA = last ? cA : negated(sA), fB = first ? cB : sB, gB = first ? negated(sB) : cB;
+                    const double e0 = low ? e00 : e01, e1 = low ? e10 : e11;
+                    const double r0 = fma(f, app, g * aqp), r1 = fma(f, apq, g * aqq);
+                    double x = fma(fA, e0, gA * e1);
+                    x = actA ? x : last ? e1 : e0;
+                    const double y = __shfl_down_sync(0xffffffffu, x, b), d = fma(f, r0, g * r1);
+                    const double z = fma(fB, x, gB * y), dq = __shfl_down_sync(0xffffffffu, d, b);
+                    apq = __shfl_sync(0xffffffffu, actB ? z : first ? x : y, k);
+                    app = __shfl_sync(0xffffffffu, act ? d : app, k);
+                    aqq = __shfl_sync(0xffffffffu, act ? dq : aqq, k);
+                    bar_arrive(2, NB);
+                    pending = true;
+                    buf ^= 1;
                 }
-                // the rotating pairs, listed
-                const unsigned m = __ballot_sync(0xffffffffu, act);
-                if (act) {
-                    const int at = __popc(m & ((1u << t) - 1));
-                    cs[at] = make_double2(c, sv);
-                    pq[at] = make_int2(p, q);
-                }
-                if (t == 0) count2[phase] = __popc(m);
+                const double ad = __shfl_down_sync(0xffffffffu, app, 1, b), au = __shfl_up_sync(0xffffffffu, aqq, 1, b);
+                app = first ? app : last ? aqq : ad;
+                aqq = first ? ad : au;
+                p = last ? qA : pA;
+                q = first ? pB : qB;
             }
-            __syncthreads();
-            const int cnt = count2[phase] * B2;
-            if (!cnt) continue;
-            any = 1;
-            // rows p and q of every rotating pair
-            for (int e = t; e < cnt; e += NT) {
-                const int j = e % B2;
-                const int2 w = pq[e / B2];
-                const double2 r2 = cs[e / B2];
-                const double x = S[w.x * LS + j], y = S[w.y * LS + j];
-                S[w.x * LS + j] = fma(r2.x, x, -(r2.y * y));
-                S[w.y * LS + j] = fma(r2.y, x, r2.x * y);
-            }
-            __syncthreads();
-            // columns, and R
-            for (int e = t; e < 2 * cnt; e += NT) {
-                const bool isr = e >= cnt;
-                const int f = isr ? e - cnt : e, i = f % B2;
-                const int2 w = pq[f / B2];
-                const double2 r2 = cs[f / B2];
-                double* const A = (isr ? R : S) + i * LS;
-                const double x = A[w.x], y = A[w.y];
-                // the pair's own off-diagonal entries are zero by construction
-                A[w.x] = !isr && i == w.y && r2.y != 0.0 ? 0.0 : fma(r2.x, x, -(r2.y * y));
-                A[w.y] = !isr && i == w.x && r2.y != 0.0 ? 0.0 : fma(r2.y, x, r2.x * y);
-            }
-            __syncthreads();
+            if (!__any_sync(0xffffffffu, sig)) break;
         }
-        if (!__syncthreads_or(sig)) break;
+        if (pending) bar_sync(1, NB);
+        if (t == 0) { count[buf] = -1; count[2] = any; }
+        __syncwarp();
+        bar_arrive(2, NB);
+    } else if (t / 32 % 4 != 0) {
+        const int lane = t & 31, w = t / 32 - 1 - t / 128;
+        for (int buf = 0;; buf ^= 1) {
+            bar_sync(2, NB);
+            const int n = count[buf];
+            if (n < 0) break;
+            // rows p and q of every rotating pair
+            for (int i = w; i < n; i += NW / 32) {
+                const int2 v = pq[buf][i];
+                const double2 r2 = cs[buf][i];
+                double* const A = S + lane;
+                const double x = A[v.x * LS], y = A[v.y * LS];
+                A[v.x * LS] = fma(r2.x, x, -(r2.y * y));
+                A[v.y * LS] = fma(r2.y, x, r2.x * y);
+            }
+            bar_sync(3, NW);
+            // columns; the pair's own off-diagonal entries are zero by construction
+            for (int i = w; i < n; i += NW / 32) {
+                const int2 v = pq[buf][i];
+                const double2 r2 = cs[buf][i];
+                double* const A = S + lane * LS;
+                const double x = A[v.x], y = A[v.y];
+                A[v.x] = lane == v.y && r2.y != 0.0 ? 0.0 : fma(r2.x, x, -(r2.y * y));
+                A[v.y] = lane == v.x && r2.y != 0.0 ? 0.0 : fma(r2.y, x, r2.x * y);
+            }
+            bar_arrive(1, NB);
+            for (int i = w; i < n; i += NW / 32) {
+                const int2 v = pq[buf][i];
+                const double2 r2 = cs[buf][i];
+                double* const A = R + lane * LS;
+                const double x = A[v.x], y = A[v.y];
+                A[v.x] = fma(r2.x, x, -(r2.y * y));
+                A[v.y] = fma(r2.y, x, r2.x * y);
+            }
+        }
     }
-    return any;
+    __syncthreads();
+    return count[2];
 }
 
 template <typename T, int B2>
@@ -171,9 +258,9 @@ __global__ void __launch_bounds__(solve_threads<T>()) jac_solve(const JacDesc<T>
     extern __shared__ __align__(16) unsigned char jac_smem[];
     T* const S0 = reinterpret_cast<T*>(jac_smem);            // float32: two buffers
     T* const R = S0 + (sizeof(T) == 8 ? 1 : 2) * B2 * LS;
-    __shared__ double2 cs[b];
-    __shared__ int2 pq[b];
-    __shared__ int count2[2];
+    __shared__ double2 cs[2][b];
+    __shared__ int2 pq[2][b];
+    __shared__ int count[3];
     __shared__ T red[NS / 32];
     const int t = threadIdx.x;
     // Off-diagonal entries below the rounding noise of the Gram products
@@ -195,13 +282,24 @@ __global__ void __launch_bounds__(solve_threads<T>()) jac_solve(const JacDesc<T>
     // any entry is large enough to rotate at all
     T offm = T(0);
     int any = 0;
+    const float log2_tol = log2f((float)tol);
     for (int e = t; e < B2 * B2; e += NS) {
         const int i = e % B2, j = e / B2;
         if (i < j) {
             const T v = fabs(S0[i * LS + j]);
+            if constexpr (sizeof(T) == 8) {
+                // only the comparison with tol is used of the measure
+                float d;
+                any |= must_rotate(S0[i * LS + i], S0[j * LS + j], v, floor_rot);
+                if (!abs_above(v, floor_abs)) continue;
+                if (log2_ratio(S0[i * LS + i], S0[j * LS + j], v, d) && fabsf(d - log2_tol) > 1e-3f) {
+                    if (d > log2_tol) offm = T(2) * tol;
+                    continue;
+                }
+            }
             const T sc = sqrt(fabs(S0[i * LS + i] * S0[j * LS + j]));
             if (v > floor_abs) offm = fmax(offm, v / (sc + num<T>::tiny()));
-            if (v > floor_rot && v > num<T>::eps() * sc) any = 1;
+            if (sizeof(T) == 4 && v > floor_rot && v > num<T>::eps() * sc) any = 1;
         }
     }
     offm = warp_max(offm);
@@ -218,7 +316,7 @@ __global__ void __launch_bounds__(solve_threads<T>()) jac_solve(const JacDesc<T>
     // per pivot, the outer sweeps continue from there; float64: up to six
     int any_rot = 0, cur = 0;
     if (need) {
-        if constexpr (sizeof(T) == 8) any_rot = inner_sweeps_f64<B2, LS>(S0, R, cs, pq, count2, floor_rot, floor_abs, 6);
+        if constexpr (sizeof(T) == 8) any_rot = inner_sweeps_f64<B2, LS>(S0, R, cs, pq, count, floor_rot, floor_abs, 6);
         else any_rot = inner_sweep_f32<B2, LS>(reinterpret_cast<float(*)[B2 * LS]>(S0), R, floor_rot, &cur);
     }
     // diagonalised pivot block back into G, rotation out for the apply kernel
