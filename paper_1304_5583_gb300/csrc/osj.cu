@@ -1060,18 +1060,29 @@ OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster) {
     // resident at once -- a block waiting for a second wave would double the
     // time of the whole batch.  A cluster with room for several CTAs per pivot
     // splits its pivots, while a member keeps at least two chunks of rows.
-    // Wide CTAs where a whole round's pivots fit the chip that way.
+    // Wide CTAs are taken while that leaves at most twice as many pivots to a
+    // CTA as the streamed form would: ten blocks of 11 pivots fit as clusters of
+    // 10 wide or 11 streamed CTAs, 170 against 225 ms over the 245 iterations of
+    // the 500 x 5000 solve; 12 blocks of 13 pivots as 10 or 13, 188 against 266
+    // (6 wide, 249); 40 blocks of 18 pivots as 3 or 10, 2.9 against 2.0 s.
     const int pairs = std::max(1, pairs_of<T>(max_p)), cmax = osj_max_cluster<T>();
     const int limit = cluster > 0 ? std::min(cluster, cmax) : cmax;
     auto fits = [&](const OsjShape& sh) { return resident_clusters<T>(sh) >= nmat; };
-    for (int split = 4; split >= 1; split /= 2) {
+    for (int split = 4; split > 1; split /= 2) {
         const OsjShape sh{pairs * split, split, 1, max_L, max_p};
-        if (sh.cluster > limit || (split > 1 && split * 64 > max_L + max_p)) continue;
-        if (fits(sh)) return sh;
+        if (sh.cluster <= limit && split * 64 <= max_L + max_p && fits(sh)) return sh;
     }
-    for (int c = std::min(limit, pairs); c > 1; --c)
-        if (cluster > 0 || fits(OsjShape{c, 1, 0, max_L, max_p})) return OsjShape{c, 1, 0, max_L, max_p};
-    return OsjShape{1, 1, 0, max_L, max_p};
+    // the largest cluster of each form
+    auto largest = [&](int wide) {
+        for (int c = std::min(limit, pairs); c > 0; --c) {
+            const OsjShape sh{c, 1, wide, max_L, max_p};
+            if (fits(sh) || (!wide && cluster > 0)) return sh;
+        }
+        return OsjShape{wide ? 0 : 1, 1, wide, max_L, max_p};
+    };
+    const OsjShape wide = largest(1), streamed = largest(0);
+    if (wide.cluster > 0 && ceil_div(pairs, wide.cluster) <= 2 * ceil_div(pairs, streamed.cluster)) return wide;
+    return streamed;
 }
 
 template <typename T>
