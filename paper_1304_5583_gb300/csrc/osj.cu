@@ -142,6 +142,11 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -155,33 +160,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // to working accuracy.  Hardware reciprocal and reciprocal square root: the
 // rotation only steers the pivot towards diagonal form, the accumulated R is
 // re-orthonormalised before use, and the next sweep forms its Grams afresh.
-__device__ __forceinline__ void rotation(float app, float aqq, float apq, float& c, float& s) {
-    const float d = aqq - app, b = 2.f * apq;
+__device__ __forceinline__ void rotation(float d, float apq, float& t, float& c, float& s) {
+    const float b = 2.f * apq;
     const unsigned e = __float_as_uint(fmaxf(fabsf(d), fabsf(b))) & 0x7F800000u;
     const float sc = __uint_as_float(0x7F000000u - e);
     const float fd = d * sc, fb = b * sc;
     const float h = fmaf(fd, fd, fb * fb);
-    const float t = fb * rcp_approx(fd + copysignf(h * rsqrt_approx(h), fd));
+    t = fb * rcp_approx(fd + copysignf(h * rsqrt_approx(h), fd));
     c = rsqrt_approx(fmaf(t, t, 1.f));
     s = t * c;
-}
-// float64: c and s from the float32 units (a float64 divide or square root
-// costs more than the rest of a round), then scaled to c^2 + s^2 = 1 in float64:
-// the rotation is orthogonal to float64 rounding and leaves about 1e-7 of s_pq,
-// which the second pass and the next sweep take.
-__device__ __forceinline__ void rotation(double app, double aqq, double apq, double& c, double& s) {
-    double d = aqq - app, b = 2.0 * apq;
-    const int e = __double2hiint(fmax(fabs(d), fabs(b))) & 0x7FF00000;
-    const double sc = __hiloint2double(0x7FE00000 - e, 0);
-    const float fd = (float)(d * sc), fb = (float)(b * sc);
-    const float h = fmaf(fd, fd, fb * fb);
-    const float t = fb * rcp_approx(fd + copysignf(h * rsqrt_approx(h), fd));
-    const float c0 = rsqrt_approx(fmaf(t, t, 1.f));
-    const double cd = (double)c0, sd = (double)(t * c0);
-    const double q = fma(-cd, cd, fma(-sd, sd, 1.0));      // the squares of 24-bit values are exact
-    const double g = q * fma(0.375, q, 0.5);               // (1 - q)^(-1/2) - 1 to O(q^3), q about 1e-7
-    c = fma(cd, g, cd);
-    s = fma(sd, g, sd);
 }
 // |s_pq| > eps sqrt(s_pp s_qq), with a square root good to a few per cent
 __device__ __forceinline__ bool needs_rotation(float app, float aqq, float apq) {
@@ -189,12 +176,6 @@ __device__ __forceinline__ bool needs_rotation(float app, float aqq, float apq) 
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(fabsf(app * aqq)));
     return fabsf(apq) > FLT_MIN && fabsf(apq) > FLT_EPSILON * q;
 }
-__device__ __forceinline__ bool needs_rotation(double app, double aqq, double apq) {
-    const int hi = __double2hiint(fabs(app * aqq));
-    const double q = __hiloint2double((hi >> 1) + 0x1FF80000, 0);    // exponent halved
-    return fabs(apq) > DBL_MIN && fabs(apq) > DBL_EPSILON * q;
-}
-
 // non-negative norms ordered by their bits (a NaN sorts first: the order stays
 // a permutation whatever the input holds)
 __device__ __forceinline__ unsigned key_of(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
@@ -287,7 +268,8 @@ template <typename T>
 struct PivotCtx {
     T *X, *W;
     int ldx, ldw, L, p;
-    T scale, tau, floor2;
+    T scale, tau, floor2, inv_scale;
+    float ftau;
     T *stage, *panel, *wpanel;      // stage; kept columns of X and of W (512 threads)
     int rank, split, member, stride, wstride;
     bool first_round;     // first round of the sweep: pairs inside the column blocks too
@@ -449,6 +431,114 @@ __device__ __forceinline__ void tile_update(const double* R4, const double* cols
         for (int i = 0; i < RT; ++i) store(i, v, cols[(h * 8 + v) * stride + 32 * i] + a[i][v]);
 }
 
+// The inner rotations of a float64 pivot (sorted schedule), in float32 apart
+// from the diagonal, which is kept as pairs of float32 so that the gaps of close
+// columns are known to 2^-48.  A float64 operation takes 65 cycles and one warp
+// instruction every 19 keeps the whole SM's unit busy: 32 us a pivot in float64,
+// of 80.  The rotations only steer: what float32 leaves behind is 1e-7 of what
+// was rotated away, found again by the next sweep's float64 Gram, while R is
+// made orthogonal to float64 rounding before it is applied.  Up to two passes; the
+// second is left out when no tangent was above 1e-6 (its square is below
+// float32's own error by then).
+__device__ __forceinline__ void inner_f64(Smem<double>& sm, double scale, double floor2, bool first_round) {
+    constexpr int OB = Cfg<double>::OB, B2 = 2 * OB, LS = Cfg<double>::LS;
+    const int t = threadIdx.x;
+    float* const S2 = reinterpret_cast<float*>(sm.S[1]);       // two buffers
+    float* const R = reinterpret_cast<float*>(sm.G);
+    float* const lo2 = R + B2 * LS;                            // low parts of the diagonal, two buffers
+    static_assert(B2 * LS + 2 * B2 <= 2 * B2 * B2, "R and the low parts in the place of R^T R");
+    // the largest column's square to 2^60: entries down to 1e-56 of it are normal
+    const int e = 1023 + 60 - ((__double2hiint(scale) >> 20) - 1023);
+    const int ec = min(max(e, 1), 2045);
+    const double sc = __hiloint2double(ec << 20, 0), inv_sc = __hiloint2double((2046 - ec) << 20, 0);
+    if (t < B2 * B2) {
+        const int i = t / B2, j = t % B2;
+        const double v = sm.S[0][i * LS + j] * sc;
+        const float f = (float)v;
+        S2[i * LS + j] = f;
+        R[i * LS + j] = i == j ? 1.f : 0.f;
+        if (i == j) lo2[i] = (float)(v - (double)f);
+    }
+    const float ffloor = (float)(floor2 * sc);
+    __syncthreads();
+    if (t < OB * OB) {
+        const int k = t % OB, l = t / OB;
+        int cur = 0, rotated = 0;
+        const int r_first = first_round ? -(OB - 1) : 0;
+        for (int pass = 0; pass < 2; ++pass) {
+            int big = 0;
+            for (int r = r_first; r < OB; ++r) {
+                int pk, qk, pl, ql;
+                if (r >= 0) {
+                    pk = k; qk = OB + ((k + r) & (OB - 1));
+                    pl = l; ql = OB + ((l + r) & (OB - 1));
+                } else {
+                    // pairs inside column block a (first half) and c
+                    constexpr int H = OB / 2;
+                    const int rr = r + OB - 1, ok = k < H ? 0 : OB, ol = l < H ? 0 : OB;
+                    pk = ok + circle_item(k & (H - 1), rr, OB); qk = ok + circle_item(OB - 1 - (k & (H - 1)), rr, OB);
+                    pl = ol + circle_item(l & (H - 1), rr, OB); ql = ol + circle_item(OB - 1 - (l & (H - 1)), rr, OB);
+                }
+                const float* const S = S2 + cur * B2 * LS;
+                float* const D = S2 + (cur ^ 1) * B2 * LS;
+                const float* const lo = lo2 + cur * B2;
+                float* const lo_new = lo2 + (cur ^ 1) * B2;
+                const float app = S[pk * LS + pk], aqq = S[qk * LS + qk], apq = S[pk * LS + qk];
+                const float lp = lo[pk], lq = lo[qk];
+                const float s_pu = S[pk * LS + pl], s_pv = S[pk * LS + ql], s_qu = S[qk * LS + pl], s_qv = S[qk * LS + ql];
+                const float x0 = R[k * LS + pl], y0 = R[k * LS + ql];
+                const float x1 = R[(k + OB) * LS + pl], y1 = R[(k + OB) * LS + ql];
+                float tk, ck, sk;
+                rotation((aqq - app) + (lq - lp), apq, tk, ck, sk);
+                const bool act = fabsf(apq) > FLT_MIN &&
+                                 fabsf(apq) > (float)DBL_EPSILON * (sqrt_approx(fabsf(app)) * sqrt_approx(fabsf(aqq)));
+                tk = act ? tk : 0.f;
+                ck = act ? ck : 1.f;
+                sk = act ? sk : 0.f;
+                rotated |= act;
+                big |= act && fabsf(apq) > ffloor && fabsf(tk) > 1e-6f;
+                const float clr = __shfl_sync(0xffffffffu, ck, l), slr = __shfl_sync(0xffffffffu, sk, l);
+                const float r_pu = fmaf(ck, s_pu, -(sk * s_qu)), r_pv = fmaf(ck, s_pv, -(sk * s_qv));
+                const float r_qu = fmaf(sk, s_pu, ck * s_qu), r_qv = fmaf(sk, s_pv, ck * s_qv);
+                float d_pu = fmaf(clr, r_pu, -(slr * r_pv)), d_pv = fmaf(slr, r_pu, clr * r_pv);
+                float d_qu = fmaf(clr, r_qu, -(slr * r_qv)), d_qv = fmaf(slr, r_qu, clr * r_qv);
+                if (k == l) {
+                    // the pair's own block: diagonal +- t s_pq in pairs of float32
+                    const float x = tk * apq;
+                    const float hp = app - x, bp = hp - app, ep = ((app - (hp - bp)) + (-x - bp)) + lp;
+                    const float hq = aqq + x, bq = hq - aqq, eq = ((aqq - (hq - bq)) + (x - bq)) + lq;
+                    d_pu = hp + ep; lo_new[pk] = ep - (d_pu - hp);
+                    d_qv = hq + eq; lo_new[qk] = eq - (d_qv - hq);
+                    d_pv = act ? 0.f : s_pv;
+                    d_qu = act ? 0.f : s_qu;
+                }
+                D[pk * LS + pl] = d_pu;
+                D[pk * LS + ql] = d_pv;
+                D[qk * LS + pl] = d_qu;
+                D[qk * LS + ql] = d_qv;
+                R[k * LS + pl] = fmaf(clr, x0, -(slr * y0));
+                R[k * LS + ql] = fmaf(slr, x0, clr * y0);
+                R[(k + OB) * LS + pl] = fmaf(clr, x1, -(slr * y1));
+                R[(k + OB) * LS + ql] = fmaf(slr, x1, clr * y1);
+                cur ^= 1;
+                if (r == OB - 1) {
+                    if (big) sm.sig[pass] = 1;
+                    if (rotated) sm.rot = 1;
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(OB * OB) : "memory");
+            }
+            if (!sm.sig[pass]) break;
+        }
+        if (t == 0) sm.cur = cur;
+    }
+    __syncthreads();
+    if (t < B2 * B2) {
+        const int i = t / B2, j = t % B2;
+        sm.R[i * LS + j] = (double)R[i * LS + j];
+        if (i == j) sm.S[0][i * LS + i] = ((double)S2[sm.cur * B2 * LS + i * LS + i] + (double)lo2[sm.cur * B2 + i]) * inv_sc;
+    }
+}
+
 // One pivot (logical column blocks a and c) of one round: Gram, measure,
 // rotation.  Returns the convergence measure of the pivot (CTA-uniform);
 // top_a / top_c receive the two largest squared norms of the column blocks.
@@ -532,8 +622,8 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     } else {
         // the differences are taken in T, the rest in float32 on values relative
         // to the largest column: the measure only steers the sweeps
-        const T inv_scale = T(1) / (cx.scale + num<T>::tiny());
-        const float ftau = (float)(tau * sqrt(inv_scale));
+        const T inv_scale = cx.inv_scale;
+        const float ftau = cx.ftau;
         for (int e = t; e < B2 * B2; e += NT) {
             const int j = e % B2, i = e / B2;
             if (i >= j) continue;
@@ -616,12 +706,12 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     //      of these b^2 threads and one chain of shared read, rotation, write
     //      (0.25 us; 0.7 us with a barrier on either side of the rotations).
     //      Sorted: 62 rounds in the first round of a sweep, else 32, or half of
-    //      that when the first pass found only small angles (float32; no tangent
-    //      above 3e-4, in float64 1e-8: what the second would still find is the
-    //      square of that).  Kept: 31 rounds.
-    if (t < OB * OB) {
+    //      that when the first pass found only small angles (no tangent above
+    //      3e-4: what the second would still find is the square of that).  Kept: 31 rounds.
+    if constexpr (sizeof(T) == 8) {
+        inner_f64(sm, cx.scale, cx.floor2, cx.first_round);
+    } else if (t < OB * OB) {
         const int k = t % OB, l = t / OB;
-        const T exit_tan = sizeof(T) == 4 ? T(3e-4) : T(1e-8);
         int cur = 0, rotated = 0;
         const int r_first = KEEP ? 0 : cx.first_round ? -(OB - 1) : 0, r_end = KEEP ? B2 - 1 : OB;
         for (int pass = 0; pass < (KEEP ? 1 : 2); ++pass) {
@@ -656,20 +746,21 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
                     jacobi_rotation<T>(app, aqq, apq, ck, sk);
                 } else {
                     act = needs_rotation(app, aqq, apq);
-                    rotation(app, aqq, apq, ck, sk);
+                    float tn;
+                    rotation(aqq - app, apq, tn, ck, sk);
                 }
                 ck = act ? ck : T(1);
                 sk = act ? sk : T(0);
                 rotated |= act;
-                if (!KEEP) big |= act && fabs(apq) > cx.floor2 && fabs(sk) > exit_tan * ck;
+                if (!KEEP) big |= act && fabs(apq) > cx.floor2 && fabs(sk) > T(3e-4) * ck;
                 const T clr = __shfl_sync(0xffffffffu, ck, l), slr = __shfl_sync(0xffffffffu, sk, l);
                 // (fused multiply-adds written out: which product of a sum of two is
                 // rounded first is part of the kept schedule's arithmetic)
                 const T r_pu = fma(ck, s_pu, -(sk * s_qu)), r_pv = fma(ck, s_pv, -(sk * s_qv));
                 const T r_qu = fma(sk, s_pu, ck * s_qu), r_qv = fma(sk, s_pv, ck * s_qv);
-                // float32: the rotated pair's own off-diagonal entries are zero
-                // by construction (to the rounding of the next fresh Gram)
-                const bool zero = sizeof(T) == 4 && k == l && sk != T(0);
+                // the rotated pair's own off-diagonal entries are zero by
+                // construction (to the rounding of the next fresh Gram)
+                const bool zero = k == l && sk != T(0);
                 D[pk * LS + pl] = fma(clr, r_pu, -(slr * r_pv));
                 D[pk * LS + ql] = zero ? T(0) : fma(slr, r_pu, clr * r_pv);
                 D[qk * LS + pl] = zero ? T(0) : fma(clr, r_qu, -(slr * r_qv));
@@ -690,7 +781,7 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
         if (t == 0) sm.cur = cur;
     }
     __syncthreads();
-    Sd = sm.S[sm.cur];
+    if (sizeof(T) == 4) Sd = sm.S[sm.cur];
     tops();
     if (!sm.rot) {
         __syncthreads();
@@ -701,43 +792,55 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     // ~sqrt(count) eps; one Newton-Schulz step R <- R (3I - R^T R)/2 restores
     // orthogonality to ~eps^2 before R touches X and W (applied to graded
     // columns the defect would mix eps-sized parts of the large columns into
-    // the small ones)
+    // the small ones).  (Float64: R comes from float32 rotations, is orthogonal to
+    // some 1e-6 only and takes a second step unless all angles were tiny.)
     constexpr int PE = B2 * B2 / 256;             // consecutive entries of a row per thread
     const int ni = t * PE / B2, nj = t * PE % B2;
-    if (t < 256) {
-        T g[PE];
+    for (bool more = sizeof(T) == 8;;) {
+        int far = 0;
+        if (t < 256) {
+            T g[PE];
 #pragma unroll
-        for (int u = 0; u < PE; ++u) g[u] = T(0);
+            for (int u = 0; u < PE; ++u) g[u] = T(0);
 #pragma unroll 8
-        for (int k = 0; k < B2; ++k) {
-            const T x = sm.R[k * LS + ni];
+            for (int k = 0; k < B2; ++k) {
+                const T x = sm.R[k * LS + ni];
 #pragma unroll
-            for (int u = 0; u < PE; ++u) g[u] = fma(x, sm.R[k * LS + nj + u], g[u]);
+                for (int u = 0; u < PE; ++u) g[u] = fma(x, sm.R[k * LS + nj + u], g[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < PE; ++u) {
+                sm.G[ni * B2 + nj + u] = g[u];
+                if (sizeof(T) == 8) far |= fabs(g[u] - (ni == nj + u ? T(1) : T(0))) > T(1e-9);
+            }
         }
+        if (sizeof(T) == 8) more = __syncthreads_or(far) && more;
+        else __syncthreads();
+        // the rotation is applied in update form, x_j <- x_j + sum_k x_k (R - I)_kj:
+        // once the sweeps have converged R - I is tiny and so is the rounding it
+        // adds, instead of a fresh eps |x| at every application
+        if (t < 256) {
+            T y[PE];
 #pragma unroll
-        for (int u = 0; u < PE; ++u) sm.G[ni * B2 + nj + u] = g[u];
-    }
-    __syncthreads();
-    // the rotation is applied in update form, x_j <- x_j + sum_k x_k (R - I)_kj:
-    // once the sweeps have converged R - I is tiny and so is the rounding it
-    // adds, instead of a fresh eps |x| at every application
-    if (t < 256) {
-        T y[PE];
-#pragma unroll
-        for (int u = 0; u < PE; ++u) y[u] = T(0);
+            for (int u = 0; u < PE; ++u) y[u] = T(0);
 #pragma unroll 8
-        for (int k = 0; k < B2; ++k) {
-            const T x = sm.R[ni * LS + k];
+            for (int k = 0; k < B2; ++k) {
+                const T x = sm.R[ni * LS + k];
 #pragma unroll
-            for (int u = 0; u < PE; ++u) y[u] = fma(x, sm.G[k * B2 + nj + u], y[u]);
-        }
+                for (int u = 0; u < PE; ++u) y[u] = fma(x, sm.G[k * B2 + nj + u], y[u]);
+            }
 #pragma unroll
-        for (int u = 0; u < PE; ++u) {
-            const T rn = fma(T(1.5), sm.R[ni * LS + nj + u], T(-0.5) * y[u]);
-            sm.R4[ni * B2 + nj + u] = rn - (ni == nj + u ? T(1) : T(0));
+            for (int u = 0; u < PE; ++u) {
+                const T rn = fma(T(1.5), sm.R[ni * LS + nj + u], T(-0.5) * y[u]);
+                sm.R4[ni * B2 + nj + u] = rn - (ni == nj + u ? T(1) : T(0));
+            }
         }
+        __syncthreads();
+        if (sizeof(T) == 4 || !more) break;
+        more = false;
+        for (int e = t; e < B2 * B2; e += NT) sm.R[e / B2 * LS + e % B2] = sm.R4[e] + (e / B2 == e % B2 ? T(1) : T(0));
+        __syncthreads();
     }
-    __syncthreads();
 
     // ---- 4. X_P <- X_P R and W_P <- W_P R
     constexpr int OW = 8 * (8 / sizeof(T));       // output columns at a time: 16 floats, 8 doubles
@@ -909,6 +1012,8 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                 cx.scale = warp_max(mx);
                 const T noise = T(4) * num<T>::eps();
                 cx.floor2 = noise * noise * cx.scale + num<T>::tiny();
+                cx.inv_scale = T(1) / (cx.scale + num<T>::tiny());
+                cx.ftau = (float)(cx.tau * sqrt(cx.inv_scale));
             }
         }
         T mine = T(0);
