@@ -77,27 +77,37 @@ struct OsjDesc {
     int64_t ldx, ldw;
     int L, p, pp;
     int strict;         // 1: resolve pairs straddling tau to angle tol (C-step block)
+    // Workspace of the clusterless form (nullptr: not to be used): osj_grid_bytes,
+    // the first osj_grid_head bytes zero before the first launch; *fail is set
+    // to 1 when a wait in it gave up (the results are then void).
+    void* grid;
+    int* fail;
 };
+template <typename T> size_t osj_grid_bytes(int p);
+template <typename T> size_t osj_grid_head(int p);
 
 // Launch shape: CTAs per block's cluster, CTAs per pivot, 512-thread CTAs or
 // not, longest columns and most columns of a block.
 struct OsjShape {
     int cluster, split, wide, max_L, max_p;
+    int grid;           // 1: no cluster, the CTAs of a block meet through global memory
 };
 // the shape for nmat blocks of at most max_p columns and max_L rows; cluster
-// > 0 fixes the largest cluster size to use
+// > 0 fixes the largest cluster size to use; grid: every block has a workspace
+// for the clusterless form
 template <typename T>
-OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster = 0);
+OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster = 0, bool grid = false);
 
 // Schedule of the sweeps (osj.cu); float64 always runs `sorted`.
 enum class OsjMode { kept, sorted };
 
 // One launch: every block is a thread-block cluster that runs its sweeps
 // until converged or `sweeps` are done.  `quad_exit`: stop one sweep early
-// once quadratic convergence guarantees the tolerance (see osj_svd).
+// once quadratic convergence guarantees the tolerance (see osj_svd).  `list`
+// (device): the nmat blocks to run, nullptr for the first nmat.
 template <typename T>
 cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
-                       cudaStream_t s, OsjMode mode, int quad_exit = 0);
+                       cudaStream_t s, OsjMode mode, int quad_exit = 0, const int* list = nullptr);
 // largest cluster size osj_sweeps uses on the current device (16 or 8)
 template <typename T>
 int osj_max_cluster();

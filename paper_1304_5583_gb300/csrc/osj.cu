@@ -64,10 +64,11 @@ namespace {
 // when there are more blocks than that (or columns too long to keep): their
 // phases cover one another's latencies.
 constexpr int NT_MANY = 256, NT_FEW = 512;
-// A Gram is summed in four row slots: of every chunk of 64 rows, slot s has the
-// 16 rows from 16 s.  Each chunk's 16 products are summed on their own and then
-// added to the slot's total; the totals are added in slot order.
-constexpr int NSLOT = 4, SR = 16, CHR = NSLOT * SR;
+// A Gram is summed in row slots: of every chunk of 64 rows, slot s has the SR
+// rows from SR s (float32: 4 slots of 16 rows, each chunk's 16 products summed on
+// their own and then added to the slot's total; float64: 16 of 4).  The slots'
+// totals are added in slot order.
+constexpr int CHR = 64;
 constexpr size_t SMEM_MAX = 227 * 1024;
 
 // Column-block width: float32 16 (pivots of 32 columns).  float64 8: the inner
@@ -75,15 +76,15 @@ constexpr size_t SMEM_MAX = 227 * 1024;
 // a 16-column pivot has an eighth of a 32-column pivot's inner work while a
 // round then has twice as many pivots to spread over the SMs.
 template <typename T> struct Cfg;
-template <> struct Cfg<float> { static constexpr int OB = 16, V = 4, LS = 34; };
-template <> struct Cfg<double> { static constexpr int OB = 8, V = 2, LS = 18; };
+template <> struct Cfg<float> { static constexpr int OB = 16, V = 4, LS = 34, NSLOT = 4, SR = 16; };
+template <> struct Cfg<double> { static constexpr int OB = 8, V = 2, LS = 18, NSLOT = 16, SR = 4; };
 
 template <typename T>
 struct __align__(16) Smem {                       // followed by the stage
     static constexpr int B2 = 2 * Cfg<T>::OB;
     static constexpr int ST = CHR + Cfg<T>::V;    // column stride of a staged chunk (conflict-free 16-byte reads)
     static constexpr int PS = B2 + Cfg<T>::V;     // row stride of a partial Gram
-    static constexpr int PART = NSLOT * B2 * PS;  // the four partial Grams
+    static constexpr int PART = Cfg<T>::NSLOT * B2 * PS;  // the partial Grams
     static constexpr int STAGE = PART + 2 * B2 * ST;
     T S[2][B2 * Cfg<T>::LS];
     T R[B2 * Cfg<T>::LS];
@@ -91,7 +92,7 @@ struct __align__(16) Smem {                       // followed by the stage
     T R4[B2 * B2];                                // R - I, rows of 16-byte multiples
     T red[NT_FEW / 32];
     int cid[B2];                                  // physical column of each pivot column, -1: none
-    int sig[2], rot, cur;
+    int sig[2], rot, cur, fail;
     OsjDesc<T> d;                                 // the block's descriptor (kept out of the registers)
 };
 
@@ -102,13 +103,14 @@ struct __align__(16) Smem {                       // followed by the stage
 // are also read by the other members, so there W has a place of its own.
 constexpr int WROWS = 512;
 // rows of X of a split pivot's member: of every chunk the NSLOT / split slots it owns
+template <typename T>
 __host__ __device__ constexpr int local_rows(int L, int split) {
-    return (L + CHR - 1) / CHR * (NSLOT / split) * SR;
+    return (L + CHR - 1) / CHR * (Cfg<T>::NSLOT / split) * Cfg<T>::SR;
 }
 // column strides of the kept columns: one bank quad past a multiple of 32 words
 template <typename T>
 __host__ __device__ constexpr int panel_stride(int L, int split) {
-    return (local_rows(L, split) + 31) / 32 * 32 + Cfg<T>::V;
+    return (local_rows<T>(L, split) + 31) / 32 * 32 + Cfg<T>::V;
 }
 template <typename T>
 __host__ __device__ constexpr int wpanel_stride(int p, int split) {
@@ -183,7 +185,7 @@ __device__ __forceinline__ unsigned long long key_of(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 }
 
-// part += (16 rows, column by column)^T (the same): lane (ti, tj) of 16 x 2
+// acc += (SR rows, column by column)^T (the same): lane (ti, tj) of 16 x 2
 // holds the entries (ti + 16u, j0 + tj + 2v) of TI x TJ, so that 16-byte reads,
 // each worth V rows of one column, meet no bank twice.
 template <typename T, int TI, int TJ>
@@ -193,9 +195,9 @@ __device__ __forceinline__ void gram_rows(const T* st, int stride, int ti, int j
 #pragma unroll
     for (int u = 0; u < TI; ++u)
 #pragma unroll
-        for (int v = 0; v < TJ; ++v) part[u][v] = T(0);
+        for (int v = 0; v < TJ; ++v) part[u][v] = sizeof(T) == 4 ? T(0) : acc[u][v];
 #pragma unroll
-    for (int q = 0; q < SR; q += V) {
+    for (int q = 0; q < Cfg<T>::SR; q += V) {
         T xi[TI][V];
 #pragma unroll
         for (int u = 0; u < TI; ++u) lds16(st + (ti + 16 * u) * stride + q, xi[u]);
@@ -212,7 +214,7 @@ __device__ __forceinline__ void gram_rows(const T* st, int stride, int ti, int j
 #pragma unroll
     for (int u = 0; u < TI; ++u)
 #pragma unroll
-        for (int v = 0; v < TJ; ++v) acc[u][v] += part[u][v];
+        for (int v = 0; v < TJ; ++v) acc[u][v] = sizeof(T) == 4 ? acc[u][v] + part[u][v] : part[u][v];
 }
 template <typename T, int TI, int TJ>
 __device__ __forceinline__ void put_partial(T* part, int ti, int j0, const T (&acc)[TI][TJ]) {
@@ -224,14 +226,15 @@ __device__ __forceinline__ void put_partial(T* part, int ti, int j0, const T (&a
 
 // 256 threads: the partial Grams from chunks staged by the whole CTA, the next
 // chunk's loads in flight during the products; two warps to a slot, half of
-// the columns each.  (Warps that stage their own rows and columns need no
+// the columns each (float64: two slots to a warp).  (Warps that stage their own rows and columns need no
 // barrier, but three times the shared memory and more registers.)
 template <typename T>
 __device__ __forceinline__ void gram_staged(const Smem<T>& sm, T* stage) {
-    constexpr int B2 = Smem<T>::B2, ST = Smem<T>::ST, TI = B2 / 16, TJ = B2 / 4, PER = B2 * CHR / NT_MANY;
+    constexpr int B2 = Smem<T>::B2, ST = Smem<T>::ST, TI = B2 / 16, PER = B2 * CHR / NT_MANY;
+    constexpr int WPS = sizeof(T) == 4 ? 2 : 1, SPW = sizeof(T) == 4 ? 1 : 2, TJ = B2 / 2 / WPS;   // warps per slot, slots per warp
     const OsjDesc<T>& d = sm.d;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int slot = warp & 3, j0 = (warp >> 2) * (B2 / 2) + (lane >> 4), ti = lane & 15;
+    const int slot = WPS == 2 ? warp & 3 : warp, j0 = (WPS == 2 ? (warp >> 2) * (B2 / 2) : 0) + (lane >> 4), ti = lane & 15;
     T* const buf = stage + Smem<T>::PART;
     const int frow = t % CHR, fcol = t / CHR;
     T pre[PER];
@@ -245,11 +248,13 @@ __device__ __forceinline__ void gram_staged(const Smem<T>& sm, T* stage) {
             pre[u] = (ok && gc >= 0) ? __ldcg(base + (int64_t)gc * d.ldx) : T(0);
         }
     };
-    T acc[TI][TJ];
+    T acc[SPW][TI][TJ];
 #pragma unroll
-    for (int u = 0; u < TI; ++u)
+    for (int w = 0; w < SPW; ++w)
 #pragma unroll
-        for (int v = 0; v < TJ; ++v) acc[u][v] = T(0);
+        for (int u = 0; u < TI; ++u)
+#pragma unroll
+            for (int v = 0; v < TJ; ++v) acc[w][u][v] = T(0);
     const int nch = (d.L + CHR - 1) / CHR;
     fetch(0);
     for (int ch = 0; ch < nch; ++ch) {
@@ -258,9 +263,11 @@ __device__ __forceinline__ void gram_staged(const Smem<T>& sm, T* stage) {
         for (int u = 0; u < PER; ++u) st[(fcol + u * (NT_MANY / CHR)) * ST + frow] = pre[u];
         __syncthreads();      // (the buffer's last readers passed the previous chunk's barrier)
         if (ch + 1 < nch) fetch(ch + 1);
-        gram_rows<T, TI, TJ>(st + slot * SR, ST, ti, j0, acc);
+#pragma unroll
+        for (int w = 0; w < SPW; ++w) gram_rows<T, TI, TJ>(st + (slot + 8 * w) * Cfg<T>::SR, ST, ti, j0, acc[w]);
     }
-    put_partial<T, TI, TJ>(stage + slot * B2 * Smem<T>::PS, ti, j0, acc);
+#pragma unroll
+    for (int w = 0; w < SPW; ++w) put_partial<T, TI, TJ>(stage + (slot + 8 * w) * B2 * Smem<T>::PS, ti, j0, acc[w]);
 }
 
 // what a pivot needs to know of its block (in registers)
@@ -269,17 +276,20 @@ struct PivotCtx {
     T *X, *W;
     int ldx, ldw, L, p;
     T scale, tau, floor2, inv_scale;
-    float ftau;
+    float ftau, ffloor;             // tau and floor2 relative to the scale
     T *stage, *panel, *wpanel;      // stage; kept columns of X and of W (512 threads)
+    T* gpart;                       // clusterless: the team's partial Grams, else nullptr
+    unsigned *team, *gave_up;       // and its arrivals
     int rank, split, member, stride, wstride;
     bool first_round;     // first round of the sweep: pairs inside the column blocks too
 };
 
 // 512 threads: the member's rows of the pivot columns into shared memory, all
 // loads in flight together (an L2 load takes about 0.65 us); rows past L are zero.
-// Local row (c own + j) 16 + i is row 64 c + 16 (member own + j) + i.
+// Local row (c own + j) SR + i is row 64 c + SR (member own + j) + i.
 template <typename T>
 __device__ __forceinline__ int global_row(int lr, int own, int member) {
+    constexpr int SR = Cfg<T>::SR;
     const int g = lr / SR;
     return g / own * CHR + (member * own + g % own) * SR + lr % SR;
 }
@@ -305,14 +315,14 @@ __device__ __forceinline__ void load_panel(const PivotCtx<T>& d, const Smem<T>& 
     }
 }
 
-// 512 threads: partial Grams from the kept columns, four warps to a slot, a
-// quarter of the columns each (a split pivot's member has fewer slots and
-// leaves the other warps out).
-template <typename T>
-__device__ __forceinline__ void gram_kept(const PivotCtx<T>& d, int own) {
-    constexpr int B2 = Smem<T>::B2, TI = B2 / 16, TJ = B2 / 8;
+// 512 threads: the partial Grams of the member's slots from the kept columns into
+// `part`, WPS warps to a slot with their shares of the columns (a split pivot's
+// member has fewer slots and leaves the other warps out).
+template <typename T, int WPS>
+__device__ __forceinline__ void gram_slots(const PivotCtx<T>& d, int own, T* part) {
+    constexpr int B2 = Smem<T>::B2, TI = B2 / 16, TJ = B2 / 2 / WPS;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int j = warp >> 2, j0 = (warp & 3) * (B2 / 4) + (lane >> 4), ti = lane & 15;
+    const int j = warp / WPS, j0 = (warp % WPS) * (B2 / WPS) + (lane >> 4), ti = lane & 15;
     if (j >= own) return;
     T acc[TI][TJ];
 #pragma unroll
@@ -321,8 +331,52 @@ __device__ __forceinline__ void gram_kept(const PivotCtx<T>& d, int own) {
         for (int v = 0; v < TJ; ++v) acc[u][v] = T(0);
     const int nch = (d.L + CHR - 1) / CHR;
 #pragma unroll 1
-    for (int c = 0; c < nch; ++c) gram_rows<T, TI, TJ>(d.panel + (c * own + j) * SR, d.stride, ti, j0, acc);
-    put_partial<T, TI, TJ>(d.stage + j * B2 * Smem<T>::PS, ti, j0, acc);
+    for (int c = 0; c < nch; ++c) gram_rows<T, TI, TJ>(d.panel + (c * own + j) * Cfg<T>::SR, d.stride, ti, j0, acc);
+    put_partial<T, TI, TJ>(part + j * B2 * Smem<T>::PS, ti, j0, acc);
+}
+template <typename T>
+__device__ __forceinline__ void gram_kept(const PivotCtx<T>& d, int own, T* part) {
+    if constexpr (sizeof(T) == 4) {
+        gram_slots<T, 4>(d, own, part);       // (more warps to a slot only read the same columns more often)
+    } else {
+        if (own == 16) gram_slots<T, 1>(d, own, part);
+        else if (own == 8) gram_slots<T, 2>(d, own, part);
+        else if (own == 4) gram_slots<T, 4>(d, own, part);
+        else gram_slots<T, 8>(d, own, part);
+    }
+}
+
+// Clusterless form: the CTAs of a block meet through its workspace, of
+// unsigned integers first (arrivals of the block, CTAs that have left, given up,
+// unused, arrivals of each team), then the partial Grams of every team, twice
+// (a member may be one pivot ahead of the slowest reader).  The launch is
+// cooperative, so the CTAs are all resident; a wait still gives up after some
+// seconds, and with it every other.
+constexpr int GRID_HEAD = 4;
+constexpr int POLLS = 1 << 22;
+__host__ __device__ constexpr size_t grid_head_words(int npairs) { return ((size_t)GRID_HEAD + npairs + 31) / 32 * 32; }
+
+__device__ __forceinline__ unsigned poll(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)) : "memory");
+    return v;
+}
+// all threads of the n CTAs that share `count` (zero before the first meeting)
+__device__ __forceinline__ void meet(unsigned* count, unsigned n, unsigned* gave_up, int& fail) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned before = atomicAdd(count, 1u), target = before - before % n + n;
+        int polls = 0;
+        while ((int)(poll(count) - target) < 0) {
+            if (++polls < POLLS && (polls % 64 != 0 || poll(gave_up) == 0)) continue;
+            atomicExch(gave_up, 1u);
+            fail = 1;
+            break;
+        }
+        __threadfence();
+    }
+    __syncthreads();
 }
 
 // One row of 2b pivot columns times (R - I): x_j <- x_j + sum_k x_k (R - I)_kj,
@@ -556,6 +610,7 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     __syncthreads();
 
     // ---- 1. Gram
+    constexpr int NSLOT = Cfg<T>::NSLOT;
     const int own = NSLOT / split;
     if constexpr (NT == NT_MANY) {
         gram_staged<T>(sm, reinterpret_cast<T*>(&sm + 1));
@@ -563,20 +618,34 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     } else {
         load_panel<T>(cx, sm, own, member);
         __syncthreads();
-        gram_kept<T>(cx, own);
+        const bool shared = split == 1 || !cx.gpart;
+        gram_kept<T>(cx, own, shared ? cx.stage : cx.gpart + member * own * B2 * Smem<T>::PS);
         if (split == 1) __syncthreads();
-        else cl.sync();
+        else if (shared) cl.sync();
+        else meet(cx.team, (unsigned)split, cx.gave_up, sm.fail);
     }
     for (int e = t; e < B2 * B2; e += NT) {
         const int i = e / B2, j = e % B2;
         T p[NSLOT];
+        constexpr int SLOT = B2 * Smem<T>::PS;
+        const int at = i * Smem<T>::PS + j;
+        const T* const mem = cx.gpart + at;
+        const T* const here = reinterpret_cast<T*>(&sm + 1) + at;
+        if (NT == NT_FEW && split > 1 && cx.gpart) {
 #pragma unroll
-        for (int sl = 0; sl < NSLOT; ++sl) {
-            const T* src = reinterpret_cast<T*>(&sm + 1) + (sl % own) * B2 * Smem<T>::PS + i * Smem<T>::PS + j;
-            if (NT == NT_FEW && split > 1) src = cl.map_shared_rank(src, cx.rank - member + sl / own);
-            p[sl] = *src;
+            for (int sl = 0; sl < NSLOT; ++sl) p[sl] = __ldcg(mem + sl * SLOT);
+        } else if (NT == NT_FEW && split > 1) {
+#pragma unroll
+            for (int sl = 0; sl < NSLOT; ++sl)
+                p[sl] = *cl.map_shared_rank(here + (sl % own) * SLOT, cx.rank - member + sl / own);
+        } else {
+#pragma unroll
+            for (int sl = 0; sl < NSLOT; ++sl) p[sl] = here[sl * SLOT];
         }
-        sm.S[0][i * LS + j] = ((p[0] + p[1]) + p[2]) + p[3];
+        T sum = p[0];
+#pragma unroll
+        for (int sl = 1; sl < NSLOT; ++sl) sum += p[sl];
+        sm.S[0][i * LS + j] = sum;
         sm.R[i * LS + j] = (i == j) ? T(1) : T(0);
     }
     __syncthreads();
@@ -599,7 +668,8 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     //      subspace the C step projects onto) also needs that subspace itself:
     //      pairs that straddle tau are measured by t alone.
     const T tau = cx.tau, tau2 = tau * tau;
-    T offm = T(0);
+    using M = std::conditional_t<KEEP, T, float>;
+    M offm = M(0);
     if constexpr (KEEP) {
         const T smax = sqrt(cx.scale);
         const T inv_smax = T(1) / (smax + num<T>::tiny());
@@ -628,9 +698,9 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
             const int j = e % B2, i = e / B2;
             if (i >= j) continue;
             const T sii = sm.S[0][i * LS + i], sjj = sm.S[0][j * LS + j];
-            if (sii > cx.floor2 && sjj > cx.floor2) {
+            const float a2 = (float)(sii * inv_scale), b2 = (float)(sjj * inv_scale);
+            if (a2 > cx.ffloor && b2 > cx.ffloor) {
                 const T sij = fabs(sm.S[0][i * LS + j]);
-                const float a2 = (float)(sii * inv_scale), b2 = (float)(sjj * inv_scale);
                 const float fs = (float)(sij * inv_scale), df = fabsf((float)((sii - sjj) * inv_scale));
                 const float na = sqrtf(a2), nb = sqrtf(b2), gap = df / (na + nb);       // |na - nb|
                 // tangent 2 s / (|a^2 - b^2| + sqrt((a^2 - b^2)^2 + 4 s^2)), scaled against underflow
@@ -645,16 +715,18 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
                 } else if (sii > tau2 && sjj > tau2) mm = tn * gap + ftau * fs / (na * nb);
                 else if (sii > tau2 || sjj > tau2) mm = sm.d.strict ? tn : tn * gap;
                 else mm = tn * (float)((sii + sjj - tau2) * inv_scale) / (sqrtf(a2 + b2) + ftau);
-                offm = fmax(offm, (T)mm);
+                offm = fmaxf(offm, mm);
             }
         }
     }
     offm = warp_max(offm);
-    if (lane == 0) sm.red[warp] = offm;
+    M* const red = reinterpret_cast<M*>(sm.red);
+    if (lane == 0) red[warp] = offm;
     __syncthreads();
-    T mx = T(0);
+    M mxm = M(0);
 #pragma unroll
-    for (int w = 0; w < NW; ++w) mx = fmax(mx, sm.red[w]);
+    for (int w = 0; w < NW; ++w) mxm = fmax(mxm, red[w]);
+    const T mx = (T)mxm;
 
     // two largest diagonal entries of each column block (read by the next
     // rounds' skip test; member 0 writes them)
@@ -792,55 +864,63 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     // ~sqrt(count) eps; one Newton-Schulz step R <- R (3I - R^T R)/2 restores
     // orthogonality to ~eps^2 before R touches X and W (applied to graded
     // columns the defect would mix eps-sized parts of the large columns into
-    // the small ones).  (Float64: R comes from float32 rotations, is orthogonal to
-    // some 1e-6 only and takes a second step unless all angles were tiny.)
+    // the small ones).  Float64: R comes from float32 rotations, with E = I - R^T R
+    // up to some 1e-6, and R (I - E)^(-1/2) is taken to second order, R + R (E / 2 +
+    // 3/8 E^2), which leaves E^3; E^2 in float32 is good to 1e-19.
+    // The rotation is applied in update form, x_j <- x_j + sum_k x_k (R - I)_kj:
+    // once the sweeps have converged R - I is tiny and so is the rounding it
+    // adds, instead of a fresh eps |x| at every application.
     constexpr int PE = B2 * B2 / 256;             // consecutive entries of a row per thread
     const int ni = t * PE / B2, nj = t * PE % B2;
-    for (bool more = sizeof(T) == 8;;) {
-        int far = 0;
-        if (t < 256) {
-            T g[PE];
+    float* const Ef = reinterpret_cast<float*>(sm.S[1]);      // (float64; the rotations' S is done with)
+    if (t < 256) {
+        T g[PE];
 #pragma unroll
-            for (int u = 0; u < PE; ++u) g[u] = T(0);
+        for (int u = 0; u < PE; ++u) g[u] = sizeof(T) == 8 && ni == nj + u ? T(-1) : T(0);
 #pragma unroll 8
-            for (int k = 0; k < B2; ++k) {
-                const T x = sm.R[k * LS + ni];
+        for (int k = 0; k < B2; ++k) {
+            const T x = sm.R[k * LS + ni];
 #pragma unroll
-                for (int u = 0; u < PE; ++u) g[u] = fma(x, sm.R[k * LS + nj + u], g[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < PE; ++u) {
-                sm.G[ni * B2 + nj + u] = g[u];
-                if (sizeof(T) == 8) far |= fabs(g[u] - (ni == nj + u ? T(1) : T(0))) > T(1e-9);
-            }
+            for (int u = 0; u < PE; ++u) g[u] = fma(x, sm.R[k * LS + nj + u], g[u]);
         }
-        if (sizeof(T) == 8) more = __syncthreads_or(far) && more;
-        else __syncthreads();
-        // the rotation is applied in update form, x_j <- x_j + sum_k x_k (R - I)_kj:
-        // once the sweeps have converged R - I is tiny and so is the rounding it
-        // adds, instead of a fresh eps |x| at every application
+#pragma unroll
+        for (int u = 0; u < PE; ++u) {
+            sm.G[ni * B2 + nj + u] = g[u];
+            if (sizeof(T) == 8) Ef[ni * B2 + nj + u] = (float)g[u];
+        }
+    }
+    __syncthreads();
+    if constexpr (sizeof(T) == 8) {
         if (t < 256) {
-            T y[PE];
+            float e2 = 0.f;
 #pragma unroll
-            for (int u = 0; u < PE; ++u) y[u] = T(0);
-#pragma unroll 8
-            for (int k = 0; k < B2; ++k) {
-                const T x = sm.R[ni * LS + k];
-#pragma unroll
-                for (int u = 0; u < PE; ++u) y[u] = fma(x, sm.G[k * B2 + nj + u], y[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < PE; ++u) {
-                const T rn = fma(T(1.5), sm.R[ni * LS + nj + u], T(-0.5) * y[u]);
-                sm.R4[ni * B2 + nj + u] = rn - (ni == nj + u ? T(1) : T(0));
-            }
+            for (int k = 0; k < B2; ++k) e2 = fmaf(Ef[ni * B2 + k], Ef[k * B2 + nj], e2);
+            sm.G[t] = fma(T(-0.5), sm.G[t], (T)(0.375f * e2));
         }
-        __syncthreads();
-        if (sizeof(T) == 4 || !more) break;
-        more = false;
-        for (int e = t; e < B2 * B2; e += NT) sm.R[e / B2 * LS + e % B2] = sm.R4[e] + (e / B2 == e % B2 ? T(1) : T(0));
         __syncthreads();
     }
+    if (t < 256) {
+        T y[PE];
+#pragma unroll
+        for (int u = 0; u < PE; ++u) y[u] = T(0);
+#pragma unroll 8
+        for (int k = 0; k < B2; ++k) {
+            const T x = sm.R[ni * LS + k];
+#pragma unroll
+            for (int u = 0; u < PE; ++u) y[u] = fma(x, sm.G[k * B2 + nj + u], y[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < PE; ++u) {
+            const T rr = sm.R[ni * LS + nj + u], one = ni == nj + u ? T(1) : T(0);
+            if (sizeof(T) == 8) {
+                sm.R4[ni * B2 + nj + u] = (rr - one) + y[u];
+            } else {
+                const T rn = fma(T(1.5), rr, T(-0.5) * y[u]);
+                sm.R4[ni * B2 + nj + u] = rn - one;
+            }
+        }
+    }
+    __syncthreads();
 
     // ---- 4. X_P <- X_P R and W_P <- W_P R
     constexpr int OW = 8 * (8 / sizeof(T));       // output columns at a time: 16 floats, 8 doubles
@@ -878,7 +958,7 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
         // the columns: the tiles of X first, then those of the W rows fetched above
         // (W rows past the first WROWS follow in turn)
         constexpr int RT = sizeof(T) == 4 ? 4 : 1;
-        const int xg = (cx.stride - Cfg<T>::V) / 32, lrows = local_rows(cx.L, split);
+        const int xg = (cx.stride - Cfg<T>::V) / 32, lrows = local_rows<T>(cx.L, split);
         for (int w0 = 0; w0 < wrows || w0 == 0; w0 += WROWS) {
             const int wg = min(wchunks - w0 / 32, WROWS / 32);
             if (t < wg * 32) {
@@ -921,17 +1001,19 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
 // below the tolerance.
 template <typename T, int NT, bool KEEP>
 __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDesc<T>* __restrict__ descs, int sweeps, T tol,
-                                              int* __restrict__ sweeps_run, int quad_exit, int split) {
+                                              int* __restrict__ sweeps_run, int quad_exit, int split, int grid,
+                                              const int* __restrict__ list) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem<T>& sm = *reinterpret_cast<Smem<T>*>(smem_raw);
     constexpr int OB = Cfg<T>::OB, NW = NT / 32;
-    const int mat = blockIdx.y;
+    const int mat = list ? list[blockIdx.y] : (int)blockIdx.y;
     if (threadIdx.x == 0) sm.d = descs[mat];
     __syncthreads();
     const OsjDesc<T>& d = sm.d;
     if (d.active && *d.active == 0) return;     // uniform over the cluster
     cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank(), csize = (int)cl.num_blocks();
+    const bool clusterless = NT == NT_FEW && grid;
+    const int rank = (int)blockIdx.x, csize = (int)gridDim.x;      // (a cluster spans the grid's x)
     const int team = rank / split, nteams = csize / split;
     const int nb = 2 * ((d.p + 2 * OB - 1) / (2 * OB)), npairs = nb / 2;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -951,6 +1033,21 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
         cx.wpanel = split > 1 ? cx.stage + Smem<T>::PART : cx.stage;
         cx.panel = cx.stage + (split > 1 ? Smem<T>::PART + B2 * cx.wstride : max(Smem<T>::PART, B2 * cx.wstride));
     }
+    // clusterless: the workspace
+    unsigned* const head = static_cast<unsigned*>(d.grid);
+    constexpr int GP = Cfg<T>::NSLOT * 2 * OB * Smem<T>::PS;        // a team's partial Grams
+    T* const gparts = clusterless ? reinterpret_cast<T*>(head + grid_head_words(npairs)) + (size_t)team * 2 * GP : nullptr;
+    cx.gpart = gparts;
+    cx.gave_up = head + 2;
+    cx.team = head + GRID_HEAD + team;
+    if (t == 0) sm.fail = clusterless && poll(head + 2) != 0;
+    __syncthreads();
+    if (sm.fail) return;
+    auto sync_block = [&]() {
+        if (clusterless) meet(head, (unsigned)csize, head + 2, sm.fail);
+        else cl.sync();
+    };
+    int flip = 0;
     cx.tau = d.mu ? (T)(1.0 / *d.mu) : T(0);
     // scaled off-diagonals below ~64 eps are at the rounding level of the
     // fresh pivot Grams
@@ -969,9 +1066,9 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                 acc = warp_sum(acc);
                 if (lane == 0) nrm[j] = acc;
             }
-            cl.sync();
+            sync_block();
             // each column's place in the order: how many come before it
-            constexpr int TS = Smem<T>::PART;
+            constexpr int TS = 2 * OB * Smem<T>::PS;
             T* const stage = reinterpret_cast<T*>(&sm + 1);
             for (int jb = rank * NT; !KEEP && jb < d.p; jb += csize * NT) {
                 const int j = jb + t;
@@ -989,7 +1086,8 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                 }
                 if (j < d.p) d.ord[before] = j;
             }
-            if (!KEEP) cl.sync();
+            if (!KEEP) sync_block();
+            if (clusterless && sm.fail) break;                 // (the order may be incomplete)
             // the two largest norms of every column block
             if (rank == 0)
                 for (int b = t; b < nb; b += NT) {
@@ -1004,7 +1102,7 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                     top[(par * nb + b) * 2] = n1;
                     top[(par * nb + b) * 2 + 1] = n2;
                 }
-            cl.sync();
+            sync_block();
             if (sw == 0) {
                 // the largest column: the scale of the measure and of the rounding floor
                 T mx = T(0);
@@ -1014,6 +1112,7 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                 cx.floor2 = noise * noise * cx.scale + num<T>::tiny();
                 cx.inv_scale = T(1) / (cx.scale + num<T>::tiny());
                 cx.ftau = (float)(cx.tau * sqrt(cx.inv_scale));
+                cx.ffloor = (float)(cx.floor2 * cx.inv_scale);
             }
         }
         T mine = T(0);
@@ -1055,22 +1154,33 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                     const int pa = __shfl_sync(0xffffffffu, a, bit), pc = __shfl_sync(0xffffffffu, c, bit);
                     mine = fmax(mine, osj_pivot<T, NT, KEEP>(sm, cl, cx, pa, pc, to + 2 * pa, to + 2 * pc));
                     met = true;
+                    if (clusterless) cx.gpart = gparts + ((flip ^= 1) ? GP : 0);
                 }
             }
-            // a split pivot has one cluster barrier inside; every CTA passes
+            // a split pivot of a cluster has one cluster barrier inside; every CTA passes
             // exactly one per round (a round has at most one pivot per team)
-            if (!met) cl.sync();
-            cl.sync();
+            if (!met && !clusterless) cl.sync();
+            sync_block();
+            if (clusterless && sm.fail) break;
             par ^= 1;
         }
         if (t == 0) {
             atomic_max_nonneg(d.off + sw % 3, mine);
             if (rank == 0) d.off[(sw + 1) % 3] = T(0);
         }
-        cl.sync();
+        sync_block();
+        if (clusterless && sm.fail) break;
         const T o = __ldcg(d.off + sw % 3);
         if (rank == 0 && t == 0 && sweeps_run) sweeps_run[mat] += 1;
         if (o <= t_eff || (quad_exit && T(16) * o * o <= t_eff)) break;
+    }
+    if (clusterless && t == 0) {
+        // the last CTA to leave makes the workspace ready for the next launch
+        if (sm.fail) *d.fail = 1;
+        else if (atomicInc(head + 1, (unsigned)csize - 1) == (unsigned)csize - 1) {
+            head[0] = 0;
+            for (int i = 0; i < npairs; ++i) head[GRID_HEAD + i] = 0;
+        }
     }
 }
 
@@ -1092,33 +1202,48 @@ size_t smem_bytes(const OsjShape& sh) {
 
 template <typename T, int NT, bool KEEP>
 cudaError_t launch(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
-                   cudaStream_t s, int quad_exit, int* resident) {
+                   cudaStream_t s, int quad_exit, const int* list, int* resident) {
     // resident != nullptr: no launch, only how many such clusters fit the device
     static std::atomic<uint64_t> smem_set{0};
-    cudaError_t e = ensure_smem_limit(osj_svd<T, NT, KEEP>, NT == NT_FEW ? (int)SMEM_MAX : (int)smem_bytes<T>(OsjShape{1, 1, 0, 1, 1}),
+    cudaError_t e = ensure_smem_limit(osj_svd<T, NT, KEEP>, NT == NT_FEW ? (int)SMEM_MAX : (int)smem_bytes<T>(OsjShape{1, 1, 0, 1, 1, 0}),
                                       smem_set);
     if (e != cudaSuccess) return e;
-    if (shape.cluster > 8) {
+    if (!shape.grid && shape.cluster > 8) {
         e = cudaFuncSetAttribute(osj_svd<T, NT, KEEP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
+    const bool clusterless = shape.grid != 0;
+    if (clusterless && resident) {
+        int dev = 0, sms = 0, per_sm = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, osj_svd<T, NT, KEEP>, NT, smem_bytes<T>(shape));
+        *resident = per_sm * sms / shape.cluster;
+        return e;
+    }
     cfg.gridDim = dim3((unsigned)shape.cluster, (unsigned)nmat, 1);
     cfg.blockDim = dim3(NT, 1, 1);
     cfg.dynamicSmemBytes = smem_bytes<T>(shape);
     cfg.stream = s;
     cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)shape.cluster; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    if (clusterless) {
+        at.id = cudaLaunchAttributeCooperative;
+        at.val.cooperative = 1;
+    } else {
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)shape.cluster; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    }
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     if (resident) return cudaOccupancyMaxActiveClusters(resident, osj_svd<T, NT, KEEP>, &cfg);
-    e = cudaLaunchKernelEx(&cfg, osj_svd<T, NT, KEEP>, d_desc, sweeps, tol, sweeps_run, quad_exit, shape.split);
+    e = cudaLaunchKernelEx(&cfg, osj_svd<T, NT, KEEP>, d_desc, sweeps, tol, sweeps_run, quad_exit, shape.split, shape.grid, list);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
-// clusters of this shape that fit the current device at once; the runtime's
+// blocks of this shape that fit the current device at once; the runtime's
 // answer (some 10 us a query, and a shape is chosen by a dozen) is kept per
 // device, cluster size, thread count and shared memory
 template <typename T>
@@ -1129,7 +1254,7 @@ int resident_clusters(const OsjShape& sh) {
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     static std::mutex mu;
     static std::map<std::tuple<int, int, int, size_t>, int> known;
-    const auto key = std::make_tuple(dev, sh.cluster, sh.wide, smem);
+    const auto key = std::make_tuple(dev, sh.cluster, sh.wide + 2 * sh.grid, smem);
     {
         std::lock_guard<std::mutex> lock(mu);
         const auto it = known.find(key);
@@ -1137,8 +1262,8 @@ int resident_clusters(const OsjShape& sh) {
     }
     int n = 0;
     // (both schedules use the same shared memory and register limits)
-    const cudaError_t e = sh.wide ? launch<T, NT_FEW, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, &n)
-                                  : launch<T, NT_MANY, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, &n);
+    const cudaError_t e = sh.wide ? launch<T, NT_FEW, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, nullptr, &n)
+                                  : launch<T, NT_MANY, false>(nullptr, 1, sh, 0, T(0), nullptr, nullptr, 0, nullptr, &n);
     if (e != cudaSuccess) n = 0;
     (void)cudaGetLastError();
     std::lock_guard<std::mutex> lock(mu);
@@ -1154,12 +1279,19 @@ int osj_max_cluster() {
     // 16 (the non-portable limit) when the device schedules clusters that
     // large for this kernel, else 8
     static std::atomic<int> big_ok{-1};
-    if (big_ok.load() < 0) big_ok.store(resident_clusters<T>(OsjShape{16, 1, 0, 1, 1}) > 0 ? 1 : 0);
+    if (big_ok.load() < 0) big_ok.store(resident_clusters<T>(OsjShape{16, 1, 0, 1, 1, 0}) > 0 ? 1 : 0);
     return big_ok.load() ? 16 : 8;
 }
 
 template <typename T>
-OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster) {
+size_t osj_grid_head(int p) { return sizeof(unsigned) * grid_head_words(pairs_of<T>(p)); }
+template <typename T>
+size_t osj_grid_bytes(int p) {
+    return osj_grid_head<T>(p) + sizeof(T) * (size_t)pairs_of<T>(p) * 2 * Smem<T>::PART;
+}
+
+template <typename T>
+OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster, bool grid) {
     // Cluster size: the caller's choice (autotuned), else the largest (up to
     // one CTA per pivot of a round) at which every block's cluster can be
     // resident at once -- a block waiting for a second wave would double the
@@ -1173,40 +1305,66 @@ OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster) {
     const int pairs = std::max(1, pairs_of<T>(max_p)), cmax = osj_max_cluster<T>();
     const int limit = cluster > 0 ? std::min(cluster, cmax) : cmax;
     auto fits = [&](const OsjShape& sh) { return resident_clusters<T>(sh) >= nmat; };
+    auto in_cluster = [&]() {
     for (int split = 4; split > 1; split /= 2) {
-        const OsjShape sh{pairs * split, split, 1, max_L, max_p};
+        const OsjShape sh{pairs * split, split, 1, max_L, max_p, 0};
         if (sh.cluster <= limit && split * 64 <= max_L + max_p && fits(sh)) return sh;
     }
     // the largest cluster of each form
     auto largest = [&](int wide) {
         for (int c = std::min(limit, pairs); c > 0; --c) {
-            const OsjShape sh{c, 1, wide, max_L, max_p};
+            const OsjShape sh{c, 1, wide, max_L, max_p, 0};
             if (fits(sh) || (!wide && cluster > 0)) return sh;
         }
-        return OsjShape{wide ? 0 : 1, 1, wide, max_L, max_p};
+        return OsjShape{wide ? 0 : 1, 1, wide, max_L, max_p, 0};
     };
     const OsjShape wide = largest(1), streamed = largest(0);
     if (wide.cluster > 0 && ceil_div(pairs, wide.cluster) <= 2 * ceil_div(pairs, streamed.cluster)) return wide;
     return streamed;
+    };
+    OsjShape best = in_cluster();
+    if (!grid || cluster > 0) return best;
+    // Without a cluster the CTAs of a block may lie anywhere, and there may be more
+    // than 16.  The estimate, in us a round: a pivot takes about 17 whatever its
+    // size (measure, inner rotations, R) and its Gram and update by the rate
+    // measured on one SM, over the CTAs that share it; a meeting through memory
+    // costs 2 to 3 more than a cluster barrier, and a split pivot has one inside.
+    // (Whole pivots gain nothing: 10 blocks of 11, as clusters of 10 or so, 172 and
+    // 175 ms in the 500 x 5000 solve.)  The 1000 x 487 float32 SVT, 64 CTAs for 16,
+    // went from 16.5 to 12 ms; the 100 x 500 float64 one, 112 for 14, from 8 to 4.
+    const double b2 = 2.0 * Cfg<T>::OB, work = (2.0 * max_L + max_p) * b2 * b2 / (sizeof(T) == 4 ? 110e3 : 3.7e3);
+    auto cost = [&](const OsjShape& sh) {
+        const int turns = (int)ceil_div((int64_t)pairs * sh.split, sh.cluster);
+        return turns * (17.0 + work / sh.split) * (sh.wide ? 1.0 : 2.0) + (sh.grid ? 5.0 : 0.0);
+    };
+    auto consider = [&](const OsjShape& sh) {
+        if (fits(sh) && cost(sh) < cost(best)) best = sh;
+    };
+    for (int split = Cfg<T>::NSLOT; split > 1; split /= 2) consider({pairs * split, split, 1, max_L, max_p, 1});
+    return best;
 }
 
 template <typename T>
 cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
-                       cudaStream_t s, OsjMode mode, int quad_exit) {
+                       cudaStream_t s, OsjMode mode, int quad_exit, const int* list) {
     if (nmat <= 0 || sweeps <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 4) {
         if (mode == OsjMode::kept)
-            return shape.wide ? launch<T, NT_FEW, true>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr)
-                              : launch<T, NT_MANY, true>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr);
+            return shape.wide ? launch<T, NT_FEW, true>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, list, nullptr)
+                              : launch<T, NT_MANY, true>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, list, nullptr);
     }
-    return shape.wide ? launch<T, NT_FEW, false>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr)
-                      : launch<T, NT_MANY, false>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, nullptr);
+    return shape.wide ? launch<T, NT_FEW, false>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, list, nullptr)
+                      : launch<T, NT_MANY, false>(d_desc, nmat, shape, sweeps, tol, sweeps_run, s, quad_exit, list, nullptr);
 }
 
-template cudaError_t osj_sweeps<float>(const OsjDesc<float>*, int, OsjShape, int, float, int*, cudaStream_t, OsjMode, int);
-template cudaError_t osj_sweeps<double>(const OsjDesc<double>*, int, OsjShape, int, double, int*, cudaStream_t, OsjMode, int);
-template OsjShape osj_shape<float>(int, int, int, int);
-template OsjShape osj_shape<double>(int, int, int, int);
+template cudaError_t osj_sweeps<float>(const OsjDesc<float>*, int, OsjShape, int, float, int*, cudaStream_t, OsjMode, int, const int*);
+template cudaError_t osj_sweeps<double>(const OsjDesc<double>*, int, OsjShape, int, double, int*, cudaStream_t, OsjMode, int, const int*);
+template OsjShape osj_shape<float>(int, int, int, int, bool);
+template OsjShape osj_shape<double>(int, int, int, int, bool);
+template size_t osj_grid_head<float>(int);
+template size_t osj_grid_head<double>(int);
+template size_t osj_grid_bytes<float>(int);
+template size_t osj_grid_bytes<double>(int);
 template int osj_max_cluster<float>();
 template int osj_max_cluster<double>();
 

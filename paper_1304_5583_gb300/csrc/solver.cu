@@ -370,7 +370,7 @@ struct GemmSet {
 // Graphs of iteration chunks, recorded on a stream of their own; they and the
 // stream end with the solve.
 struct ChunkGraphs {
-    using Key = std::tuple<int, bool, bool, int, int, int>;
+    using Key = std::tuple<int, bool, bool, int, int, int, int>;
     struct Entry {
         cudaGraphExec_t exec = nullptr;
         int64_t launches = 0, calls[LRR_NPHASE] = {};
@@ -439,6 +439,16 @@ bool use_tc32(const lrr_problem* p, const lrr_options* o) {
     return std::is_same<T, float>::value && o->precision != LRR_PREC_F64 && o->tc_products && p->n <= kTcMaxN;
 }
 
+// Workspaces of the Jacobi's clusterless form (osj.cu), one per block, after an
+// integer that a wait which gave up sets and the list of the active blocks.  They come after everything else: a caller's
+// workspace of the size without them is taken too, and the form then left out.
+template <typename T>
+size_t jgrid_bytes(const std::vector<BlockInfo<T>>& blk) {
+    size_t n = 3 * kAlign + sizeof(int) * blk.size();
+    for (const auto& b : blk) n += (osj_grid_bytes<T>(b.pmax) + kAlign - 1) / kAlign * kAlign;
+    return n;
+}
+
 template <typename T, typename Tin>
 int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_bytes, lrr_result* res,
                cudaStream_t s, bool dfc) {
@@ -451,10 +461,11 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     carve<T>(probe, p, need_md, blk, mixed, tc32);
     const size_t need = probe.off + kAlign;
     void* own = nullptr;
+    const size_t grid_bytes = jgrid_bytes<T>(blk);
     if (!ws) {
-        if (scratch_alloc(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
+        if (scratch_alloc(&own, need + grid_bytes, s) != cudaSuccess) return LRR_ERR_CUDA;
         ws = own;
-        ws_bytes = need;
+        ws_bytes = need + grid_bytes;
     }
     struct Free {
         void* p; cudaStream_t s;
@@ -463,6 +474,8 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     if (ws_bytes < need - kAlign || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0) return LRR_ERR_WORKSPACE;
     Arena arena(ws);
     Buffers<T> B = carve<T>(arena, p, need_md, blk, mixed, tc32);
+    char* const jgrid = ws_bytes >= need + grid_bytes ? arena.take<char>(grid_bytes) : nullptr;
+    if (jgrid) LRR_CUDA_TRY(cudaMemsetAsync(jgrid, 0, grid_bytes, s));
     const int64_t m = p->m, n = p->n;
     const int t = p->t;
     const Tin* M = static_cast<const Tin*>(p->M);
@@ -668,6 +681,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     LRR_CUDA_TRY(cudaMemcpyAsync(B.ppv, ppv.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
     std::vector<OsjDesc<T>> jdh((size_t)t);
     int64_t cols_off = 0;
+    size_t grid_off = kAlign + (sizeof(int) * t + kAlign - 1) / kAlign * kAlign;
     for (int i = 0; i < t; ++i) {
         OsjDesc<T>& j = jdh[i];
         j.X = B.D + blk[i].col0 * r;
@@ -679,6 +693,9 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         cols_off += blk[i].ppmax;
         j.mu = B.mu + i;
         j.strict = (dfc && t > 1 && i == 0) ? 1 : 0;
+        j.grid = jgrid ? jgrid + grid_off : nullptr;
+        j.fail = reinterpret_cast<int*>(jgrid);
+        grid_off += (osj_grid_bytes<T>(blk[i].pmax) + kAlign - 1) / kAlign * kAlign;
     }
     LRR_CUDA_TRY(cudaMemcpyAsync(B.jd, jdh.data(), sizeof(OsjDesc<T>) * t, cudaMemcpyHostToDevice, s));
     // the float32 Jacobi stops without its confirming sweep once quadratic
@@ -700,7 +717,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         }
         if (!have) {
             std::vector<int> cand;
-            for (int c : {4, 8, 16})
+            for (int c : {0, 4, 8, 16})         // 0: osj_shape's own choice
                 if (c <= osj_max_cluster<T>()) cand.push_back(c);
             std::vector<int> on((size_t)t, 1);
             std::vector<double> mu_t((size_t)t, 1e10);
@@ -715,7 +732,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
                 for (int i = 0; i < t; ++i)
                     k::init_padded<T><<<grid1((int64_t)ppv[i] * ppv[i]), 256, 0, s>>>(B.W[i], pv[i], ppv[i], T(1), 1);
                 cudaEventRecord(ta, s);
-                const cudaError_t e = osj_sweeps<T>(B.jd, t, osj_shape<T>(t, max_p, max_L, c), 2, jtol_of<T>(), nullptr, s,
+                const cudaError_t e = osj_sweeps<T>(B.jd, t, osj_shape<T>(t, max_p, max_L, c, jgrid != nullptr), 2, jtol_of<T>(), nullptr, s,
                                                     OsjMode::kept, quad_exit);
                 cudaEventRecord(tb, s);
                 if (e != cudaSuccess || cudaEventSynchronize(tb) != cudaSuccess) {
@@ -735,7 +752,9 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     // launch shape of the Jacobi for the blocks still active (the others' clusters
     // leave at once); re-picked as blocks converge
     int jshape_n = t;
-    OsjShape jshape = osj_shape<T>(t, max_p, max_L, jcluster);
+    int* const jlist = reinterpret_cast<int*>(jgrid ? jgrid + kAlign : nullptr);
+    std::vector<int> jact;
+    OsjShape jshape = osj_shape<T>(t, max_p, max_L, jcluster, jgrid != nullptr);
 
     // grouped GEMM descriptor sets
     std::vector<GemmDesc<T>> gh;
@@ -862,7 +881,8 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         LRR_CUDA_TRY(run_set(S_XW));
         prof.end(LRR_PH_GRAM, 1 + nl(S_XT) + nl(S_XW));
         prof.begin();
-        LRR_CUDA_TRY(osj_sweeps<T>(B.jd, t, jshape, sweeps, jtol, B.jsweeps, q, OsjMode::kept, quad_exit));
+        LRR_CUDA_TRY(osj_sweeps<T>(B.jd, jshape.grid ? jshape_n : t, jshape, sweeps, jtol, B.jsweeps, q, OsjMode::kept, quad_exit,
+                                   jshape.grid ? jlist : nullptr));
         prof.end(LRR_PH_JACOBI, 1);
         prof.begin();
         k::svt_weights<T><<<dim3((unsigned)t, ceil_div(max_pp, k::kWeightCols)), 256, 0, q>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
@@ -945,7 +965,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     // per-phase events the launches are issued one by one.
     ChunkGraphs graphs;
     auto run_chunk = [&](int len) -> int {
-        const auto key = std::make_tuple(len, bf16_phase, tc_window, jshape.cluster, jshape.split, jshape.wide);
+        const auto key = std::make_tuple(len, bf16_phase, tc_window, jshape.cluster, jshape.split, jshape.wide, jshape.grid ? jshape_n : 0);
         ChunkGraphs::Entry* e = prof.on ? nullptr : graphs.find(key);
         // (the second time a set comes up: every kernel is loaded by then)
         if (!prof.on && !e && graphs.again(key) && graphs.begin()) {
@@ -983,13 +1003,24 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         std::vector<int> ah((size_t)t), fh((size_t)t);
         int done_it = 0, nneed = 0;
         const int chunk = 4;
-        auto pick_shape = [&](const std::vector<int>& act) {
+        auto pick_shape = [&](const std::vector<int>& act) -> cudaError_t {
             const int na = (int)std::count_if(act.begin(), act.end(), [](int v) { return v != 0; });
-            if (na == 0 || na == jshape_n) return;
+            if (na == 0) return cudaSuccess;
+            if (jgrid && act != jact) {
+                // (a clusterless launch is made of the active blocks only: all of it must be resident)
+                std::vector<int> ids;
+                for (int i = 0; i < t; ++i)
+                    if (act[i]) ids.push_back(i);
+                const cudaError_t e = cudaMemcpyAsync(jlist, ids.data(), sizeof(int) * na, cudaMemcpyHostToDevice, s);
+                if (e != cudaSuccess) return e;
+                jact = act;
+            }
+            if (na == jshape_n) return cudaSuccess;
             jshape_n = na;
-            jshape = osj_shape<T>(na, max_p, max_L, na == t ? jcluster : 0);
+            jshape = osj_shape<T>(na, max_p, max_L, na == t ? jcluster : 0, jgrid != nullptr);
+            return cudaSuccess;
         };
-        pick_shape(act0);
+        LRR_CUDA_TRY(pick_shape(act0));
         tc_window = false;
         while (done_it < o->max_iter) {
             const int len = std::min(chunk, o->max_iter - done_it);
@@ -1013,7 +1044,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
                 if (!any16) bf16_phase = false;
             }
             if (std::none_of(ah.begin(), ah.end(), [](int v) { return v != 0; })) break;
-            pick_shape(ah);
+            LRR_CUDA_TRY(pick_shape(ah));
         }
         return LRR_OK;
     };
@@ -1029,6 +1060,12 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         }
     }
     LRR_CUDA_TRY(cudaEventRecord(ev[2], s));
+    if (jgrid) {
+        int fail = 0;
+        LRR_CUDA_TRY(cudaMemcpyAsync(&fail, jgrid, sizeof(int), cudaMemcpyDeviceToHost, s));
+        LRR_CUDA_TRY(cudaStreamSynchronize(s));
+        if (fail) return LRR_ERR_CUDA;
+    }
 
     // ---- C step
     int k1 = 0;
@@ -1184,7 +1221,7 @@ template <typename T>
 struct SvtParams {
     double mu;
     T *W, *H, *h, *T1;            // pointer tables of one entry each
-    int act, on, rank, sweeps, p, pp;
+    int act, on, rank, fail, sweeps, p, pp;
     T off[3];
     OsjDesc<T> od;
     GemmDesc<T> g[3];
@@ -1194,13 +1231,15 @@ template <typename T>
 struct SvtScratch {
     T *X, *W, *H, *T1, *h;
     SvtParams<T>* par;
-    SvtScratch(Arena& a, int L, int p, int pp) {
+    char* grid = nullptr;
+    SvtScratch(Arena& a, int L, int p, int pp, bool with_grid) {
         X = a.take<T>((size_t)L * p);
         W = a.take<T>((size_t)pp * pp);
         H = a.take<T>((size_t)pp * pp);
         T1 = a.take<T>((size_t)pp * pp);
         h = a.take<T>(pp);
         par = a.take<SvtParams<T>>(1);
+        if (with_grid) grid = a.take<char>(osj_grid_bytes<T>(p));
     }
 };
 
@@ -1208,7 +1247,8 @@ struct SvtScratch {
 // and the parameter block; one thread block per 32 x 32 tile of X.
 template <typename T>
 __global__ void svt_begin(const T* __restrict__ A, int64_t lda, int L, int p, int pp, int tall, T* __restrict__ X,
-                          T* __restrict__ W, const SvtParams<T> par, SvtParams<T>* __restrict__ dst) {
+                          T* __restrict__ W, const SvtParams<T> par, SvtParams<T>* __restrict__ dst, unsigned* __restrict__ zero,
+                          int nzero) {
     __shared__ T tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int64_t tiles_r = (L + 31) / 32, ntile = tiles_r * ((p + 31) / 32);
@@ -1228,7 +1268,10 @@ __global__ void svt_begin(const T* __restrict__ A, int64_t lda, int L, int p, in
     }
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)pp * pp; e += (int64_t)gridDim.x * blockDim.x)
         W[e] = e % pp == e / pp ? T(1) : T(0);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *dst = par;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) *dst = par;
+        for (int i = threadIdx.x; i < nzero; i += blockDim.x) zero[i] = 0;
+    }
 }
 
 // Stand-alone singular-value thresholding with the solver's own SVT kernels
@@ -1248,15 +1291,17 @@ int svt_run(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* 
     par.od.cols = q.T1;                   // T1 and H are written only after the Jacobi: its scratch until then
     par.od.ord = reinterpret_cast<int*>(q.H);
     par.od.ldx = L; par.od.ldw = pp; par.od.L = L; par.od.p = p; par.od.pp = pp; par.od.strict = 1;
+    par.od.grid = q.grid; par.od.fail = &d->fail;
     par.g[0] = gdesc<T>(q.W, pp, q.W, pp, q.T1, pp, p, p, p, nullptr);                   // W^T W
     par.g[1] = gdesc<T>(q.W, pp, q.T1, pp, q.H, pp, p, p, p, nullptr);                   // W (W^T W)
     if (tall) par.g[2] = gdesc<T>(q.X, L, q.T1, pp, J, ldj, (int)rows, (int)cols, p, nullptr);   // J = X h W^{-1}
     else par.g[2] = gdesc<T>(q.T1, pp, q.X, L, J, ldj, (int)rows, (int)cols, p, nullptr);        // J = W^{-T} h X^T
     par.g[2].kscale = q.h;
     const int64_t tiles = (int64_t)((L + 31) / 32) * ((p + 31) / 32);
-    svt_begin<T><<<(unsigned)std::min<int64_t>(tiles, 152 * 8), 256, 0, s>>>(A, lda, L, p, pp, tall ? 1 : 0, q.X, q.W, par, d);
+    svt_begin<T><<<(unsigned)std::min<int64_t>(tiles, 152 * 8), 256, 0, s>>>(A, lda, L, p, pp, tall ? 1 : 0, q.X, q.W, par, d,
+        reinterpret_cast<unsigned*>(q.grid), q.grid ? (int)(osj_grid_head<T>(p) / sizeof(unsigned)) : 0);
     LRR_CUDA_TRY(cudaGetLastError());
-    LRR_CUDA_TRY(osj_sweeps<T>(&d->od, 1, osj_shape<T>(1, p, L), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), &d->sweeps, s,
+    LRR_CUDA_TRY(osj_sweeps<T>(&d->od, 1, osj_shape<T>(1, p, L, 0, q.grid != nullptr), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), &d->sweeps, s,
                                OsjMode::sorted));
     k::svt_weights<T><<<dim3(1, (unsigned)ceil_div(pp, k::kWeightCols)), 256, 0, s>>>(&d->od, &d->h, &d->act, &d->on,
                                                                                      &d->mu, &d->rank, 1);
@@ -1264,10 +1309,12 @@ int svt_run(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* 
     LRR_CUDA_TRY(gemm_grouped<T>(&d->g[1], 1, false, false, p, p, s));
     k::ns_orth<T><<<dim3(64, 1), 256, 0, s>>>(&d->W, &d->H, &d->T1, &d->p, &d->pp, &d->on, 1);
     LRR_CUDA_TRY(gemm_grouped<T>(&d->g[2], 1, false, true, (int)rows, (int)cols, s));
-    int rk_h = 0;
-    LRR_CUDA_TRY(cudaMemcpyAsync(&rk_h, &d->rank, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int rank_fail[2] = {0, 0};
+    static_assert(offsetof(SvtParams<T>, fail) == offsetof(SvtParams<T>, rank) + sizeof(int), "copied together");
+    LRR_CUDA_TRY(cudaMemcpyAsync(rank_fail, &d->rank, sizeof(rank_fail), cudaMemcpyDeviceToHost, s));
     LRR_CUDA_TRY(cudaStreamSynchronize(s));
-    if (rank_out) *rank_out = rk_h;
+    if (rank_fail[1]) return LRR_ERR_CUDA;
+    if (rank_out) *rank_out = rank_fail[0];
     return LRR_OK;
 }
 
@@ -1277,7 +1324,7 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
              cudaStream_t s) {
     const int p = (int)std::min(rows, cols), L = (int)std::max(rows, cols), pp = round_up(p, osj_pivot_width());
     Arena sz(nullptr);
-    SvtScratch<T>(sz, L, p, pp);
+    SvtScratch<T>(sz, L, p, pp, true);
     void* mem = nullptr;
     if (scratch_alloc(&mem, sz.off + kAlign, s) != cudaSuccess) return LRR_ERR_CUDA;
     struct Free {
@@ -1285,7 +1332,7 @@ int svt_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T*
         ~Free() { if (p) cudaFreeAsync(p, s); }
     } guard{mem, s};
     Arena a(mem);
-    return svt_run<T>(A, rows, cols, lda, tau, J, ldj, rank_out, s, SvtScratch<T>(a, L, p, pp));
+    return svt_run<T>(A, rows, cols, lda, tau, J, ldj, rank_out, s, SvtScratch<T>(a, L, p, pp, true));
 }
 
 // ---------------------------------------------------------------------------
@@ -1323,12 +1370,14 @@ int svt_noalloc_impl(const T* A, int64_t rows, int64_t cols, int64_t lda, double
                      int32_t* rank_out, cudaStream_t s) {
     const int p = (int)std::min(rows, cols), L = (int)std::max(rows, cols), pp = round_up(p, osj_pivot_width());
     Arena sz(nullptr);
-    SvtScratch<T>(sz, L, p, pp);
+    SvtScratch<T>(sz, L, p, pp, false);
     if (sz.off > kNoAllocScratchBytes) return LRR_ERR_TOO_LARGE;
+    Arena with_grid(nullptr);
+    SvtScratch<T>(with_grid, L, p, pp, true);
     void* base = svt_scratch_address();
     if (!base) return LRR_ERR_CUDA;
     Arena a(base);
-    return svt_run<T>(A, rows, cols, lda, tau, J, ldj, rank_out, s, SvtScratch<T>(a, L, p, pp));
+    return svt_run<T>(A, rows, cols, lda, tau, J, ldj, rank_out, s, SvtScratch<T>(a, L, p, pp, with_grid.off <= kNoAllocScratchBytes));
 }
 
 template <typename T, typename Tin>
@@ -1336,7 +1385,7 @@ size_t workspace_impl(const lrr_problem* p, const lrr_options* o, bool mixed) {
     const auto blk = block_info<T>(p);
     Arena probe(nullptr);
     carve<T>(probe, p, !std::is_same<Tin, double>::value, blk, mixed, use_tc32<T>(p, o));
-    return probe.off + kAlign;
+    return probe.off + kAlign + jgrid_bytes<T>(blk);
 }
 
 // The problem with a NULL perm / offsets replaced by the D step's defaults

@@ -215,6 +215,7 @@ struct Engine {
     T *ocols, *ooff;
     int *oord, *oon;
     OsjShape oshape;
+    char* ogrid = nullptr;       // the Jacobi's clusterless workspace, after an integer a wait that gave up sets
     T **pW, **pH, **pT;
     int *pv, *ppv;
     GemmDesc<T>* gd;
@@ -570,7 +571,9 @@ int engine_init(Engine<T>& g) {
     // singular pair resolved, including the ones the SVT removes
     d.mu = nullptr;
     d.ldx = g.n; d.ldw = g.pp; d.L = (int)g.n; d.p = g.r; d.pp = g.pp; d.strict = 1;
-    g.oshape = osj_shape<T>(1, g.r, (int)g.n);
+    d.grid = g.ogrid ? g.ogrid + kAl : nullptr;
+    d.fail = reinterpret_cast<int*>(g.ogrid);
+    g.oshape = osj_shape<T>(1, g.r, (int)g.n, 0, g.ogrid != nullptr);
     UTRY(cudaMemcpyAsync(g.od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     T* ptrs[3] = {g.Wj, g.Wg, g.Wt};
     UTRY(cudaMemcpyAsync(g.pW, &ptrs[0], sizeof(T*), cudaMemcpyHostToDevice, s));
@@ -617,7 +620,7 @@ size_t unrolled_ws(int64_t m, int64_t n, const lrr_unrolled_options* o, bool gra
     Engine<T> g = make_engine<T>(nullptr, m, n, std::max<int64_t>(m, 1), o, grad);
     if (!grad) g.cp = 0;
     Bump b(nullptr);
-    return carve_engine<T>(g, b);
+    return carve_engine<T>(g, b) + 2 * kAl + osj_grid_bytes<T>(g.r);
 }
 
 template <typename T>
@@ -631,10 +634,12 @@ int unrolled_run(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unr
     Bump probe(nullptr);
     const size_t need = carve_engine<T>(g, probe);
     void* own = nullptr;
+    // (after everything else: a caller's workspace of the size without it is taken too)
+    const size_t grid_bytes = 2 * kAl + osj_grid_bytes<T>(g.r);
     if (!ws) {
-        if (scratch_alloc(&own, need, s) != cudaSuccess) return LRR_ERR_CUDA;
+        if (scratch_alloc(&own, need + grid_bytes, s) != cudaSuccess) return LRR_ERR_CUDA;
         ws = own;
-        wsb = need;
+        wsb = need + grid_bytes;
     }
     struct Free {
         void* p; cudaStream_t s;
@@ -643,6 +648,10 @@ int unrolled_run(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unr
     if (wsb < need - kAl || (reinterpret_cast<uintptr_t>(ws) % kAl) != 0) return LRR_ERR_WORKSPACE;
     Bump b(ws);
     carve_engine<T>(g, b);
+    if (wsb >= need + grid_bytes) {
+        g.ogrid = b.take<char>(grid_bytes);
+        UTRY(cudaMemsetAsync(g.ogrid, 0, grid_bytes, s));
+    }
     int rc = setup<T>(g, o->rank_tol > 0 ? o->rank_tol : 1e-6);
     if (rc != LRR_OK) return rc;
     rc = engine_init<T>(g);
@@ -689,8 +698,10 @@ int unrolled_run(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unr
         UTRY(cudaStreamSynchronize(s));
         if (lambar) *lambar = lb;
     }
+    int fail = 0;
+    if (g.ogrid) UTRY(cudaMemcpyAsync(&fail, g.ogrid, sizeof(int), cudaMemcpyDeviceToHost, s));
     UTRY(cudaStreamSynchronize(s));
-    return LRR_OK;
+    return fail ? LRR_ERR_CUDA : LRR_OK;
 }
 
 }  // namespace
