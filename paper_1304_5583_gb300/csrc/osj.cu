@@ -754,22 +754,26 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
         return mx;
     }
 
-    // 512 threads: the first rows of W are fetched while the pivot rotates (split
-    // members take alternate chunks)
+    // 512 threads: the first rows of W are copied to shared memory while the pivot
+    // rotates (split members take alternate 32-row groups), as 16-byte asynchronous
+    // copies: through registers, 32 a thread, the copy and its spills took 2.3 us.
+    // (Rows past p of the last group are read, W being padded, and not used.)
     const int wchunks = ((cx.p + 31) / 32 - member + split - 1) / split, wrows = wchunks * 32;
     auto wrow = [&](int lw) { return ((lw / 32) * split + member) * 32 + lw % 32; };
-    T wx[NT == NT_FEW ? B2 : 1];
-    auto load_w = [&](int row) {
+    auto fetch_w = [&](int w0) {
         if constexpr (NT == NT_FEW) {
-            const T* const base = cx.W + row;
-#pragma unroll
-            for (int k = 0; k < B2; ++k) {
-                const int gc = sm.cid[k];
-                wx[k] = (row < cx.p && gc >= 0) ? __ldcg(base + (int64_t)gc * cx.ldw) : T(0);
-            }
+            constexpr int V = Cfg<T>::V, PER = 32 / V;
+            static_assert(PER * B2 == 256, "256 copies to a group of 32 rows");
+            const int wg = min(wchunks - w0 / 32, WROWS / 32), k = (t & 255) / PER, v = (t & 255) % PER * V;
+            const int gc = sm.cid[k];
+            const T* const src = cx.W + (int64_t)max(gc, 0) * cx.ldw + v;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(cx.wpanel + k * cx.wstride + v);
+            for (int g = t >> 8; g < wg; g += NT / 256)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + g * 32 * (unsigned)sizeof(T)),
+                             "l"(__cvta_generic_to_global(src + wrow(w0 + g * 32))), "r"(gc >= 0 ? 16 : 0) : "memory");
         }
     };
-    if (t < wrows) load_w(wrow(t));
+    fetch_w(0);
 
     // ---- 3. rotate the pivot Gram towards diagonal form.  Thread (k, l) of
     //      b x b owns the 2 x 2 sub-block of pairs k and l: it reads the old S,
@@ -856,6 +860,7 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     if (sizeof(T) == 4) Sd = sm.S[sm.cur];
     tops();
     if (!sm.rot) {
+        asm volatile("cp.async.wait_all;" ::: "memory");      // (W's place is the next pivot's stage)
         __syncthreads();
         return mx;
     }
@@ -961,11 +966,8 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
         const int xg = (cx.stride - Cfg<T>::V) / 32, lrows = local_rows<T>(cx.L, split);
         for (int w0 = 0; w0 < wrows || w0 == 0; w0 += WROWS) {
             const int wg = min(wchunks - w0 / 32, WROWS / 32);
-            if (t < wg * 32) {
-                if (w0 > 0) load_w(wrow(w0 + t));
-#pragma unroll
-                for (int k = 0; k < B2; ++k) cx.wpanel[k * cx.wstride + t] = wx[k];
-            }
+            if (w0 > 0) fetch_w(w0);
+            asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
             const int xt = w0 == 0 ? (xg + RT - 1) / RT : 0, wt = (wg + RT - 1) / RT;
             for (int tile = warp; tile < 2 * (xt + wt); tile += NT / 32) {
