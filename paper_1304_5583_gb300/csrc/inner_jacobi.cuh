@@ -11,6 +11,17 @@ __device__ __forceinline__ int circle_item(int pos, int r, int N) {
     return pos == 0 ? 0 : 1 + ((pos - 1 + r) % (N - 1));
 }
 
+// off > eps sqrt(g) exactly (g >= 0): the rounded root, some 40 dependent cycles and
+// a branch of its own, only where the hardware's approximation does not decide
+__device__ __forceinline__ bool above_eps_root(float off, float g) {
+    const bool low = g < 1e-30f;             // (subnormal products are common: scaled, exactly)
+    float q;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(low ? g * 0x1p100f : g));
+    const float bound = (low ? 0x1p-50f * FLT_EPSILON : FLT_EPSILON) * q;
+    if (off > 1.0001f * bound || off < 0.9999f * bound) return off > bound;
+    return off > FLT_EPSILON * sqrtf(g);
+}
+
 // Rotation (c, s) that annihilates s_pq: tan(2 theta) = 2 s_pq / (s_qq - s_pp),
 // the tangent's root of smaller magnitude.
 template <typename T>

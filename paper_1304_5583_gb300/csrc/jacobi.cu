@@ -40,15 +40,14 @@ __device__ int inner_sweep_f32(float (*S2)[B2 * LS], float* R, float floor_rot, 
     static_assert(b == 32 && solve_threads<float>() == b * b, "a warp holds every pair's rotation");
     const int k = threadIdx.x % b, l = threadIdx.x / b;
     int rotated = 0, cur = 0;
+    int p = k, q = B2 - 1 - k, u = l, v = B2 - 1 - l;       // the circle method's round 0
     for (int r = 0; r < B2 - 1; ++r) {
-        const int p = circle_item(k, r, B2), q = circle_item(B2 - 1 - k, r, B2);
-        const int u = circle_item(l, r, B2), v = circle_item(B2 - 1 - l, r, B2);
         const float* const S = S2[cur];
         float* const D = S2[cur ^ 1];
         const float app = S[p * LS + p], aqq = S[q * LS + q], apq = S[p * LS + q];
         const float s_pu = S[p * LS + u], s_pv = S[p * LS + v], s_qu = S[q * LS + u], s_qv = S[q * LS + v];
         const float x0 = R[k * LS + u], y0 = R[k * LS + v], x1 = R[(k + b) * LS + u], y1 = R[(k + b) * LS + v];
-        const bool act = fabsf(apq) > floor_rot && fabsf(apq) > FLT_EPSILON * sqrtf(fabsf(app * aqq));
+        const bool act = fabsf(apq) > floor_rot && above_eps_root(fabsf(apq), fabsf(app * aqq));
         float ck, sk;
         jacobi_rotation<float>(app, aqq, apq, ck, sk);
         ck = act ? ck : 1.f;
@@ -68,6 +67,10 @@ __device__ int inner_sweep_f32(float (*S2)[B2 * LS], float* R, float floor_rot, 
         R[(k + b) * LS + u] = fmaf(cl, x1, -(sl * y1));
         R[(k + b) * LS + v] = fmaf(sl, x1, cl * y1);
         cur ^= 1;
+        p = k ? (p == B2 - 1 ? 1 : p + 1) : 0;
+        u = l ? (u == B2 - 1 ? 1 : u + 1) : 0;
+        q = q == B2 - 1 ? 1 : q + 1;
+        v = v == B2 - 1 ? 1 : v + 1;
         __syncthreads();
     }
     *cur_out = cur;

@@ -789,14 +789,13 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
     } else if (t < OB * OB) {
         const int k = t % OB, l = t / OB;
         int cur = 0, rotated = 0;
+        int pk = k, qk = B2 - 1 - k, pl = l, ql = B2 - 1 - l;       // the circle method's round 0
         const int r_first = KEEP ? 0 : cx.first_round ? -(OB - 1) : 0, r_end = KEEP ? B2 - 1 : OB;
         for (int pass = 0; pass < (KEEP ? 1 : 2); ++pass) {
             int big = 0;
             for (int r = r_first; r < r_end; ++r) {
-                int pk, qk, pl, ql;
                 if (KEEP) {
-                    pk = circle_item(k, r, B2); qk = circle_item(B2 - 1 - k, r, B2);
-                    pl = circle_item(l, r, B2); ql = circle_item(B2 - 1 - l, r, B2);
+                    // (moved on at the end of the round)
                 } else if (r >= 0) {
                     pk = k; qk = OB + ((k + r) & (OB - 1));
                     pl = l; ql = OB + ((l + r) & (OB - 1));
@@ -818,7 +817,7 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
                 T ck, sk;
                 bool act;
                 if constexpr (KEEP) {
-                    act = fabs(apq) > num<T>::tiny() && fabs(apq) > num<T>::eps() * sqrt(fabs(app * aqq));
+                    act = fabs(apq) > num<T>::tiny() && above_eps_root(fabs(apq), fabs(app * aqq));
                     jacobi_rotation<T>(app, aqq, apq, ck, sk);
                 } else {
                     act = needs_rotation(app, aqq, apq);
@@ -846,6 +845,12 @@ __device__ T osj_pivot(Smem<T>& sm, cg::cluster_group& cl, const PivotCtx<T>& cx
                 sm.R[(k + OB) * LS + pl] = fma(clr, x1, -(slr * y1));
                 sm.R[(k + OB) * LS + ql] = fma(slr, x1, clr * y1);
                 cur ^= 1;
+                if (KEEP) {
+                    pk = k ? (pk == B2 - 1 ? 1 : pk + 1) : 0;
+                    pl = l ? (pl == B2 - 1 ? 1 : pl + 1) : 0;
+                    qk = qk == B2 - 1 ? 1 : qk + 1;
+                    ql = ql == B2 - 1 ? 1 : ql + 1;
+                }
                 if (r == r_end - 1) {
                     if (big) sm.sig[pass] = 1;
                     if (rotated) sm.rot = 1;
