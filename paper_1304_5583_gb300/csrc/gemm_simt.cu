@@ -92,8 +92,14 @@ __device__ __forceinline__ void load_slab(T* S, const T* P, int64_t ld, int x0, 
     }
 }
 
+// CTAs to an SM the registers are cut for: four of the float32 64 x 64 tiles (128
+// registers: M Z of the 600 x 6000 solve 88 -> 75 us), but three when both
+// operands run along K (U^T P: 90 us at three, 118 at four, where it spills).
+template <typename T, bool TA, bool TB, int TM>
+constexpr int min_ctas() { return sizeof(T) == 4 && TM == 8 ? (TA && !TB ? 3 : 4) : 1; }
+
 template <typename T, bool TA, bool TB, int TM, int TN>
-__global__ void __launch_bounds__(NT) gemm_kernel(const GemmDesc<T>* __restrict__ descs, int tiles_m) {
+__global__ void __launch_bounds__(NT, min_ctas<T, TA, TB, TM>()) gemm_kernel(const GemmDesc<T>* __restrict__ descs, int tiles_m) {
     constexpr int BM = 8 * TM, BN = 16 * TN, V = 16 / sizeof(T);
     constexpr int LA = BM + V, LB = BN + V, SLAB = BK * (LA + LB);
     static_assert(BN * LA <= STAGES * SLAB, "C leaves through the ring");
@@ -102,6 +108,12 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const GemmDesc<T>* __restrict_
     const int tm = blockIdx.x % tiles_m, tn = blockIdx.x / tiles_m;
     const int m0 = tm * BM, n0 = tn * BN;
     if (m0 >= d.m || n0 >= d.n) return;
+    // A^T A and A A^T: the tiles above the diagonal are computed and stored twice
+    // (the mirrored element has the same products in the same order)
+    static_assert(BM == BN, "square tiles");
+    const bool sym = TA != TB && d.A == d.B && d.lda == d.ldb && d.m == d.n && d.beta == T(0) && !d.ccol && !d.kscale &&
+                     !d.absmax;
+    if (sym && tm > tn) return;
 
     extern __shared__ __align__(16) unsigned char gemm_smem[];
     T* const ring = reinterpret_cast<T*>(gemm_smem);
@@ -187,6 +199,11 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const GemmDesc<T>* __restrict_
         if (d.beta != T(0)) v = fma(d.beta, *c, v);
         *c = v;
     }
+    if (sym && tm != tn)
+        for (int e = t; e < BM * BN; e += NT) {
+            const int j = e % BN, i = e / BN, gi = m0 + i, gj = n0 + j;
+            if (gi < d.m && gj < d.n) d.C[gj + (int64_t)gi * d.ldc] = Cs[j * LA + i];
+        }
 }
 
 template <typename T, int TM, int TN>
