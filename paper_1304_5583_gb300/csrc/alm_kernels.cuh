@@ -136,20 +136,12 @@ static __global__ void svt_gate(const int* __restrict__ act, double* __restrict_
 // 1000 x 487 SVT took 90 us.
 constexpr int kWeightCols = 32;
 template <typename T>
-__global__ void svt_weights(const OsjDesc<T>* __restrict__ descs, T* const* __restrict__ h,
-                            const int* __restrict__ act, const int* __restrict__ svt_on,
-                            const double* __restrict__ mu, int* __restrict__ rank, int nblk) {
-    const int b = blockIdx.x;
-    if (b >= nblk || !act[b]) return;
-    const OsjDesc<T> d = descs[b];
-    T* hb = h[b];
-    const double tau = 1.0 / mu[b];
+__device__ __forceinline__ void weights_of(const OsjDesc<T>& d, T* hb, double mu, int on, int j0, int j1, int* rank) {
+    const double tau = 1.0 / mu;
     const T tau_t = (T)tau;
-    const int on = svt_on[b];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int j1 = min(d.pp, (int)(blockIdx.y + 1) * kWeightCols);
     int cnt = 0;
-    for (int j = blockIdx.y * kWeightCols + warp; j < j1; j += nw) {
+    for (int j = j0 + warp; j < j1; j += nw) {
         T w = T(0);
         if (on && j < d.p) {
             const T* x = d.X + (int64_t)j * d.ldx;
@@ -163,7 +155,68 @@ __global__ void svt_weights(const OsjDesc<T>* __restrict__ descs, T* const* __re
             if (w > T(0)) ++cnt;
         }
     }
-    if (lane == 0 && cnt) atomicAdd(&rank[b], cnt);
+    if (lane == 0 && cnt) atomicAdd(rank, cnt);
+}
+template <typename T>
+__global__ void svt_weights(const OsjDesc<T>* __restrict__ descs, T* const* __restrict__ h,
+                            const int* __restrict__ act, const int* __restrict__ svt_on,
+                            const double* __restrict__ mu, int* __restrict__ rank, int nblk) {
+    const int b = blockIdx.x;
+    if (b >= nblk || !act[b]) return;
+    const OsjDesc<T> d = descs[b];
+    const int j0 = blockIdx.y * kWeightCols;
+    weights_of<T>(d, h[b], mu[b], svt_on[b], j0, min(d.pp, j0 + kWeightCols), &rank[b]);
+}
+
+// svt_weights, the two products W^T W and W (W^T W), and ns_orth (below) in one
+// launch, a CTA per block, for blocks of at most 64 columns: four launches of
+// some 3 us each for a few kFMA.  The products are summed as gemm_grouped sums
+// them (a fresh partial for every 16 terms), so nothing changes but the time.
+constexpr int kFinishCols = 64, kFinishThreads = 512;
+template <typename T>
+__global__ void __launch_bounds__(kFinishThreads) svt_finish(const OsjDesc<T>* __restrict__ descs, T* const* __restrict__ h,
+                                                             T* const* __restrict__ Wi, const int* __restrict__ act,
+                                                             const int* __restrict__ svt_on, const double* __restrict__ mu,
+                                                             int* __restrict__ rank) {
+    constexpr int LD = kFinishCols + 1;
+    extern __shared__ __align__(16) unsigned char finish_smem[];
+    T* const W = reinterpret_cast<T*>(finish_smem);          // W[i * LD + j]: row i, column j
+    T* const G = W + kFinishCols * LD;
+    const int b = blockIdx.x, t = threadIdx.x;
+    if (!act[b]) return;
+    const OsjDesc<T> d = descs[b];
+    const int on = svt_on[b], p = d.p;
+    weights_of<T>(d, h[b], mu[b], on, 0, d.pp, &rank[b]);
+    if (!on) return;
+    for (int e = t; e < p * p; e += kFinishThreads) W[e % p * LD + e / p] = d.W[e % p + (int64_t)(e / p) * d.ldw];
+    __syncthreads();
+    for (int e = t; e < p * p; e += kFinishThreads) {
+        const int i = e / p, j = e % p;
+        T acc = T(0);
+        for (int k0 = 0; k0 < p; k0 += 16) {
+            T part = T(0);
+            const int k1 = min(p, k0 + 16);
+            for (int k = k0; k < k1; ++k) part = fma(W[k * LD + i], W[k * LD + j], part);
+            acc += part;
+        }
+        G[i * LD + j] = acc;
+    }
+    __syncthreads();
+    T* const wi = Wi[b];
+    for (int e = t; e < p * p; e += kFinishThreads) {
+        const int i = e % p, j = e / p;
+        T acc = T(0);
+        for (int k0 = 0; k0 < p; k0 += 16) {
+            T part = T(0);
+            const int k1 = min(p, k0 + 16);
+            for (int k = k0; k < k1; ++k) part = fma(W[i * LD + k], G[k * LD + j], part);
+            acc += part;
+        }
+        const int64_t o = i + (int64_t)j * d.ldw;
+        const T wv = W[i * LD + j];
+        wi[o] = T(2) * wv - acc;
+        d.W[o] = T(1.5) * wv - T(0.5) * acc;
+    }
 }
 
 // Z-step in reduced coordinates, fused with the Y2 dual step and the next

@@ -749,6 +749,13 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
             g_tune_cluster[key] = jcluster;
         }
     }
+    // small blocks finish their SVT in one launch
+    const bool finish = max_pp <= k::kFinishCols;
+    const size_t finish_smem = sizeof(T) * 2 * k::kFinishCols * (k::kFinishCols + 1);
+    if (finish) {
+        static std::atomic<uint64_t> smem_set{0};
+        LRR_CUDA_TRY(ensure_smem_limit(k::svt_finish<T>, (int)finish_smem, smem_set));
+    }
     // launch shape of the Jacobi for the blocks still active (the others' clusters
     // leave at once); re-picked as blocks converge
     int jshape_n = t;
@@ -885,13 +892,19 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
                                    jshape.grid ? jlist : nullptr));
         prof.end(LRR_PH_JACOBI, 1);
         prof.begin();
-        k::svt_weights<T><<<dim3((unsigned)t, ceil_div(max_pp, k::kWeightCols)), 256, 0, q>>>(B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
         // W^T W and W (W^T W): first-order inverse for J, Newton-Schulz for the warm start
-        LRR_CUDA_TRY(run_set(S_O1));
-        LRR_CUDA_TRY(run_set(S_O2));
-        k::ns_orth<T><<<dim3(64, (unsigned)t), 256, 0, q>>>(B.Wp, B.Hp, B.T1p, B.pv, B.ppv, B.svt_on, t);
+        if (finish) {
+            k::svt_finish<T><<<(unsigned)t, k::kFinishThreads, finish_smem, q>>>(B.jd, B.hp, B.T1p, B.act, B.svt_on, B.mu,
+                                                                                B.rank_cur);
+        } else {
+            k::svt_weights<T><<<dim3((unsigned)t, ceil_div(max_pp, k::kWeightCols)), 256, 0, q>>>(
+                B.jd, B.hp, B.act, B.svt_on, B.mu, B.rank_cur, t);
+            LRR_CUDA_TRY(run_set(S_O1));
+            LRR_CUDA_TRY(run_set(S_O2));
+            k::ns_orth<T><<<dim3(64, (unsigned)t), 256, 0, q>>>(B.Wp, B.Hp, B.T1p, B.pv, B.ppv, B.svt_on, t);
+        }
         LRR_CUDA_TRY(run_set(S_J));
-        prof.end(LRR_PH_SVT_APPLY, 5);
+        prof.end(LRR_PH_SVT_APPLY, finish ? 2 : 5);
         // Z-step
         prof.begin();
         if constexpr (std::is_same<T, float>::value) {
