@@ -33,9 +33,11 @@
 // updates visible to the next).  Where a cluster has more CTAs than a round
 // has pivots, `split` CTAs share one pivot: each forms the Gram of its rows,
 // the partial Grams meet through distributed shared memory, every member runs
-// the same (tiny) inner rotation and applies it to its own rows.  A Gram is
-// always the sum of the same four row-slot partials in the same order, so
-// neither the cluster size nor the split changes a bit of the result.
+// the same (tiny) inner rotation and applies it to its own rows.  A cluster ends
+// at 16 CTAs; the clusterless form (below, `meet`) splits the pivots of a few
+// blocks over more of the chip, its CTAs meeting through memory.  A Gram is
+// always the sum of the same row-slot partials in the same order, so neither
+// the cluster size nor the split nor the form changes a bit of the result.
 // After each sweep the cluster reduces the largest convergence measure seen in
 // it and stops once that is below the tolerance, so a converged block costs
 // nothing further and the others are not held to a common sweep count.
@@ -58,11 +60,12 @@ namespace {
 
 // Threads per CTA (a CTA works on one pivot, or one member's share of it, at a
 // time).  512, one CTA to an SM, with the pivot's columns of X kept in shared
-// memory from the Gram to the rotation, when the blocks' clusters have the SMs
-// to themselves: a pivot's own chain of loads, products and rotations is then
-// all there is to wait for.  256 at up to 80 registers, three CTAs to an SM,
-// when there are more blocks than that (or columns too long to keep): their
-// phases cover one another's latencies.
+// memory from the Gram to the rotation, when the blocks' CTAs have the SMs to
+// themselves: a pivot's own chain of loads, products and rotations is then all
+// there is to wait for (a rotated pivot of the 350 x 256 float32 SVT: 20 us, 8 of
+// them the inner rotations, 6 the update, 2 the Gram).  256 at up to 80
+// registers, three CTAs to an SM, when there are more blocks than that (or
+// columns too long to keep): their phases cover one another's latencies.
 constexpr int NT_MANY = 256, NT_FEW = 512;
 // A Gram is summed in row slots: of every chunk of 64 rows, slot s has the SR
 // rows from SR s (float32: 4 slots of 16 rows, each chunk's 16 products summed on

@@ -269,10 +269,12 @@ size_t seg_layout(SegBuf& b, char* base, int64_t n, int k, int K, int restarts) 
     b.Ri = (float*)take(sizeof(float) * K * K);
     b.d = (double*)take(sizeof(double) * std::max<int64_t>(n, k));
     b.cost = (double*)take(sizeof(double) * restarts);
-    b.cols = (float*)take(sizeof(float) * 2 * pp);
+    // the Jacobi's scratch: in the affinity's place, which is written after it (n >= k
+    // > pp - 32, so n^2 >= 3 pp past one pivot)
+    b.cols = pp > 32 ? b.A : (float*)take(sizeof(float) * 64);
     b.of3 = (float*)take(sizeof(float) * 3);
     b.d2 = (float*)take(sizeof(float) * n * restarts);
-    b.ord = (int*)take(sizeof(int) * pp);
+    b.ord = pp > 32 ? reinterpret_cast<int*>(b.A + 2 * pp) : (int*)take(sizeof(int) * 32);
     b.on = (int*)take(sizeof(int));
     b.idx = (int*)take(sizeof(int) * k);
     b.labels = (int*)take(sizeof(int) * n * restarts);

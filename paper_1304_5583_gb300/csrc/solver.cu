@@ -106,8 +106,8 @@ struct Buffers {
     std::vector<int*> rot;
     int* rot_d;
     double *mu, *mu_fin, *resid;
-    int *act, *iters, *svt_on, *rank_cur, *rank_fin, *need_exact, *conv_bound, *conv, *jord, *j_on, *colblk, *flag;
-    T *r1, *dmax, *r2x, *jcols, *joff;
+    int *act, *iters, *svt_on, *rank_cur, *rank_fin, *need_exact, *conv_bound, *conv, *j_on, *colblk, *flag;
+    T *r1, *dmax, *r2x, *joff;
     int64_t* perm;
     // descriptor / pointer tables
     GemmDesc<T>* gd;       // 12 * t descriptors
@@ -221,16 +221,12 @@ Buffers<T> carve(Arena& a, const lrr_problem* p, bool need_md, const std::vector
     b.need_exact = a.take<int>(t);
     b.conv_bound = a.take<int>(t);
     b.conv = a.take<int>(t);
-    size_t cols_pad = 0;      // every block's columns, each padded to the pivot width
-    for (int i = 0; i < t; ++i) cols_pad += (size_t)blk[i].ppmax;
-    b.jord = a.take<int>(cols_pad);
     b.j_on = a.take<int>(t);
     b.colblk = a.take<int>(n);
     b.flag = a.take<int>(4);
     b.r1 = a.take<T>(t);
     b.dmax = a.take<T>(t);
     b.r2x = a.take<T>(t);
-    b.jcols = a.take<T>(2 * cols_pad);
     b.joff = a.take<T>(3 * (size_t)t);   // three convergence slots per block
     b.perm = a.take<int64_t>(n);
     b.gd = a.take<GemmDesc<T>>(16 * (size_t)t + 16);
@@ -440,8 +436,9 @@ bool use_tc32(const lrr_problem* p, const lrr_options* o) {
 }
 
 // Workspaces of the Jacobi's clusterless form (osj.cu), one per block, after an
-// integer that a wait which gave up sets and the list of the active blocks.  They come after everything else: a caller's
-// workspace of the size without them is taken too, and the form then left out.
+// integer that a wait which gave up sets and the list of the active blocks.  They
+// come after everything else: a caller's workspace of the size without them is
+// taken too, and the form then left out.
 template <typename T>
 size_t jgrid_bytes(const std::vector<BlockInfo<T>>& blk) {
     size_t n = 3 * kAlign + sizeof(int) * blk.size();
@@ -680,7 +677,6 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     LRR_CUDA_TRY(cudaMemcpyAsync(B.pv, pv.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
     LRR_CUDA_TRY(cudaMemcpyAsync(B.ppv, ppv.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
     std::vector<OsjDesc<T>> jdh((size_t)t);
-    int64_t cols_off = 0;
     size_t grid_off = kAlign + (sizeof(int) * t + kAlign - 1) / kAlign * kAlign;
     for (int i = 0; i < t; ++i) {
         OsjDesc<T>& j = jdh[i];
@@ -689,8 +685,8 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         j.L = tall[i] ? r : blk[i].l;
         j.W = B.W[i]; j.ldw = ppv[i]; j.p = pv[i]; j.pp = ppv[i];
         j.off = B.joff + 3 * i; j.active = B.svt_on + i;
-        j.cols = B.jcols + 2 * cols_off; j.ord = B.jord + cols_off;
-        cols_off += blk[i].ppmax;
+        // T1 and H of a block are written only after its Jacobi: its scratch until then
+        j.cols = B.T1[i]; j.ord = reinterpret_cast<int*>(B.H[i]);
         j.mu = B.mu + i;
         j.strict = (dfc && t > 1 && i == 0) ? 1 : 0;
         j.grid = jgrid ? jgrid + grid_off : nullptr;

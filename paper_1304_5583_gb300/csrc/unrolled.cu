@@ -270,8 +270,11 @@ size_t carve_engine(Engine<T>& g, Bump& b) {
     g.rank_d = b.take<int>(1);
     g.Wh = b.take<T>((size_t)pp * pp); g.Wg = b.take<T>((size_t)pp * pp); g.Wt = b.take<T>((size_t)pp * pp);
     g.od = b.take<OsjDesc<T>>(1);
-    g.ocols = b.take<T>(2 * (size_t)pp); g.ooff = b.take<T>(3);
-    g.oord = b.take<int>(pp); g.oon = b.take<int>(1);
+    g.ooff = b.take<T>(3);
+    g.oon = b.take<int>(1);
+    // the Jacobi's scratch: Wh is written only after it
+    g.ocols = g.Wh;
+    g.oord = reinterpret_cast<int*>(g.Wh ? g.Wh + 2 * (size_t)pp : nullptr);
     g.pW = b.take<T*>(1); g.pH = b.take<T*>(1); g.pT = b.take<T*>(1);
     g.pv = b.take<int>(1); g.ppv = b.take<int>(1);
     g.gd = b.take<GemmDesc<T>>(64);
