@@ -103,28 +103,34 @@ __global__ void init_padded(T* __restrict__ G, int p, int pp, T diag, int eye) {
 // Per-block SVT gate: ||A||_F^2 <= tau^2 means every singular value of A is
 // <= tau, so the threshold removes all of them and J = 0 with no SVD.
 // The Z-step kernel of the same iteration then accumulates the next value.
-static __global__ void svt_gate(const int* __restrict__ act, double* __restrict__ afro, const double* __restrict__ mu,
-                         int* __restrict__ svt_on, int* __restrict__ j_on, int* __restrict__ calls,
-                         int* __restrict__ rank,
-                         int* __restrict__ fp32_on, int* __restrict__ gemm32, double margin, int nblk) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nblk) return;
-    const double tau = 1.0 / mu[b];
+struct Gate {
+    double* afro;
+    int *svt_on, *j_on, *calls, *rank, *fp32_on, *gemm32;
+    double margin;
+};
+static __device__ __forceinline__ void gate_block(const Gate& g, int b, bool act, double mu) {
+    const double tau = 1.0 / mu, afro = g.afro[b];
     // J is formed while the block's SVT acts, and once more (as zero) after it
     // stops acting; before its first SVT it is zero already
-    const int was_on = svt_on[b];
-    svt_on[b] = (act[b] && afro[b] > tau * tau) ? 1 : 0;
-    j_on[b] = act[b] && (svt_on[b] || was_on);
-    if (svt_on[b]) calls[b] += 1;
+    const int was_on = g.svt_on[b], on = act && afro > tau * tau;
+    g.svt_on[b] = on;
+    g.j_on[b] = act && (on || was_on);
+    if (on) g.calls[b] += 1;
     // mixed precision: float32 products from the first iteration in which
     // ||A||_F exceeds margin * tau (sticky); before that J = 0 and the bf16
     // rounding of the products is forgotten by the iteration
-    if (afro[b] > margin * margin * tau * tau) fp32_on[b] = 1;
-    gemm32[b] = (act[b] && fp32_on[b]) ? 1 : 0;
-    if (act[b]) {
-        afro[b] = 0.0;
-        rank[b] = 0;
+    int f32 = g.fp32_on[b];
+    if (afro > g.margin * g.margin * tau * tau) g.fp32_on[b] = f32 = 1;
+    g.gemm32[b] = act && f32;
+    if (act) {
+        g.afro[b] = 0.0;
+        g.rank[b] = 0;
     }
+}
+// before the first iteration; after that the stop test's last kernel does it
+static __global__ void svt_gate(const int* __restrict__ act, const double* __restrict__ mu, const Gate g, int nblk) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < nblk) gate_block(g, b, act[b] != 0, mu[b]);
 }
 
 // After the one-sided Jacobi the columns x_j of X are orthogonal and
@@ -219,6 +225,30 @@ __global__ void __launch_bounds__(kFinishThreads) svt_finish(const OsjDesc<T>* _
     }
 }
 
+// The scalars of a column's step: 1/mu, mu, 1/mu' (the next iteration's mu) and
+// lambda/mu, from float64 quotients.  A float64 quotient is some 25 operations of
+// the one float64 unit of an SM, whatever the lanes: one warp takes them for all
+// of the CTA's columns, a lane each (e_update, 5000 columns of 500: 28 us when
+// every warp took its own, 25 so).
+constexpr int kStepWarps = 8;
+template <typename T>
+struct StepScalars {
+    T imu, mu, imun, thr;
+};
+template <typename T>
+__device__ __forceinline__ void step_scalars(StepScalars<T>* out, int64_t n, const int* colblk, const int* act,
+                                             const double* mu, double rho, double mu_max, double lam) {
+    const int64_t j = blockIdx.x * (int64_t)kStepWarps + threadIdx.x;
+    if (threadIdx.x < kStepWarps && j < n) {
+        const int b = colblk[j];
+        if (act[b]) {
+            const double mud = mu[b], mun = fmin(rho * mud, mu_max);
+            out[threadIdx.x] = StepScalars<T>{(T)(1.0 / mud), (T)mud, (T)(1.0 / mun), (T)(lam / mud)};
+        }
+    }
+    __syncthreads();
+}
+
 // Z-step in reduced coordinates, fused with the Y2 dual step and the next
 // SVT input; one warp per column.  With T = U^T (Y1/mu - E) on entry:
 //   Zt = (sigma (Theta + T) + Jt - Y2t/mu) / (1 + sigma^2)
@@ -233,12 +263,13 @@ __global__ void z_update(int r, int64_t n, const int* __restrict__ colblk, const
                          float* __restrict__ dhi, float* __restrict__ dlo, int64_t lds) {
     const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    __shared__ StepScalars<T> scalars[kStepWarps];
+    step_scalars<T>(scalars, n, colblk, act, mu, rho, mu_max, 0.0);
     if (j >= n) return;
     const int b = colblk[j];
     if (!act[b]) return;
-    const double mud = mu[b];
-    const double mun = fmin(rho * mud, mu_max);
-    const T imu = (T)(1.0 / mud), muT = (T)mud, imun = (T)(1.0 / mun);
+    const StepScalars<T> q = scalars[threadIdx.x >> 5];
+    const T imu = q.imu, muT = q.mu, imun = q.imun;
     const int64_t o = j * r;
     T acc = T(0), aacc = T(0);
     for (int i = lane; i < r; i += 32) {
@@ -278,13 +309,13 @@ __global__ void e_update(int64_t m, int64_t n, const int* __restrict__ colblk, c
                          float* __restrict__ qlo, int64_t lds) {
     const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    __shared__ StepScalars<T> scalars[kStepWarps];
+    step_scalars<T>(scalars, n, colblk, act, mu, rho, mu_max, lam);
     if (j >= n) return;
     const int b = colblk[j];
     if (!act[b]) return;
-    const double mud = mu[b];
-    const double mun = fmin(rho * mud, mu_max);
-    const T imu = (T)(1.0 / mud), muT = (T)mud, imun = (T)(1.0 / mun);
-    const T thr = (T)(lam / mud);
+    const StepScalars<T> q = scalars[threadIdx.x >> 5];
+    const T imu = q.imu, muT = q.mu, imun = q.imun, thr = q.thr;
     const int64_t o = j * m;
     T acc = T(0);
     for (int64_t i = lane; i < m; i += 32) {
@@ -384,11 +415,13 @@ __global__ void stop_part2(int nblk, int* __restrict__ act, int* __restrict__ it
                            T* __restrict__ dmax, T* __restrict__ r2x, const int* __restrict__ need_exact,
                            const int* __restrict__ conv_bound, T nu, double* __restrict__ resid,
                            const int* __restrict__ rank_cur, int* __restrict__ rank_fin, int* __restrict__ conv,
-                           double* __restrict__ mu_fin, double* __restrict__ afro, int* __restrict__ tc_dec,
-                           unsigned* __restrict__ bmax, int* __restrict__ any_need) {
+                           double* __restrict__ mu_fin, int* __restrict__ tc_dec, unsigned* __restrict__ bmax,
+                           int* __restrict__ any_need, const Gate gate) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nblk) return;
-    if (act[b]) {
+    bool on = act[b] != 0;
+    double mub = mu[b];
+    if (on) {
         const int it = ++iters[b];
         const bool ok = conv_bound[b] || (need_exact[b] && (double)r2x[b] < eps);
         const bool have = need_exact[b] || (tc_dec && tc_dec[b]);
@@ -396,14 +429,16 @@ __global__ void stop_part2(int nblk, int* __restrict__ act, int* __restrict__ it
         resid[2 * b] = (double)r1[b];
         resid[2 * b + 1] = rz;
         rank_fin[b] = rank_cur[b];
-        mu_fin[b] = mu[b];
+        mu_fin[b] = mub;
         if (ok || it >= max_iter) {
             act[b] = 0;
             conv[b] = ok ? 1 : 0;
+            on = false;
         } else {
-            mu[b] = fmin(rho * mu[b], mu_max);
+            mu[b] = mub = fmin(rho * mub, mu_max);
         }
     }
+    gate_block(gate, b, on, mub);          // of the next iteration
     r1[b] = T(0);
     dmax[b] = T(0);
     r2x[b] = T(0);

@@ -874,15 +874,14 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     // the tensor-core stage of the stop test runs in chunks that follow one in
     // which some block needed ||V D||_inf (its empty launches are not free)
     bool tc_window = false;
+    const k::Gate gate{B.afro, B.svt_on, B.j_on, B.svtcalls, B.rank_cur, B.fp32_on, B.gemm32, switch_margin};
     auto iteration = [&]() -> int {
         prof.iterations += 1;
         // J-step: SVT of A = Zt + Y2t/mu through the Gram eigendecomposition
         prof.begin();
-        k::svt_gate<<<ceil_div(t, 128), 128, 0, q>>>(B.act, B.afro, B.mu, B.svt_on, B.j_on, B.svtcalls, B.rank_cur,
-                                                         B.fp32_on, B.gemm32, switch_margin, t);
         LRR_CUDA_TRY(run_set(S_XT));
         LRR_CUDA_TRY(run_set(S_XW));
-        prof.end(LRR_PH_GRAM, 1 + nl(S_XT) + nl(S_XW));
+        prof.end(LRR_PH_GRAM, nl(S_XT) + nl(S_XW));
         prof.begin();
         LRR_CUDA_TRY(osj_sweeps<T>(B.jd, jshape.grid ? jshape_n : t, jshape, sweeps, jtol, B.jsweeps, q, OsjMode::kept, quad_exit,
                                    jshape.grid ? jlist : nullptr));
@@ -962,7 +961,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         k::stop_part2<T><<<ceil_div(t, 128), 128, 0, q>>>(t, B.act, B.iters, B.mu, o->rho, o->mu_max, o->eps,
                                                           o->max_iter, B.r1, B.dmax, B.r2x, B.need_exact,
                                                           B.conv_bound, nu_h, B.resid, B.rank_cur, B.rank_fin,
-                                                          B.conv, B.mu_fin, B.afro, B.tc_dec, B.bmax, B.any_need);
+                                                          B.conv, B.mu_fin, B.tc_dec, B.bmax, B.any_need, gate);
         prof.end(LRR_PH_STOP, tc_stage ? 6 : 3);
         LRR_CUDA_TRY(cudaGetLastError());
         return LRR_OK;
@@ -1030,6 +1029,9 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
             return cudaSuccess;
         };
         LRR_CUDA_TRY(pick_shape(act0));
+        prof.begin();
+        k::svt_gate<<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.mu, gate, t);
+        prof.end(LRR_PH_GRAM, 1);
         tc_window = false;
         while (done_it < o->max_iter) {
             const int len = std::min(chunk, o->max_iter - done_it);
