@@ -231,6 +231,9 @@ __global__ void __launch_bounds__(kFinishThreads) svt_finish(const OsjDesc<T>* _
 // of the CTA's columns, a lane each (e_update, 5000 columns of 500: 28 us when
 // every warp took its own, 25 so).
 constexpr int kStepWarps = 8;
+// rows of 32 whose loads a warp has in flight together: a column is a serial chain
+// of its rows otherwise, and 5000 columns are half a wave
+constexpr int kStepRows = 4;
 template <typename T>
 struct StepScalars {
     T imu, mu, imun, thr;
@@ -272,22 +275,35 @@ __global__ void z_update(int r, int64_t n, const int* __restrict__ colblk, const
     const T imu = q.imu, muT = q.mu, imun = q.imun;
     const int64_t o = j * r;
     T acc = T(0), aacc = T(0);
-    for (int i = lane; i < r; i += 32) {
-        const T th = Theta[o + i], jv = Jt[o + i], y2 = Y2t[o + i];
-        const T z = dinv[i] * (sig[i] * (th + Tt[o + i]) + jv - y2 * imu);
-        const T dl = th - sig[i] * z;
-        const T dd = z - jv;
-        const T y2n = y2 + muT * dd;
-        const T av = z + y2n * imun;
-        Zt[o + i] = z;
-        Tt[o + i] = dl;
-        if (dbf) split_bf16((float)dl, dbf[i + j * ldd], dbf_lo[i + j * ldd]);
-        if (dhi) split_tf32((float)dl, dhi[i + j * lds], dlo[i + j * lds]);
-        D[o + i] = dd;
-        Y2t[o + i] = y2n;
-        A[o + i] = av;
-        acc += dd * dd;
-        aacc += av * av;
+    for (int i0 = lane; i0 < r; i0 += 32 * kStepRows) {
+        T th[kStepRows], jv[kStepRows], y2[kStepRows], tt[kStepRows], sg[kStepRows], di[kStepRows];
+#pragma unroll
+        for (int u = 0; u < kStepRows; ++u) {
+            const int i = i0 + 32 * u;
+            if (i < r) {
+                th[u] = Theta[o + i]; jv[u] = Jt[o + i]; y2[u] = Y2t[o + i]; tt[u] = Tt[o + i];
+                sg[u] = sig[i]; di[u] = dinv[i];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kStepRows; ++u) {
+            const int i = i0 + 32 * u;
+            if (i >= r) break;
+            const T z = di[u] * (sg[u] * (th[u] + tt[u]) + jv[u] - y2[u] * imu);
+            const T dl = th[u] - sg[u] * z;
+            const T dd = z - jv[u];
+            const T y2n = y2[u] + muT * dd;
+            const T av = z + y2n * imun;
+            Zt[o + i] = z;
+            Tt[o + i] = dl;
+            if (dbf) split_bf16((float)dl, dbf[i + j * ldd], dbf_lo[i + j * ldd]);
+            if (dhi) split_tf32((float)dl, dhi[i + j * lds], dlo[i + j * lds]);
+            D[o + i] = dd;
+            Y2t[o + i] = y2n;
+            A[o + i] = av;
+            acc += dd * dd;
+            aacc += av * av;
+        }
     }
     acc = warp_sum(acc);
     aacc = warp_sum(aacc);
@@ -318,28 +334,49 @@ __global__ void e_update(int64_t m, int64_t n, const int* __restrict__ colblk, c
     const T imu = q.imu, muT = q.mu, imun = q.imun, thr = q.thr;
     const int64_t o = j * m;
     T acc = T(0);
-    for (int64_t i = lane; i < m; i += 32) {
-        const T res = (Cp ? Cp[o + i] : T(0)) + UD[o + i];
-        const T x = res + Y1[o + i] * imu;
-        acc += x * x;
+    for (int64_t i0 = lane; i0 < m; i0 += 32 * kStepRows) {
+        T cp[kStepRows], ud[kStepRows], y1[kStepRows];
+#pragma unroll
+        for (int u = 0; u < kStepRows; ++u) {
+            const int64_t i = i0 + 32 * u;
+            if (i < m) { cp[u] = Cp ? Cp[o + i] : T(0); ud[u] = UD[o + i]; y1[u] = Y1[o + i]; }
+        }
+#pragma unroll
+        for (int u = 0; u < kStepRows; ++u) {
+            if (i0 + 32 * u >= m) break;
+            const T res = cp[u] + ud[u];
+            const T x = res + y1[u] * imu;
+            acc += x * x;
+        }
     }
     const T nrm = sqrt(warp_sum(acc));
     const T sc = nrm > thr ? T(1) - thr / nrm : T(0);
     T amax = T(0);
-    for (int64_t i = lane; i < m; i += 32) {
-        const T res = (Cp ? Cp[o + i] : T(0)) + UD[o + i];
-        const T y1 = Y1[o + i];
-        const T x = res + y1 * imu;
-        const T e = sc * x;
-        const T l1 = res - e;
-        const T y1n = y1 + muT * l1;
-        E[o + i] = e;
-        Y1[o + i] = y1n;
-        const T qv = y1n * imun - e;
-        Q[o + i] = qv;
-        if (qbf) split_bf16((float)qv, qbf[i + j * ldq], qbf_lo[i + j * ldq]);
-        if (qhi) split_tf32((float)qv, qhi[i + j * lds], qlo[i + j * lds]);
-        amax = fmax(amax, fabs(l1));
+    for (int64_t i0 = lane; i0 < m; i0 += 32 * kStepRows) {
+        T cp[kStepRows], ud[kStepRows], y1s[kStepRows];
+#pragma unroll
+        for (int u = 0; u < kStepRows; ++u) {
+            const int64_t i = i0 + 32 * u;
+            if (i < m) { cp[u] = Cp ? Cp[o + i] : T(0); ud[u] = UD[o + i]; y1s[u] = Y1[o + i]; }
+        }
+#pragma unroll
+        for (int u = 0; u < kStepRows; ++u) {
+            const int64_t i = i0 + 32 * u;
+            if (i >= m) break;
+            const T res = cp[u] + ud[u];
+            const T y1 = y1s[u];
+            const T x = res + y1 * imu;
+            const T e = sc * x;
+            const T l1 = res - e;
+            const T y1n = y1 + muT * l1;
+            E[o + i] = e;
+            Y1[o + i] = y1n;
+            const T qv = y1n * imun - e;
+            Q[o + i] = qv;
+            if (qbf) split_bf16((float)qv, qbf[i + j * ldq], qbf_lo[i + j * ldq]);
+            if (qhi) split_tf32((float)qv, qhi[i + j * lds], qlo[i + j * lds]);
+            amax = fmax(amax, fabs(l1));
+        }
     }
     amax = warp_max(amax);
     if (lane == 0) atomic_max_nonneg(&r1max[b], amax);
