@@ -135,3 +135,19 @@ def test_factor_of_awkward_spectra(lib, kind):
     ref = olrr.lrr_alm(M, M, lam, eps=1e-8)
     assert res.status == 0 and res.iters[0] == ref.iters
     assert _rel(res.Z.cpu().numpy(), ref.Z) < 1e-8 and _rel(res.S.cpu().numpy(), ref.E) < 1e-8
+
+
+# at least a tile of 128 x 256 for every SM: pairs of CTAs (4, 14 and 6 rows of
+# tiles, and 5 padded to 6) and single ones (3 rows)
+@pytest.mark.parametrize("M,N,K", [(512, 10000, 72), (1700, 3001, 200), (641, 7000, 64), (600, 8000, 136),
+                                   (300, 13100, 80)])
+def test_bf16_product_in_clusters_matches_float64(lib, M, N, K):
+    import torch
+    from paper_1304_5583_gb300 import binding
+    g = torch.Generator().manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=g).to(torch.bfloat16)
+    B = torch.randn(N, K, generator=g).to(torch.bfloat16)
+    C = binding.gemm_bf16(A.cuda(), B.cuda(), M, N, K).cpu().numpy()
+    ref = A.double().numpy() @ B.double().numpy().T
+    # the bar of the other bf16 products: float32 accumulation order alone
+    assert np.abs(C - ref).max() / np.abs(ref).max() < 2e-6
