@@ -966,9 +966,10 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         LRR_CUDA_TRY(cudaGetLastError());
         return LRR_OK;
     };
-    // A chunk of iterations as one graph launch: some sixteen kernels an iteration
-    // at 4 us of launch each are what a small solve takes (60 x 240: 110 of 150 us an
-    // iteration).  Recorded on a stream of its own (the legacy stream cannot be),
+    // A chunk of iterations as one graph launch: a dozen or more kernels an
+    // iteration at 4 us of launch each are what a small solve took (60 x 240: 110 of
+    // 150 us an iteration launched one by one, 64 us recorded).  Recorded on a stream
+    // of its own (the legacy stream cannot be),
     // when a set of the values that the launches depend on comes up again; with
     // per-phase events the launches are issued one by one.
     ChunkGraphs graphs;
