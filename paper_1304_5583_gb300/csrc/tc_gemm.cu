@@ -90,17 +90,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
-// the same box into the same place of every CTA of the cluster in `mask`, each
-// CTA's barrier (at the same place as `bar`) counting its own copy
-__device__ __forceinline__ void tma_load_2d_multicast(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar,
-                                                      uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-        "%3}], [%4], %5;\n" ::"r"(smem_u32(dst)),
-        "l"(map), "r"(c0), "r"(c1), "r"(smem_u32(bar)), "h"(mask)
-        : "memory");
-}
-
 // 32 columns of the warp's 32 TMEM lanes
 __device__ __forceinline__ void tmem_load_32(uint32_t addr, uint32_t (&v)[32]) {
     asm volatile(
@@ -131,19 +120,16 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// Persistent form: clusters of CL CTAs, one CTA per SM, walk the 128 x 256 tiles
-// of C, CL neighbours in M at a time (M fastest, so the clusters working at the
-// same time share the B slabs in L2).  The producer's stage ring and the
-// k-block counter run on across tiles; the accumulator is double-buffered in
-// TMEM (2 x 256 columns), so the MMAs of tile i + 1 run while the epilogue drains
-// tile i.  Bound by the operands' way from L2 (48 KB a slab and SM: 1000 x 20000 x
-// 1000 takes 5 rounds of tiles of 10.5 us for 4.5 us of MMAs): the CTAs of a
-// cluster need the same slab of B, so each fetches a CL-th of it and sends that to
-// all.  A stage is refilled once every CTA's MMAs have read it (their commits go
-// to all CL barriers).  A row of tiles past M is computed on zeros and not stored.
-// (68 us with one CTA to itself and four epilogue warps of 16 columns at a time,
-// which took as long as the operands; 62.7 with the present eight of 32; 52.5 so.)
-template <int CL>
+// Persistent form: one CTA per SM walks the 128 x 256 tiles of C (M fastest,
+// so the CTAs working at the same time share the B slabs in L2).  The
+// producer's stage ring and the k-block counter run on across tiles; the
+// accumulator is double-buffered in TMEM (2 x 256 columns), so the MMAs of
+// tile i + 1 run while the epilogue drains tile i.  Bound by the operands' way
+// from L2 (48 KB a slab and SM: 1000 x 20000 x 1000 takes 5 rounds of tiles of
+// 12 us for 4.5 us of MMAs): 68 us with four epilogue warps of 16 columns at a
+// time, which took as long as the operands, 60 with the present eight of 32.
+// (Every CTA loads its own operands, into its own shared memory only: each
+// process of a run on several GPUs loads this library.)
 __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
                                                         const __grid_constant__ CUtensorMap mapB, float* __restrict__ C,
                                                         int64_t ldc, int M, int N, int K, int* __restrict__ err,
@@ -156,20 +142,9 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // in units of CL tiles
-    const int tiles_m = (M + BM * CL - 1) / (BM * CL);
+    const int tiles_m = (M + BM - 1) / BM;
     const int ntiles = tiles_m * ((N + PBN - 1) / PBN);
     const int nk = (K + BK - 1) / BK;
-    const int rank = CL > 1 ? (int)(blockIdx.x % CL) : 0, first = blockIdx.x / CL, step = gridDim.x / CL;
-    constexpr uint16_t everyone = (uint16_t)((1u << CL) - 1);
-    auto sync_all = [&]() {
-        if constexpr (CL > 1) {
-            __syncwarp();
-            asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-        } else {
-            __syncthreads();
-        }
-    };
 
     // reduction form: the whole launch does nothing when *run == 0
     // (uniform, before any barrier or TMEM use)
@@ -188,7 +163,7 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
     if (threadIdx.x == 0) {
         for (int s = 0; s < PSTAGES; ++s) {
             mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], CL);
+            mbar_init(&empty_bar[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&accf[b], 1);
@@ -204,7 +179,7 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
-    sync_all();
+    __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = tmem_slot;
 
@@ -212,9 +187,9 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
         if (lane == 0) {
             int64_t g = 0;     // k-blocks issued over all tiles of this CTA
             bool ok = true;
-            for (int tile = first; tile < ntiles && ok; tile += step) {
+            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 if (skip(tile)) continue;
-                const int m0 = (tile % tiles_m * CL + rank) * BM, n0 = (tile / tiles_m) * PBN;
+                const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * PBN;
                 for (int kb = 0; kb < nk; ++kb, ++g) {
                     const int s = (int)(g % PSTAGES);
                     if (g >= PSTAGES && !mbar_wait(&empty_bar[s], (uint32_t)((g / PSTAGES) - 1) & 1, err)) ok = false;
@@ -225,17 +200,8 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
                     unsigned char* st = base + s * PSTAGE_BYTES;
                     mbar_expect_tx(&full_bar[s], PSTAGE_BYTES);
                     tma_load_2d(st, &mapA, kb * BK, m0, &full_bar[s]);
-                    if constexpr (CL > 1)
-                        tma_load_2d_multicast(st + TILE_A_BYTES + rank * (TILE_B_BYTES / CL), &mapB, kb * BK,
-                                              n0 + rank * (PBN / CL), &full_bar[s], everyone);
-                    else
-                        tma_load_2d(st + TILE_A_BYTES, &mapB, kb * BK, n0, &full_bar[s]);
+                    tma_load_2d(st + TILE_A_BYTES, &mapB, kb * BK, n0, &full_bar[s]);
                 }
-            }
-            if constexpr (CL > 1) {
-                // the others' last commits arrive here before the CTA may leave
-                for (int64_t j = g - PSTAGES < 0 ? 0 : g - PSTAGES; ok && j < g; ++j)
-                    ok = mbar_wait(&empty_bar[j % PSTAGES], (uint32_t)(j / PSTAGES) & 1, err);
             }
             if (!ok) {
                 abort_flag = 1;
@@ -250,7 +216,7 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
             int64_t g = 0;
             int i = 0;         // tiles computed by this CTA
             bool ok = true;
-            for (int tile = first; tile < ntiles && ok; tile += step) {
+            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 if (skip(tile)) continue;
                 const int buf = i & 1;
                 // the epilogue must have drained this accumulator (tile i - 2)
@@ -278,17 +244,9 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
                             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc),
                             "l"(da), "l"(db), "r"(idesc), "r"(accum));
                     }
-                    if constexpr (CL > 1)
-                        asm volatile(
-                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
-                            "[%0], %1;\n" ::"r"(smem_u32(&empty_bar[s])),
-                            "h"(everyone)
-                            : "memory");
-                    else
-                        asm volatile(
-                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                                smem_u32(&empty_bar[s]))
-                            : "memory");
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                                     smem_u32(&empty_bar[s]))
+                                 : "memory");
                 }
                 if (!ok) break;
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -310,13 +268,13 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
         const int q = warp & 3, half = (warp - 2) / 4;
         int i = 0;
         bool ok = true;
-        for (int tile = first; tile < ntiles; tile += step) {
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             if (skip(tile)) continue;
             const int buf = i & 1;
             ok = __all_sync(0xffffffffu, ok && mbar_wait(&accf[buf], (uint32_t)(i >> 1) & 1, err) && !abort_flag);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const int m0 = (tile % tiles_m * CL + rank) * BM, n0 = (tile / tiles_m) * PBN;
+            const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * PBN;
             const int row = m0 + q * 32 + lane;
             // reduction form: running max of the current column block; the
             // block changes at the same column for every lane of the warp
@@ -373,7 +331,7 @@ __global__ void __launch_bounds__(PNT, 1) tc_gemm_kernel(const __grid_constant__
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
-    sync_all();           // (the whole cluster's: none leaves while another may still send to it)
+    __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;\n");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * PBN));
@@ -643,52 +601,21 @@ cudaError_t tc_launch(const void* A, int64_t lda, const void* B, int64_t ldb, fl
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     if ((lda % 8) || (ldb % 8) || (reinterpret_cast<uintptr_t>(A) % 16) || (reinterpret_cast<uintptr_t>(B) % 16))
         return cudaErrorInvalidValue;
+    CUtensorMap ma, mb;
+    if (!make_map(&ma, A, K, M, lda) || !make_map(&mb, B, K, N, ldb, false, PBN)) return cudaErrorInvalidValue;
     const int64_t ntiles = (int64_t)ceil_div(M, BM) * ceil_div(N, PBN);
     if (ntiles > (1LL << 30)) return cudaErrorInvalidValue;
+    static std::atomic<uint64_t> smem_set{0};
+    const cudaError_t ea = ensure_smem_limit(tc_gemm_kernel, (int)tc_gemm_smem_bytes(), smem_set);
+    if (ea != cudaSuccess) return ea;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // pairs where every SM has work and few rows of tiles are past M (1000 x 20000 x
-    // 1000: 62.7 us without, 52.5 in pairs, 53.0 in fours, which leave SMs out)
-    const int rows = (int)ceil_div(M, BM);
-    const bool pairs = ntiles >= nsm && (rows % 2 == 0 || rows > 4);
-    auto go = [&](auto kernel, std::atomic<uint64_t>& smem_set, std::atomic<int>* fit, int c) -> cudaError_t {
-        CUtensorMap ma, mb;
-        if (!make_map(&ma, A, K, M, lda) || !make_map(&mb, B, K, N, ldb, false, PBN / c)) return cudaErrorInvalidValue;
-        cudaError_t r = ensure_smem_limit(kernel, (int)tc_gemm_smem_bytes(), smem_set);
-        if (r != cudaSuccess) return r;
-        cudaLaunchConfig_t cfg = {};
-        cfg.blockDim = dim3(PNT);
-        cfg.dynamicSmemBytes = tc_gemm_smem_bytes();
-        cfg.stream = s;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        // one CTA per SM (the 193 KB ring admits no second one); of clusters, as many as fit
-        // the device at once, looked up once
-        int clusters = nsm;
-        if (c > 1) {
-            clusters = dev < 64 ? fit[dev].load() : 0;
-            if (clusters == 0) {
-                cfg.gridDim = dim3((unsigned)c);
-                r = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
-                if (r != cudaSuccess) return r;
-                if (clusters < 1) return cudaErrorInvalidConfiguration;
-                if (dev < 64) fit[dev].store(clusters);
-            }
-        }
-        const int64_t units = (int64_t)ceil_div(M, BM * c) * ceil_div(N, PBN);
-        cfg.gridDim = dim3((unsigned)std::min<int64_t>(units, std::max(1, clusters)) * (unsigned)c);
-        r = cudaLaunchKernelEx(&cfg, kernel, ma, mb, C, ldc, M, N, K, err, am);
-        return r != cudaSuccess ? r : cudaGetLastError();
-    };
-    static std::atomic<uint64_t> smem_set[2];
-    static std::atomic<int> fit[64];
-    if (pairs) return go(tc_gemm_kernel<2>, smem_set[1], fit, 2);
-    return go(tc_gemm_kernel<1>, smem_set[0], nullptr, 1);
+    // one CTA per SM (the 193 KB ring admits no second one)
+    const unsigned grid = (unsigned)std::min<int64_t>(ntiles, std::max(1, nsm));
+    tc_gemm_kernel<<<grid, PNT, tc_gemm_smem_bytes(), s>>>(ma, mb, C, ldc, M, N, K, err, am);
+    return cudaGetLastError();
 }
 }  // namespace
 
