@@ -175,10 +175,11 @@ __device__ __forceinline__ void rotation(float d, float apq, float& t, float& c,
     c = rsqrt_approx(fmaf(t, t, 1.f));
     s = t * c;
 }
-// |s_pq| > eps sqrt(s_pp s_qq), with a square root good to a few per cent
+// |s_pq| > eps sqrt(s_pp s_qq), roots of the hardware's accuracy, a root each: the
+// product of two squared norms overflows from norms of 4e9 on (and then no pair
+// was rotated: an SVT of a 90 x 100 matrix of norm 1e10 was off by 17 %)
 __device__ __forceinline__ bool needs_rotation(float app, float aqq, float apq) {
-    float q;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(fabsf(app * aqq)));
+    const float q = sqrt_approx(fabsf(app)) * sqrt_approx(fabsf(aqq));
     return fabsf(apq) > FLT_MIN && fabsf(apq) > FLT_EPSILON * q;
 }
 // non-negative norms ordered by their bits (a NaN sorts first: the order stays
@@ -1136,7 +1137,11 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
             // at most one of them is above the rounding floor: its measure
             // would be zero.  The norms are one rotation old at most and good
             // to a few eps of the column block's largest, hence the margins.
-            // (Sorted: nor does any pair come near Gershgorin's bound.)
+            // (Sorted: nor does any pair come near Gershgorin's bound.  Its root is
+            // taken of norms relative to the largest column: the product of two
+            // squared norms itself underflows below 1e-11, columns above the floor
+            // do not; and in float32, the margin being 1e-3 -- a float64 root in
+            // every warp is 1 us of a round.)
             int cnt = 0;
             bool met = split == 1;
             for (int P0 = 0; P0 < npairs; P0 += 32) {
@@ -1149,7 +1154,10 @@ __global__ void __launch_bounds__(NT, NT == NT_MANY ? 3 : 1) osj_svd(const OsjDe
                     const T a1 = __ldcg(ti + 2 * a), a2 = __ldcg(ti + 2 * a + 1);
                     const T c1 = __ldcg(ti + 2 * c), c2 = __ldcg(ti + 2 * c + 1);
                     const T n1 = a1 > c1 ? a1 : c1, n2 = a1 > c1 ? (a2 > c1 ? a2 : c1) : (c2 > a1 ? c2 : a1);
-                    work = !((n1 + (KEEP ? n2 : T(d.p) * sqrt(n1 * n2))) * T(1.001) <= cx.tau * cx.tau) &&
+                    T other = n2;
+                    if (!KEEP)
+                        other = T(d.p) * cx.scale * (T)(sqrt_approx((float)(n1 * cx.inv_scale)) * sqrt_approx((float)(n2 * cx.inv_scale)));
+                    work = !((n1 + other) * T(1.001) <= cx.tau * cx.tau) &&
                            !(n2 * T(4) <= cx.floor2);
                     if (!work && rank == 0 && warp == 0) {
                         to[2 * a] = a1; to[2 * a + 1] = a2;

@@ -64,3 +64,28 @@ def test_many_blocks_agree_bitwise_with_one_block_at_a_time(lib, precision):
                                  raise_on_error=False) for b in (True, False)]
     assert np.array_equal(res[0].sweeps, res[1].sweeps) and res[0].sweeps.sum() > 48
     assert torch.equal(res[0].Z, res[1].Z) and torch.equal(res[0].S, res[1].S)
+
+
+# squared norms whose products leave the range (float32: below 1e-11 and above
+# 4e9), at scales where the squares themselves stay well inside it
+@pytest.mark.parametrize("dtype,scale", [("f32", 1e-14), ("f32", 1e-12), ("f32", 1e10), ("f32", 1e14),
+                                         ("f64", 1e-120), ("f64", 1e-100), ("f64", 1e100)])
+@pytest.mark.parametrize("kind", ["below the threshold one by one", "low rank"])
+def test_svt_does_not_depend_on_the_scale_of_its_input(lib, dtype, scale, kind):
+    import torch
+    from paper_1304_5583_gb300 import binding
+    dt = np.float32 if dtype == "f32" else np.float64
+    rng = np.random.default_rng(5)
+    if kind == "low rank":
+        A = rng.standard_normal((90, 40)) @ rng.standard_normal((40, 100)) / 60.0
+    else:
+        u, v = rng.standard_normal(90), rng.choice([-1.0, 1.0], 100)
+        A = np.outer(u / np.linalg.norm(u), v / 10.0) + 1e-4 * rng.standard_normal((90, 100))
+    A = (A * scale).astype(dt)
+    Jo, Uo, _, _ = olrr.svt(A.astype(np.float64), 0.3 * scale)
+    J, rank = binding.svt(torch.from_numpy(np.asfortranarray(A)).cuda(), 0.3 * scale)
+    assert rank == Uo.shape[1]
+    # the bars of the stand-alone SVT (norms of the values over the scale: a
+    # float64 norm squares them too)
+    J, Jo = J.cpu().numpy().astype(np.float64) / scale, Jo / scale
+    assert np.linalg.norm(J - Jo) <= (5e-6 if dtype == "f32" else 1e-12) * np.linalg.norm(Jo)
