@@ -91,6 +91,10 @@ template <typename T> size_t osj_grid_head(int p);
 struct OsjShape {
     int cluster, split, wide, max_L, max_p;
     int grid;           // 1: no cluster, the CTAs of a block meet through global memory
+    bool operator==(const OsjShape& o) const {
+        return cluster == o.cluster && split == o.split && wide == o.wide && max_L == o.max_L && max_p == o.max_p &&
+               grid == o.grid;
+    }
 };
 // the shape for nmat blocks of at most max_p columns and max_L rows; cluster
 // > 0 fixes the largest cluster size to use; grid: every block has a workspace

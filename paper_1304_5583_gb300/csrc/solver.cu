@@ -28,6 +28,7 @@
 
 #include "dfc_lrr.h"
 #include "alm_kernels.cuh"
+#include "autotune.h"
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -412,14 +413,6 @@ struct ChunkGraphs {
 // ---- autotuner: launch shape of the batched Jacobi (cluster size per block),
 // picked by timing the candidates on synthetic input of the problem's block
 // shapes the first time a shape is solved; cached per process and device.
-struct TuneKey {
-    int dev, prec;
-    int64_t m, n, r;
-    int t, max_pp;
-    bool operator<(const TuneKey& o) const {
-        return std::tie(dev, prec, m, n, r, t, max_pp) < std::tie(o.dev, o.prec, o.m, o.n, o.r, o.t, o.max_pp);
-    }
-};
 std::mutex g_tune_mutex;
 std::map<TuneKey, int> g_tune_cluster;
 
@@ -704,7 +697,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
     if (o->autotune) {
         int dev = 0;
         LRR_CUDA_TRY(cudaGetDevice(&dev));
-        const TuneKey key{dev, o->precision, m, n, r, t, max_pp};
+        const TuneKey key{dev, o->precision, m, n, r, t, max_pp, round_up(max_L, 64), jgrid != nullptr};
         bool have = false;
         {
             std::lock_guard<std::mutex> lk(g_tune_mutex);
@@ -712,9 +705,9 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
             if (it != g_tune_cluster.end()) { jcluster = it->second; have = true; }
         }
         if (!have) {
-            std::vector<int> cand;
+            std::vector<std::pair<int, OsjShape>> cand;
             for (int c : {0, 4, 8, 16})         // 0: osj_shape's own choice
-                if (c <= osj_max_cluster<T>()) cand.push_back(c);
+                if (c <= osj_max_cluster<T>()) cand.emplace_back(c, osj_shape<T>(t, max_p, max_L, c, jgrid != nullptr));
             std::vector<int> on((size_t)t, 1);
             std::vector<double> mu_t((size_t)t, 1e10);
             LRR_CUDA_TRY(cudaMemcpyAsync(B.svt_on, on.data(), sizeof(int) * t, cudaMemcpyHostToDevice, s));
@@ -722,25 +715,23 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
             cudaEvent_t ta, tb;
             LRR_CUDA_TRY(cudaEventCreate(&ta));
             LRR_CUDA_TRY(cudaEventCreate(&tb));
-            float best = 1e30f;
-            for (int c : cand) {
+            const bool timed = pick_fastest(cand, [&](const OsjShape& sh, bool warm_up) {
                 k::fill_hash<T><<<grid1(r * n), 256, 0, s>>>(B.D, r * n, 12345u);
                 for (int i = 0; i < t; ++i)
                     k::init_padded<T><<<grid1((int64_t)ppv[i] * ppv[i]), 256, 0, s>>>(B.W[i], pv[i], ppv[i], T(1), 1);
                 cudaEventRecord(ta, s);
-                const cudaError_t e = osj_sweeps<T>(B.jd, t, osj_shape<T>(t, max_p, max_L, c, jgrid != nullptr), 2, jtol_of<T>(), nullptr, s,
-                                                    OsjMode::kept, quad_exit);
+                const cudaError_t e = osj_sweeps<T>(B.jd, t, sh, warm_up ? 1 : 2, jtol_of<T>(), nullptr, s, OsjMode::kept,
+                                                    quad_exit);
                 cudaEventRecord(tb, s);
-                if (e != cudaSuccess || cudaEventSynchronize(tb) != cudaSuccess) {
-                    cudaEventDestroy(ta); cudaEventDestroy(tb);
-                    return LRR_ERR_CUDA;
-                }
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, ta, tb);
-                if (ms < best) { best = ms; jcluster = c; }
-            }
+                float ms = -1.f;
+                if (e != cudaSuccess || cudaEventSynchronize(tb) != cudaSuccess ||
+                    cudaEventElapsedTime(&ms, ta, tb) != cudaSuccess)
+                    return -1.f;
+                return ms;
+            }, &jcluster);
             cudaEventDestroy(ta);
             cudaEventDestroy(tb);
+            if (!timed) return LRR_ERR_CUDA;
             std::lock_guard<std::mutex> lk(g_tune_mutex);
             g_tune_cluster[key] = jcluster;
         }
