@@ -98,9 +98,24 @@ struct OsjShape {
 };
 // the shape for nmat blocks of at most max_p columns and max_L rows; cluster
 // > 0 fixes the largest cluster size to use; grid: every block has a workspace
-// for the clusterless form
+// for the clusterless form; together: how many such launches share the device
 template <typename T>
-OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster = 0, bool grid = false);
+OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster = 0, bool grid = false, int together = 1);
+
+// Held by a call that is little else than Jacobi launches (lrr_svt, the
+// unrolled iteration) while it runs; `together`: how many are held now on the
+// current device, this one included.  Results do not depend on it.
+class JacobiCall {
+public:
+    JacobiCall();
+    ~JacobiCall();
+    JacobiCall(const JacobiCall&) = delete;
+    JacobiCall& operator=(const JacobiCall&) = delete;
+    int together() const;
+
+private:
+    int slot;
+};
 
 // Schedule of the sweeps (osj.cu); float64 always runs `sorted`.
 enum class OsjMode { kept, sorted };

@@ -1309,7 +1309,7 @@ size_t osj_grid_bytes(int p) {
 }
 
 template <typename T>
-OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster, bool grid) {
+OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster, bool grid, int together) {
     // Cluster size: the caller's choice (autotuned), else the largest (up to
     // one CTA per pivot of a round) at which every block's cluster can be
     // resident at once -- a block waiting for a second wave would double the
@@ -1355,12 +1355,31 @@ OsjShape osj_shape(int nmat, int max_p, int max_L, int cluster, bool grid) {
         const int turns = (int)ceil_div((int64_t)pairs * sh.split, sh.cluster);
         return turns * (17.0 + work / sh.split) * (sh.wide ? 1.0 : 2.0) + (sh.grid ? 5.0 : 0.0);
     };
+    // Its CTAs are all resident or none, so launches that do not fit beside one
+    // another run in turn: each gets its share of the device.  (Eight threads with
+    // SVTs of 100 x 500 float64: 30 ms a call when each launch takes 112 CTAs, 8.7
+    // in clusters of 14; four threads 15 and, of 28 CTAs each, 5.5; of 1000 x 487
+    // float32 46 and 21, 29 and 14.)  Whole solves are not counted: eight at once
+    // are bound by their setup and the host's launches, and gain by what the form
+    // saves each (float64 100 x 200: 330 ms with it, 399 without).
     auto consider = [&](const OsjShape& sh) {
-        if (fits(sh) && cost(sh) < cost(best)) best = sh;
+        if (resident_clusters<T>(sh) >= nmat * together && cost(sh) < cost(best)) best = sh;
     };
     for (int split = Cfg<T>::NSLOT; split > 1; split /= 2) consider({pairs * split, split, 1, max_L, max_p, 1});
     return best;
 }
+
+namespace {
+std::atomic<int> g_jacobi_calls[64];       // per device
+}
+JacobiCall::JacobiCall() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+    slot = dev & 63;
+    g_jacobi_calls[slot].fetch_add(1, std::memory_order_relaxed);
+}
+JacobiCall::~JacobiCall() { g_jacobi_calls[slot].fetch_sub(1, std::memory_order_relaxed); }
+int JacobiCall::together() const { return std::max(1, g_jacobi_calls[slot].load(std::memory_order_relaxed)); }
 
 template <typename T>
 cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int sweeps, T tol, int* sweeps_run,
@@ -1377,8 +1396,8 @@ cudaError_t osj_sweeps(const OsjDesc<T>* d_desc, int nmat, OsjShape shape, int s
 
 template cudaError_t osj_sweeps<float>(const OsjDesc<float>*, int, OsjShape, int, float, int*, cudaStream_t, OsjMode, int, const int*);
 template cudaError_t osj_sweeps<double>(const OsjDesc<double>*, int, OsjShape, int, double, int*, cudaStream_t, OsjMode, int, const int*);
-template OsjShape osj_shape<float>(int, int, int, int, bool);
-template OsjShape osj_shape<double>(int, int, int, int, bool);
+template OsjShape osj_shape<float>(int, int, int, int, bool, int);
+template OsjShape osj_shape<double>(int, int, int, int, bool, int);
 template size_t osj_grid_head<float>(int);
 template size_t osj_grid_head<double>(int);
 template size_t osj_grid_bytes<float>(int);

@@ -1284,6 +1284,7 @@ int svt_run(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* 
             cudaStream_t s, const SvtScratch<T>& q) {
     const bool tall = cols <= rows;
     const int p = (int)std::min(rows, cols), L = (int)std::max(rows, cols), pp = round_up(p, osj_pivot_width());
+    const JacobiCall call;
     SvtParams<T> par{};
     SvtParams<T>* const d = q.par;
     par.mu = 1.0 / tau;
@@ -1304,7 +1305,7 @@ int svt_run(const T* A, int64_t rows, int64_t cols, int64_t lda, double tau, T* 
     svt_begin<T><<<(unsigned)std::min<int64_t>(tiles, 152 * 8), 256, 0, s>>>(A, lda, L, p, pp, tall ? 1 : 0, q.X, q.W, par, d,
         reinterpret_cast<unsigned*>(q.grid), q.grid ? (int)(osj_grid_head<T>(p) / sizeof(unsigned)) : 0);
     LRR_CUDA_TRY(cudaGetLastError());
-    LRR_CUDA_TRY(osj_sweeps<T>(&d->od, 1, osj_shape<T>(1, p, L, 0, q.grid != nullptr), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), &d->sweeps, s,
+    LRR_CUDA_TRY(osj_sweeps<T>(&d->od, 1, osj_shape<T>(1, p, L, 0, q.grid != nullptr, call.together()), 40, sizeof(T) == 8 ? T(1e-13) : T(2e-6), &d->sweeps, s,
                                OsjMode::sorted));
     k::svt_weights<T><<<dim3(1, (unsigned)ceil_div(pp, k::kWeightCols)), 256, 0, s>>>(&d->od, &d->h, &d->act, &d->on,
                                                                                      &d->mu, &d->rank, 1);

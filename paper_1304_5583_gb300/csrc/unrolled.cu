@@ -215,6 +215,7 @@ struct Engine {
     T *ocols, *ooff;
     int *oord, *oon;
     OsjShape oshape;
+    int together = 1;            // calls that share the device
     char* ogrid = nullptr;       // the Jacobi's clusterless workspace, after an integer a wait that gave up sets
     T **pW, **pH, **pT;
     int *pv, *ppv;
@@ -576,7 +577,7 @@ int engine_init(Engine<T>& g) {
     d.ldx = g.n; d.ldw = g.pp; d.L = (int)g.n; d.p = g.r; d.pp = g.pp; d.strict = 1;
     d.grid = g.ogrid ? g.ogrid + kAl : nullptr;
     d.fail = reinterpret_cast<int*>(g.ogrid);
-    g.oshape = osj_shape<T>(1, g.r, (int)g.n, 0, g.ogrid != nullptr);
+    g.oshape = osj_shape<T>(1, g.r, (int)g.n, 0, g.ogrid != nullptr, g.together);
     UTRY(cudaMemcpyAsync(g.od, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     T* ptrs[3] = {g.Wj, g.Wg, g.Wt};
     UTRY(cudaMemcpyAsync(g.pW, &ptrs[0], sizeof(T*), cudaMemcpyHostToDevice, s));
@@ -631,6 +632,7 @@ int unrolled_run(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unr
                  int64_t ldz, const void* Zbar, int64_t ldzb, void* Mbar, int64_t ldmb, double* lambar, void* ws,
                  size_t wsb, cudaStream_t s) {
     const bool grad = Zbar != nullptr;
+    const JacobiCall call;
     Engine<T> g = make_engine<T>(M, m, n, ldm, o, grad);
     if (!grad) g.cp = 0;
     g.s = s;
@@ -657,6 +659,7 @@ int unrolled_run(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unr
     }
     int rc = setup<T>(g, o->rank_tol > 0 ? o->rank_tol : 1e-6);
     if (rc != LRR_OK) return rc;
+    g.together = call.together();
     rc = engine_init<T>(g);
     if (rc != LRR_OK) return rc;
     rc = reset_state<T>(g);

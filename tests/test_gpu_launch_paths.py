@@ -151,3 +151,36 @@ def test_bf16_product_in_clusters_matches_float64(lib, M, N, K):
     ref = A.double().numpy() @ B.double().numpy().T
     # the bar of the other bf16 products: float32 accumulation order alone
     assert np.abs(C - ref).max() / np.abs(ref).max() < 2e-6
+
+
+@pytest.mark.parametrize("dtype,rows,cols", [("f64", 90, 90), ("f64", 100, 500), ("f32", 1000, 487)])
+def test_concurrent_svts_run_side_by_side(lib, dtype, rows, cols):
+    """Eight threads' SVTs share the chip: one alone may spread over most of it, but
+    eight that did so would run one after another, 8 times one thread's time."""
+    import time
+
+    import torch
+    from paper_1304_5583_gb300 import binding
+    rng = np.random.default_rng(4)
+    A = _dev(rng.standard_normal((rows, 40)) @ rng.standard_normal((40, cols)) / 300.0, dtype)
+
+    def work():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(6):
+                binding.svt(A, 0.05)
+
+    def run(n):
+        threads = [threading.Thread(target=work) for _ in range(n)]
+        t0 = time.perf_counter()
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        return time.perf_counter() - t0
+
+    torch.cuda.synchronize()
+    run(8)
+    alone, eight = min(run(1) for _ in range(3)), min(run(8) for _ in range(3))
+    # eight blocks in clusters of 12 to 16 CTAs are resident at once; a cluster
+    # takes up to twice a whole chip's time
+    assert eight < 4 * alone, (alone, eight)
