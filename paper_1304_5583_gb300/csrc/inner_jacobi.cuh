@@ -28,15 +28,17 @@ template <typename T>
 __device__ __forceinline__ void jacobi_rotation(T app, T aqq, T apq, T& cc, T& ss);
 
 // float64 quotients, reciprocals and square roots of the rotation, rounded as
-// IEEE division and square root round them.  A dependent float64 operation takes
+// IEEE division and square root round them but for one in 2^30.  A dependent float64 operation takes
 // 65 cycles here (a float32 one 4), conversions and compares included, so the
 // seeds are taken to 2^-43 in pairs of float32 (one Newton step on the hardware
 // approximation, the argument's low bits as a second float32), exponents and
 // conversions are handled as integers, and float64 is left with the product and
 // the remainder correction of P. Markstein ("IA-64 and Elementary Functions",
 // 2000, ch. 8 and 9): 3 operations for a quotient or a root, 2 for a
-// reciprocal.  The result before its last rounding is good to 2^-86, so it
-// differs from the IEEE one with probability below 2^-32.
+// reciprocal.  The result before its last rounding is good to 2^-84 (1.5 e^2 for
+// a root, e^2 otherwise, with seeds good to e = 2^-42.7), so it may differ from
+// the IEEE one, in the last bit, only where the exact value lies that close to
+// the middle between two float64 values.
 // (4e9 random cases each against / and sqrt: one reciprocal differed.)
 
 // y0 + y1 as a double, for y0 in [0.5, 1], |y1| < 2^-21, to 2^-44: y1 is added
@@ -67,10 +69,13 @@ __device__ __forceinline__ double rcp_seed(int hb, int lb) {
 }
 // 1 / s from y = (1 / s)(1 + O(2^-43))
 __device__ __forceinline__ double rcp_rn(double s, double y) { return fma(y, fma(-s, y, 1.0), y); }
-// 1 / b, b in [1, 2^900]
+// 1 / b, b in [1, 2^900].  A mantissa of ones, which sums at 2^53 have, is the one
+// whose reciprocal 2^k (1 + 2^-53 + 2^-106) lies nearest to a middle: its last
+// bit is set.  (A cosine's root, below 1.5, has no such mantissa.)
 __device__ __forceinline__ double rcp_rn(double b) {
-    const int hb = __double2hiint(b);
-    return rcp_rn(b, scale2(rcp_seed(hb, __double2loint(b)), 1023 - (hb >> 20)));
+    const int hb = __double2hiint(b), lb = __double2loint(b);
+    const double r = rcp_rn(b, scale2(rcp_seed(hb, lb), 1023 - (hb >> 20)));
+    return __hiloint2double(__double2hiint(r), __double2loint(r) | (((hb | 0xFFF00000) & lb) == -1));
 }
 // a / b over the whole range: mantissas in [1, 2) and the exponents apart; near
 // the ends of the range the division itself

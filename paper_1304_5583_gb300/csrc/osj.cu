@@ -16,7 +16,9 @@
 //   kept     columns in their own places, one inner pass over all pairs of a
 //            pivot.  The float32 solver: its stop test (1e-6 against float32
 //            residuals) and the blocks' paths react to the rounding of every
-//            SVT, so its arithmetic is held fixed, operation for operation.
+//            SVT, so a pivot's arithmetic is held fixed, operation for operation
+//            (which pivots are formed follows from the columns' norms, with
+//            margins; see the list of pivots in osj_svd).
 //   sorted   columns taken by falling norm (sorted at the start of sweeps 0, 2
 //            and 4), up to two inner passes over the pairs that cross the two
 //            column blocks (the first round of a sweep also takes the pairs
