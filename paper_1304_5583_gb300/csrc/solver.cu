@@ -1025,6 +1025,7 @@ int solve_impl(const lrr_problem* p, const lrr_options* o, void* ws, size_t ws_b
         k::svt_gate<<<ceil_div(t, 128), 128, 0, s>>>(B.act, B.mu, gate, t);
         prof.end(LRR_PH_GRAM, 1);
         tc_window = false;
+        bf16_phase = mixed;        // (one block at a time: every block starts in it)
         while (done_it < o->max_iter) {
             const int len = std::min(chunk, o->max_iter - done_it);
             const int rc = run_chunk(len);

@@ -95,6 +95,18 @@ def test_concurrent_svts_equal_one_alone(lib, dtype):
     assert k == rank and torch.equal(J, ref)
 
 
+def test_mixed_blocks_one_at_a_time_equal_the_batch(lib):
+    """Every block has its bf16 phase, also the ones after the first."""
+    import torch
+    from paper_1304_5583_gb300 import binding
+    w = synth.workload("small_dfc_60x240")
+    M = _dev(w.M, "mixed")
+    a, b = (binding.dfc_lrr_solve(M, w.perm, w.offsets, binding.options(w.lam, precision="mixed", batched=x),
+                                  raise_on_error=False) for x in (True, False))
+    assert np.array_equal(a.iters, b.iters)
+    assert torch.equal(a.Z, b.Z) and torch.equal(a.S, b.S)
+
+
 # ragged against the 16, 32 and 64-wide tiles and 16-term slabs; blocks at and
 # past the 64 columns that finish their SVT in one launch; one pivot of the
 # factor's eigensolver, two, and a padded last one
