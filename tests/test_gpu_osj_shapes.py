@@ -89,3 +89,23 @@ def test_svt_does_not_depend_on_the_scale_of_its_input(lib, dtype, scale, kind):
     # float64 norm squares them too)
     J, Jo = J.cpu().numpy().astype(np.float64) / scale, Jo / scale
     assert np.linalg.norm(J - Jo) <= (5e-6 if dtype == "f32" else 1e-12) * np.linalg.norm(Jo)
+
+
+@pytest.mark.parametrize("shape", [(64, 64), (100, 120), (150, 400)], ids=lambda s: f"{s[0]}x{s[1]}")
+@pytest.mark.parametrize("low", [1e-6, 1e-10, 1e-14])
+def test_float64_svt_of_graded_spectra(lib, shape, low):
+    """Rotations in float32 between columns many orders apart."""
+    import torch
+    from paper_1304_5583_gb300 import binding
+    rows, cols = shape
+    k = min(rows, cols)
+    rng = np.random.default_rng(rows + cols)
+    U = np.linalg.qr(rng.standard_normal((rows, k)))[0]
+    V = np.linalg.qr(rng.standard_normal((cols, k)))[0]
+    s = np.geomspace(1.0, low, k)
+    tau = np.sqrt(s[k // 2 - 1] * s[k // 2])           # keeps half of them
+    J, rank = binding.svt(torch.from_numpy(np.asfortranarray((U * s) @ V.T)).cuda(), tau)
+    assert rank == k // 2
+    # the bar of the stand-alone SVT
+    Jo = (U * np.maximum(s - tau, 0.0)) @ V.T
+    assert np.linalg.norm(J.cpu().numpy() - Jo) <= 1e-12 * np.linalg.norm(Jo)
