@@ -16,8 +16,11 @@
  * caller allocates and owns; (host) arrays are ordinary host memory.  Matrices
  * are column-major.  The library never frees caller memory.  Work memory is a
  * single caller-provided device buffer of at least lrr_workspace_bytes() bytes
- * (256-byte aligned); with workspace == NULL the library allocates it with
- * cudaMallocAsync on `stream` and frees it before returning.
+ * (256-byte aligned); with workspace == NULL the library allocates it on
+ * `stream` and frees it before returning.  What the library allocates itself
+ * comes from a stream-ordered memory pool of its own, one per device, which
+ * keeps up to 64 MiB of freed memory between calls until the library is
+ * unloaded (more than that returns to the system at the next synchronisation).
  *
  * Streams: all device work is queued on `stream`; the call returns after the
  * stream has drained the solve (it reads convergence flags and the per-block
@@ -202,7 +205,7 @@ LRR_API int dfc_lrr_solve(const lrr_problem* p, const lrr_options* o, void* work
  * concurrent streams (lrr_solve_batch).  r->Z (device, n x n, original order;
  * zero outside the diagonal blocks) and r->S as for dfc_lrr_solve; r->F/G are
  * not produced (LRR_ERR_UNSUPPORTED if given); r->ranks = [largest rank(C_i),
- * rank used, SVT rank of each block].  Scratch via cudaMallocAsync.
+ * rank used, SVT rank of each block].  Scratch from the library's pool.
  * Returns an lrr_status. */
 LRR_API int dfc_lrr_solve_local(const lrr_problem* p, const lrr_options* o, int64_t rank, lrr_result* r,
                                 int32_t streams, void* stream);
@@ -214,8 +217,8 @@ LRR_API int dfc_lrr_solve_local(const lrr_problem* p, const lrr_options* o, int6
  * column-major float (precision LRR_PREC_F32) or double (LRR_PREC_F64); J may
  * not alias A.  *rank (host, may be NULL) receives #{s > tau}.  Computed as in
  * the solver: one-sided block Jacobi on the columns of A (tall) or A^T (wide),
- * from a cold start.  Scratch memory is taken with cudaMallocAsync on `stream`
- * and released before returning; the call synchronises `stream`.
+ * from a cold start.  Scratch memory is taken from the library's pool on
+ * `stream` and released before returning; the call synchronises `stream`.
  * rows, cols <= 65536. */
 LRR_API int lrr_svt(const void* A, int64_t rows, int64_t cols, int64_t lda, double tau, void* J, int64_t ldj,
                     int32_t precision, int32_t* rank, void* stream);
@@ -252,7 +255,7 @@ LRR_API size_t lrr_svt_noalloc_capacity(void);
  * All device pointers; the call
  * synchronises `stream` and returns LRR_ERR_CUDA if a launch failed or a wait
  * inside the kernel timed out.
- * Scratch: one int taken with cudaMallocAsync. */
+ * Scratch: one int from the library's pool. */
 LRR_API int lrr_gemm_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc, int64_t M,
                           int64_t N, int64_t K, void* stream);
 
@@ -263,7 +266,7 @@ LRR_API int lrr_gemm_bf16(const void* A, int64_t lda, const void* B, int64_t ldb
  * part and a float32 remainder and three TF32 tensor-core products are summed
  * in float32 (error near that of a float32 product; the remainders' product,
  * below 2^-20 |a||b| per term, is dropped).  All device pointers; scratch (the
- * split operands, 8 (M + N) K bytes) is taken with cudaMallocAsync; the call
+ * split operands, 8 (M + N) K bytes) is taken from the library's pool; the call
  * synchronises `stream`. */
 LRR_API int lrr_gemm_f32(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M,
                          int64_t N, int64_t K, void* stream);
@@ -272,7 +275,7 @@ LRR_API int lrr_gemm_f32(const float* A, int64_t lda, const float* B, int64_t ld
  * it: kind 0 = the bf16 product (lrr_gemm_bf16), kind 1 = the split-TF32
  * product (lrr_gemm_f32) on operands already split, kind 2 = the split-bf16
  * product of the mixed form's bf16 phase (three bf16 MMAs, operands already
- * split).  Fills synthetic M x K and K x N operands in scratch taken with cudaMallocAsync, launches the
+ * split).  Fills synthetic M x K and K x N operands in scratch from the library's pool, launches the
  * kernel once untimed and `repeat` times back to back between two CUDA
  * events on `stream`, and stores the mean time per launch (ms). */
 LRR_API int lrr_gemm_timing(int32_t kind, int64_t M, int64_t N, int64_t K, int32_t repeat, double* ms_per_launch,
@@ -305,7 +308,7 @@ typedef struct {
 LRR_API size_t lrr_unrolled_workspace_bytes(int64_t m, int64_t n, const lrr_unrolled_options* o, int32_t with_grad);
 
 /* Z (device, n x n, ld ldz >= n) = Z_K(M, lambda).  M (device) m x n, ld ldm,
- * float or double as o->precision.  workspace NULL: cudaMallocAsync on
+ * float or double as o->precision.  workspace NULL: from the library's pool on
  * stream.  Synchronises stream.  Returns an lrr_status. */
 LRR_API int lrr_unrolled_forward(const void* M, int64_t m, int64_t n, int64_t ldm, const lrr_unrolled_options* o,
                                  void* Z, int64_t ldz, void* workspace, size_t workspace_bytes, void* stream);
@@ -326,8 +329,8 @@ LRR_API int lrr_unrolled_backward(const void* M, int64_t m, int64_t n, int64_t l
  * (k-means++ seeding from SplitMix64 of seed, `restarts` restarts, the lowest
  * cost wins).  F (device, n x k, ld ldf), G (device, k x n, ld ldg) float;
  * labels (host, n) receives cluster indices 0..clusters-1.  The n x n
- * affinity lives in the workspace (lrr_segment_workspace_bytes; NULL:
- * cudaMallocAsync).  clusters <= 64.  Synchronises stream. */
+ * affinity lives in the workspace (lrr_segment_workspace_bytes; NULL: from the
+ * library's pool).  clusters <= 64.  Synchronises stream. */
 LRR_API size_t lrr_segment_workspace_bytes(int64_t n, int64_t k, int32_t clusters, int32_t restarts);
 LRR_API int lrr_segment(const float* F, int64_t ldf, const float* G, int64_t ldg, int64_t n, int64_t k,
                         int32_t clusters, double rel_tol, uint64_t seed, int32_t restarts, int32_t power_iters,
